@@ -26,8 +26,16 @@ namespace amg {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
-// operands of the fused dot products of the SELL kernel
-enum DotOp { OP_X = 0, OP_Y = 1, OP_U1 = 2, OP_U2 = 3 };
+// the scalar step that follows a kernel's inner products (run_fin)
+enum FinKind { FIN_K1 = 0, FIN_K3 = 1, FIN_ALPHA = 2, FIN_BETA = 3 };
+
+struct FinArgs {
+  int kind;
+  double *slots;
+  const int *restart;  // FIN_BETA
+  double *partials;    // ndot x kRedBlocks
+  unsigned *ticket;    // 0 between launches
+};
 
 template <class VT>
 struct SellArgs {
@@ -43,10 +51,12 @@ struct SellArgs {
   const VT *rhs;  // right-hand side (residual / smoothing epilogues)
   const VT *wd;   // omega / A_ii
   const VT *xin;  // the iterate that the post-smoothing step updates
-  const VT *u1, *u2;  // extra dot operands
-  double *partials;   // ndot x kRedBlocks
-  int ndot;
-  int dop[3][2];
+  // fused inner products with left operand s = x (dot_y: the output): ND = 2:
+  // {s.out, s.u1}, ND = 3: {s.out, s.u1, s.u2}, ND = 1: {out.q64}; then fin
+  const VT *u1, *u2;
+  const double *q64;
+  int dot_y;
+  FinArgs fin;
   const int *pred;
   // polynomial smoother operands
   const VT *dinv;     // 1 / A_ii
@@ -75,42 +85,129 @@ template <class MV> __device__ __forceinline__ MV ld_stream(const MV *p) { retur
 template <class MV> constexpr bool kPairs = std::is_same<MV, float>::value;
 template <class MV> constexpr bool kHalfPairs = std::is_same<MV, __nv_bfloat16>::value;
 
-// per-block partial sums of up to three dot products -> partials[k*kRedBlocks + block]
-__device__ __forceinline__ void block_store_dots3(double a0, double a1, double a2, int ndot, double *partials) {
-  __shared__ double sh[3][kWarps];
-  const double in[3] = {a0, a1, a2};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    if (k < ndot) {
-      const double v = warp_sum(in[k]);
-      if ((threadIdx.x & 31) == 0) sh[k][threadIdx.x >> 5] = v;
-    }
+// ---- inner products and the scalars they lead to, in one launch
+// A kernel that ends with inner products also forms the scalars of Alg. 5 or of
+// the outer iteration: its blocks publish their partial sums, take a ticket, and
+// the block that finishes last sums all partials in block order (deterministic)
+// and runs the scalar step.  A separate one-block kernel for that costs 3-5 us of
+// dependent latency in the chain even with programmatic dependent launch; the
+// last block adds ~1.5 us (128^3, 27 outer iterations: 36 such kernels an
+// iteration removed).
+// GB300 issues an FP64 warp instruction every 16 cycles an SM, so the reduction
+// counts them: the block's values go through shared memory and one warp per
+// product adds 8 values a lane and 5 shuffles (12 warp instructions a product,
+// against 45 with a shuffle tree in each of the 8 warps).
+// the scalar step, by one thread, from the totals of the kernel's inner products
+__device__ __forceinline__ void run_fin(const FinArgs &f, const double *tot) {
+  double *slots = f.slots;
+  if (f.kind == FIN_K1) {
+    // Alg. 5 after v = A c: rho_1 and alpha_1 (CG: c^T v, c^T r; GMRES: ||v||^2, v^T r)
+    slots[S_RHO1] = tot[0];
+    slots[S_A1] = tot[1];
+    slots[S_S1] = tot[1] / tot[0];
+  } else if (f.kind == FIN_K3) {
+    // Alg. 5 after w = A d: gamma, beta, alpha_2 (CG: d^T v, d^T w, d^T r~; GMRES
+    // with w in place of d on the left), rho_2 = beta - gamma^2 / rho_1 and the
+    // combination weights; the products come as {beta, gamma, alpha_2}
+    const double bet = tot[0], gam = tot[1], a2 = tot[2];
+    const double g1 = gam / slots[S_RHO1];
+    const double cd = a2 / (bet - gam * g1);
+    slots[S_GAM] = gam;
+    slots[S_BET] = bet;
+    slots[S_A2] = a2;
+    slots[S_CC] = slots[S_S1] - g1 * cd;
+    slots[S_CD] = cd;
+  } else if (f.kind == FIN_ALPHA) {  // outer flexible CG: alpha = p^T r / p^T q
+    slots[S_PQ] = tot[0];
+    slots[S_PR] = tot[1];
+    slots[S_ALPHA] = tot[1] / tot[0];
+  } else {  // beta = -(z^T q_old) / (p_old^T q_old), 0 right after a restart
+    slots[S_ZQ] = tot[0];
+    slots[S_BETA] = *f.restart != 0 ? 0.0 : -tot[0] / slots[S_PQ];
   }
-  __syncthreads();
-  if (threadIdx.x < 32) {
+}
+
+// totals of ND inner products over the grid; true in thread 0 of the last block
+// only, with the totals in tot.  `step`: only the threads of every step-th warp
+// hold a value.  Every thread of the block calls it, all blocks of the grid.
+template <int ND>
+__device__ __forceinline__ bool grid_totals(const double (&acc)[ND], int step, double *partials, unsigned *ticket,
+                                            double (&tot)[ND]) {
+  __shared__ double sh[ND][kThreads];
+  __shared__ double tot_sh[ND];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      if (k < ndot) {
-        double v = threadIdx.x < kWarps ? sh[k][threadIdx.x] : 0.0;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) partials[k * kRedBlocks + blockIdx.x] = v;
+  for (int k = 0; k < ND; ++k) sh[k][threadIdx.x] = acc[k];
+  __syncthreads();
+  if (wid < ND) {
+    double v = sh[wid][lane];
+    for (int q = step; q < kWarps; q += step) v += sh[wid][q * 32 + lane];
+    v = warp_sum(v);
+    if (lane == 0) {
+      if (gridDim.x == 1) {
+        tot_sh[wid] = v;
+      } else {
+        partials[wid * kRedBlocks + blockIdx.x] = v;
+        __threadfence();
       }
     }
   }
+  __syncthreads();
+  if (gridDim.x > 1) {
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+      double v[kRedBlocks / kThreads + 1];
+#pragma unroll
+      for (int u = 0; u <= kRedBlocks / kThreads; ++u) {
+        const int j = threadIdx.x + u * kThreads;
+        v[u] = j < (int)gridDim.x ? __ldcg(partials + k * kRedBlocks + j) : 0.0;
+      }
+      double t = v[0];
+#pragma unroll
+      for (int u = 1; u <= kRedBlocks / kThreads; ++u)
+        if (u * kThreads < (int)gridDim.x) t += v[u];
+      sh[k][threadIdx.x] = t;
+    }
+    __syncthreads();
+    if (wid < ND) {
+      double v = sh[wid][lane];
+      for (int q = 1; q < kWarps && q * 32 < (int)gridDim.x; ++q) v += sh[wid][q * 32 + lane];
+      v = warp_sum(v);
+      if (lane == 0) tot_sh[wid] = v;
+    }
+    __syncthreads();
+  }
+  if (threadIdx.x != 0) return false;
+  if (gridDim.x > 1) *ticket = 0;
+#pragma unroll
+  for (int k = 0; k < ND; ++k) tot[k] = tot_sh[k];
+  return true;
 }
 
-template <class VT>
-__device__ __forceinline__ void block_store_dots(const double (&acc)[3], int ndot, double *partials) {
-  block_store_dots3(acc[0], acc[1], acc[2], ndot, partials);
+template <int ND>
+__device__ __forceinline__ void grid_dots(const double (&acc)[ND], int step, const FinArgs &f) {
+  double tot[ND];
+  if (grid_totals<ND>(acc, step, f.partials, f.ticket, tot)) run_fin(f, tot);
 }
 
-// y = A x over SELL-32 (one warp per slice, one lane per row) with an epilogue:
-//   E_Y     out = A x
-//   E_RESID out = rhs - A x
-//   E_POST  out = xin + wd * (rhs - A x)   (damped Jacobi after prolongation)
-// and up to three fused dot products of {x_i, y_i, u1_i, u2_i} pairs.
-__device__ __forceinline__ double dot_operand(int op, double x, double y, double u1, double u2) {
-  return op == OP_X ? x : (op == OP_Y ? y : (op == OP_U1 ? u1 : u2));
+// per-block partial sums of one inner product -> partials[block] (no finish)
+__device__ __forceinline__ void block_store_dot(double a, double *partials) {
+  __shared__ double sh[kThreads];
+  const int lane = threadIdx.x & 31;
+  sh[threadIdx.x] = a;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double v = sh[lane];
+#pragma unroll
+    for (int q = 1; q < kWarps; ++q) v += sh[q * 32 + lane];
+    v = warp_sum(v);
+    if (lane == 0) partials[blockIdx.x] = v;
+  }
 }
 
 // batch: live[sl] = 1 when some system with rows in slice sl still iterates.
@@ -135,7 +232,7 @@ __global__ void k_slice_live(int32_t n, int32_t nslices, const int32_t *__restri
 template <class VT>
 constexpr int sell_min_blocks() { return sizeof(VT) == 4 ? 6 : 4; }
 
-// DOTS: the launch fuses inner products (compiled only where used, so that the
+// ND: inner products that the launch fuses (compiled only where used, so that the
 // plain SpMV does not hold their accumulators in registers)
 // GATE: a batch's launch, skipping slices whose systems have all stopped
 // (compiled only into the batch instantiations)
@@ -145,16 +242,17 @@ constexpr int sell_min_blocks() { return sizeof(VT) == 4 ? 6 : 4; }
 // entries) goes out in one or two steps.
 // With fused inner products the FP32-vector kernel needs more than the 40
 // registers of six resident blocks (it spilled there): four blocks, 64 registers.
-template <class MV, class VT, bool DOTS>
-constexpr int sell_launch_blocks() { return DOTS ? 4 : sell_min_blocks<VT>(); }
+constexpr int kDotBlocks = 4;
+template <class VT, int ND>
+constexpr int sell_launch_blocks() { return ND ? kDotBlocks : sell_min_blocks<VT>(); }
 
-template <class MV, class VT, int EPI, bool DOTS, bool GATE, int UW = 0>
-__global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<MV, VT, DOTS>()) k_sell(SellArgs<VT> a) {
+template <class MV, class VT, int EPI, int ND, bool GATE, int UW = 0>
+__global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<VT, ND>()) k_sell(SellArgs<VT> a) {
   pdl_wait_and_trigger();
   if (a.pred && *a.pred == 0) return;
   const int lane = threadIdx.x & 31;
   const MV *__restrict__ sval = static_cast<const MV *>(a.sval);
-  double acc0 = 0.0, acc1 = 0.0, acc2 = 0.0;
+  double acc[ND ? ND : 1] = {0.0};
   // U entries of a row per step: 6 with FP32 vectors (a 7-point row without its
   // split-off diagonal in one step, at 40 registers), 8 with FP64
   constexpr int U = UW ? UW : (sizeof(VT) == 4 ? 6 : 8);
@@ -290,16 +388,17 @@ __global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<MV, VT, 
       else
         o = a.xin[row] + (a.dinv[row] * y + a.dinv[row] * (a.coef[3 * row] * a.res[row]));
       a.out[row] = o;
-      if (DOTS && a.ndot) {
-        const double ox = (double)a.x[row], oy = (double)o, o1 = a.u1 ? (double)a.u1[row] : 0.0,
-                     o2 = a.u2 ? (double)a.u2[row] : 0.0;
-        acc0 += dot_operand(a.dop[0][0], ox, oy, o1, o2) * dot_operand(a.dop[0][1], ox, oy, o1, o2);
-        if (a.ndot > 1) acc1 += dot_operand(a.dop[1][0], ox, oy, o1, o2) * dot_operand(a.dop[1][1], ox, oy, o1, o2);
-        if (a.ndot > 2) acc2 += dot_operand(a.dop[2][0], ox, oy, o1, o2) * dot_operand(a.dop[2][1], ox, oy, o1, o2);
+      if constexpr (ND == 1) {
+        acc[0] += (double)o * a.q64[row];
+      } else if constexpr (ND >= 2) {
+        const double oy = (double)o, sv = a.dot_y ? oy : (double)a.x[row];
+        acc[0] += sv * oy;
+        acc[1] += sv * (double)a.u1[row];
+        if constexpr (ND == 3) acc[2] += sv * (double)a.u2[row];
       }
     }
   }
-  if (DOTS && a.ndot) block_store_dots3(acc0, acc1, acc2, a.ndot, a.partials);
+  if constexpr (ND > 0) grid_dots<ND>(acc, 1, a.fin);
 }
 
 // out = wd * rhs: damped Jacobi from a zero initial guess
@@ -408,72 +507,37 @@ __device__ __forceinline__ double sum_partials(const double *__restrict__ part, 
   return result;
 }
 
-// Alg. 5 after v = A c: rho_1 and alpha_1 (CG: c^T v, c^T r; GMRES: ||v||^2, v^T r)
-__global__ void k_fin_k1(const double *__restrict__ part, int nb, double *__restrict__ slots, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  const double rho1 = sum_partials(part, 0, nb);
-  const double a1 = sum_partials(part, 1, nb);
-  if (threadIdx.x == 0) {
-    slots[S_RHO1] = rho1;
-    slots[S_A1] = a1;
-    slots[S_S1] = a1 / rho1;
-  }
-}
-
-// r~ = r - (alpha_1/rho_1) v, with ||r~||^2, ||r||^2 partials and the next
-// smoothing start x0 = wd * r~
+// r~ = r - (alpha_1/rho_1) v, the next smoothing start x0 = wd * r~, and the
+// test of Alg. 5 in the last block: the second inner step runs iff the enclosing
+// step runs and ||r~|| > t ||r||.  A skipped enclosing step clears the flag.
 template <class VT>
-__global__ void k_axpy_rt(int32_t n, const VT *__restrict__ r, const VT *__restrict__ v, VT *__restrict__ rt,
-                          const VT *__restrict__ wd, VT *__restrict__ x0, const double *__restrict__ slots,
-                          double *__restrict__ part, const int *pred) {
+__global__ void __launch_bounds__(kThreads) k_axpy_rt(int32_t n, const VT *__restrict__ r, const VT *__restrict__ v,
+                                                      VT *__restrict__ rt, const VT *__restrict__ wd,
+                                                      VT *__restrict__ x0, double t, double *__restrict__ slots,
+                                                      int *__restrict__ flag, double *part, unsigned *ticket,
+                                                      const int *pred) {
   pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
+  if (pred && *pred == 0) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
+    return;
+  }
   const VT s1 = (VT)slots[S_S1];
-  double acc[3] = {0.0, 0.0, 0.0};
+  double acc[2] = {0.0, 0.0};
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const VT ri = r[i];
-    const VT t = ri - s1 * v[i];
-    rt[i] = t;
-    if (wd) x0[i] = wd[i] * t;
-    acc[0] += (double)t * (double)t;
+    const VT ti = ri - s1 * v[i];
+    rt[i] = ti;
+    if (wd) x0[i] = wd[i] * ti;
+    acc[0] += (double)ti * (double)ti;
     acc[1] += (double)ri * (double)ri;
   }
-  block_store_dots<VT>(acc, 2, part);
-}
-
-// the test of Alg. 5: the second inner step runs iff the enclosing step runs
-// and ||r~|| > t ||r||.  Never predicated, so a skipped parent clears it.
-__global__ void k_decide(const double *__restrict__ part, int nb, double *__restrict__ slots, double t,
-                         const int *parent, int *__restrict__ flag) {
-  pdl_wait_and_trigger();
-  const double nrt2 = sum_partials(part, 0, nb);
-  const double nr2 = sum_partials(part, 1, nb);
-  if (threadIdx.x == 0) {
-    const int active = parent ? *parent : 1;
-    slots[S_NRT2] = nrt2;
-    slots[S_NR2] = nr2;
-    const bool accept_first = sqrt(nrt2) <= t * sqrt(nr2);
-    *flag = (active && !accept_first) ? 1 : 0;
-    if (active && !accept_first) slots[S_TAKEN] += 1.0;  // cycle trace (one thread)
-  }
-}
-
-// Alg. 5 after w = A d: gamma, beta, alpha_2, rho_2 and the combination weights
-__global__ void k_fin_k3(const double *__restrict__ part, int nb, double *__restrict__ slots, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  const double gam = sum_partials(part, 0, nb);
-  const double bet = sum_partials(part, 1, nb);
-  const double a2 = sum_partials(part, 2, nb);
-  if (threadIdx.x == 0) {
-    const double rho1 = slots[S_RHO1];
-    const double rho2 = bet - gam * gam / rho1;
-    slots[S_GAM] = gam;
-    slots[S_BET] = bet;
-    slots[S_A2] = a2;
-    slots[S_CC] = slots[S_S1] - gam * a2 / (rho1 * rho2);
-    slots[S_CD] = a2 / rho2;
+  double tot[2];
+  if (grid_totals<2>(acc, 1, part, ticket, tot)) {
+    slots[S_NRT2] = tot[0];
+    slots[S_NR2] = tot[1];
+    const bool second = !(sqrt(tot[0]) <= t * sqrt(tot[1]));
+    *flag = second ? 1 : 0;
+    if (second) slots[S_TAKEN] += 1.0;  // cycle trace (one thread)
   }
 }
 
@@ -503,101 +567,90 @@ __global__ void k_to_vt(int32_t n, const double *__restrict__ in, VT *__restrict
   }
 }
 
-// z = (double) zin, with the partials of z^T q
+// z = (double) zin
 template <class VT>
-__global__ void k_from_vt_dot(int32_t n, const VT *__restrict__ zin, double *__restrict__ z,
-                              const double *__restrict__ q, double *__restrict__ part, const int *pred) {
+__global__ void k_from_vt(int32_t n, const VT *__restrict__ zin, double *__restrict__ z, const int *pred) {
   pdl_wait_and_trigger();
   if (pred && *pred == 0) return;
-  double acc[3] = {0.0, 0.0, 0.0};
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const double v = (double)zin[i];
-    z[i] = v;
-    acc[0] += v * q[i];
-  }
-  block_store_dots<double>(acc, 1, part);
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) z[i] = (double)zin[i];
 }
 
-// p = z + beta p,  beta = -(z^T q_old)/(p_old^T q_old) (0 right after a restart)
-__global__ void k_fcg_p(int32_t n, const double *__restrict__ z, double *__restrict__ p,
-                        const double *__restrict__ part_zq, int nb, double *__restrict__ slots,
+// z^T q and beta of the outer flexible CG where the cycle has no product to fuse
+// them into (a hierarchy of one level)
+template <class VT>
+__global__ void __launch_bounds__(kThreads) k_dot_zq(int32_t n, const VT *__restrict__ z, const double *__restrict__ q,
+                                                     FinArgs fin, const int *pred) {
+  pdl_wait_and_trigger();
+  if (pred && *pred == 0) return;
+  double acc[1] = {0.0};
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    acc[0] += (double)z[i] * q[i];
+  grid_dots<1>(acc, 1, fin);
+}
+
+// p = z + beta p (beta = 0 right after a restart); z in the cycle's vector type
+template <class VT>
+__global__ void k_fcg_p(int32_t n, const VT *__restrict__ z, double *__restrict__ p, const double *__restrict__ slots,
                         const int *__restrict__ restart, const int *pred) {
   pdl_wait_and_trigger();
   if (pred && *pred == 0) return;
-  const double zq = sum_partials(part_zq, 0, nb);
   const bool rs = *restart != 0;
-  const double beta = rs ? 0.0 : -zq / slots[S_PQ];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    slots[S_ZQ] = zq;
-    slots[S_BETA] = beta;
-  }
+  const double beta = slots[S_BETA];
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = rs ? z[i] : z[i] + beta * p[i];
+    p[i] = rs ? (double)z[i] : (double)z[i] + beta * p[i];
 }
 
-// alpha = p^T r / p^T q;  x += alpha p;  r -= alpha q;  partials of ||r||^2.
-// In reduced precision also the preconditioner input (VT) and its x0.
+struct FcgState {
+  double *hist;
+  int *it, *active, *restart, *status;
+  volatile int *host;  // mapped pinned words: [0] iterations, [4] status
+};
+
+// x += alpha p;  r -= alpha q;  the preconditioner input (in reduced precision
+// also rounded to VT) and its smoothing start x0 = wd r.  The last block ends the
+// outer iteration: relative residual into the history, iteration count,
+// convergence / breakdown status (deactivates the following launches).
 template <class VT>
-__global__ void k_fcg_update(int32_t n, double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
-                             const double *__restrict__ q, const double *__restrict__ part_pq, int nb,
-                             double *__restrict__ slots, double *__restrict__ part_rr, VT *__restrict__ rvt,
-                             const VT *__restrict__ wd, VT *__restrict__ x0, const int *pred) {
+__global__ void __launch_bounds__(kThreads) k_fcg_update(int32_t n, double *__restrict__ x, double *__restrict__ r,
+                                                         const double *__restrict__ p, const double *__restrict__ q,
+                                                         double *__restrict__ slots, double *part, unsigned *ticket,
+                                                         VT *__restrict__ rvt, const VT *__restrict__ wd,
+                                                         VT *__restrict__ x0, FcgState st, const int *pred) {
   pdl_wait_and_trigger();
   if (pred && *pred == 0) return;
-  const double pq = sum_partials(part_pq, 0, nb);
-  const double pr = sum_partials(part_pq, 1, nb);
-  const double alpha = pr / pq;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    slots[S_PQ] = pq;
-    slots[S_PR] = pr;
-    slots[S_ALPHA] = alpha;
-  }
-  double acc[3] = {0.0, 0.0, 0.0};
+  const double alpha = slots[S_ALPHA];
+  double acc[1] = {0.0};
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     x[i] += alpha * p[i];
     const double ri = r[i] - alpha * q[i];
     r[i] = ri;
     acc[0] += ri * ri;
-    if (rvt) {
-      const VT v = (VT)ri;
-      rvt[i] = v;
-      x0[i] = wd[i] * v;
-    }
+    const VT v = (VT)ri;
+    if (rvt) rvt[i] = v;
+    x0[i] = wd[i] * v;
   }
-  block_store_dots<double>(acc, 1, part_rr);
-}
-
-// end of an outer iteration: relative residual into the history, iteration
-// count, convergence / breakdown status; deactivates the following launches
-__global__ void k_fcg_fin(const double *__restrict__ part_rr, int nb, double *__restrict__ slots,
-                          double *__restrict__ hist, int *__restrict__ it, int *__restrict__ active,
-                          int *__restrict__ restart, int *__restrict__ status) {
-  pdl_wait_and_trigger();
-  if (*active == 0) return;
-  const double tol = slots[S_TOL];
-  const int max_iter = (int)slots[S_MAXIT];
-  const double rr = sum_partials(part_rr, 0, nb);
-  if (threadIdx.x == 0) {
-    const double rel = sqrt(rr) / sqrt(slots[S_NB2]);
-    const int k = *it + 1;
-    *it = k;
-    hist[k] = rel;
-    slots[S_RR] = rr;
+  double tot[1];
+  if (grid_totals<1>(acc, 1, part, ticket, tot)) {
+    const double rel = sqrt(tot[0]) / sqrt(slots[S_NB2]);
+    const int k = *st.it + 1;
+    *st.it = k;
+    st.hist[k] = rel;
+    slots[S_RR] = tot[0];
     slots[S_REL] = rel;
-    *restart = 0;
-    if (!(slots[S_PQ] > 0.0)) {
-      *status = AMG_ERR_BREAKDOWN;
-      *active = 0;
-    } else if (!isfinite(rel)) {
-      *status = AMG_ERR_NAN;
-      *active = 0;
-    } else if (rel <= tol) {
-      *status = 1;  // recursive residual converged: the host checks the true residual
-      *active = 0;
-    } else if (k >= max_iter) {
-      *status = AMG_ERR_NOT_CONVERGED;
-      *active = 0;
+    *st.restart = 0;
+    int status = 0;
+    if (!(slots[S_PQ] > 0.0)) status = AMG_ERR_BREAKDOWN;
+    else if (!isfinite(rel)) status = AMG_ERR_NAN;
+    else if (rel <= slots[S_TOL]) status = 1;  // updated residual converged: the host checks the true residual
+    else if (k >= (int)slots[S_MAXIT]) status = AMG_ERR_NOT_CONVERGED;
+    if (status != 0) {
+      *st.status = status;
+      *st.active = 0;
     }
+    st.host[0] = k;
+    __threadfence_system();
+    st.host[4] = status;
+    __threadfence_system();
   }
 }
 
@@ -606,9 +659,9 @@ __global__ void k_dot64(int32_t n, const double *__restrict__ a, const double *_
                         double *__restrict__ part, const int *pred) {
   pdl_wait_and_trigger();
   if (pred && *pred == 0) return;
-  double acc[3] = {0.0, 0.0, 0.0};
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) acc[0] += a[i] * b[i];
-  block_store_dots<double>(acc, 1, part);
+  double acc = 0.0;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) acc += a[i] * b[i];
+  block_store_dot(acc, part);
 }
 
 __global__ void k_store_sum(const double *__restrict__ part, int nb, double *__restrict__ dst) {
@@ -624,7 +677,7 @@ __global__ void k_residual64(int32_t n, int32_t nslices, const int64_t *__restri
                              double *__restrict__ part) {
   pdl_wait_and_trigger();
   const int lane = threadIdx.x & 31;
-  double acc[3] = {0.0, 0.0, 0.0};
+  double acc = 0.0;
   for (int32_t sl = blockIdx.x * kWarps + (threadIdx.x >> 5); sl < nslices; sl += gridDim.x * kWarps) {
     const int64_t base = sptr[sl];
     const int32_t width = (int32_t)((sptr[sl + 1] - base) >> 5);
@@ -637,10 +690,10 @@ __global__ void k_residual64(int32_t n, int32_t nslices, const int64_t *__restri
     if (row < n) {
       const double ri = b[row] - y;
       r[row] = ri;
-      acc[0] += ri * ri;
+      acc += ri * ri;
     }
   }
-  block_store_dots<double>(acc, 1, part);
+  block_store_dot(acc, part);
 }
 
 // ---------------------------------------------------------------- outer FGMRES (FP64)
@@ -1069,7 +1122,10 @@ template <class VT>
 inline int default_sell_grid(const Level &L) {
   return grid_for((int64_t)L.nslices, kWarps, sell_min_blocks<VT>() * 152);
 }
-inline int sell_grid(const Level &L) { return L.sell_blocks; }
+// launches with fused inner products: at most one wave of their kernel, which
+// runs kDotBlocks blocks per SM (a second, short wave and its reductions took the
+// 190k-row level of 128^3 from 10 to 17 us)
+inline int dot_grid(const Level &L) { return std::min(L.sell_blocks, kDotBlocks * 152); }
 // launches without inner products have no partial-sum buffer to fill, so the
 // autotuner may give them up to one warp per slice; by default they take the
 // same wave of resident blocks (one warp per slice measured slower on the 128^3
@@ -1116,43 +1172,33 @@ struct Engine {
     a.x = x;
     a.out = out;
     a.pred = pred;
-    a.partials = L.partials;
     return a;
   }
 
-  template <int EPI>
+  // where level k's inner products end: their scalar step and its scratch
+  FinArgs fin_args(int k, FinKind kind, double *partials) {
+    return {kind, h.lev[k].slots, h.it_dev + 2, partials, ticket(h.lev[k])};
+  }
+  unsigned *ticket(const Level &L) const { return reinterpret_cast<unsigned *>(L.flag + 1); }
+
+  // ND fused inner products: after the plain product (Alg. 5) and on the last
+  // post-smoothing step of level 0 (z^T q of the outer flexible CG)
+  template <int EPI, int ND = 0>
   void sell(const SellArgs<VT> &a, int k) {
-    // fused inner products: after the plain product (Alg. 5) and on the last
-    // post-smoothing step of level 0 (z^T q of the outer flexible CG)
     if (h.batched) {  // no fused inner products in a batch: they are per system (segdot)
-      if (a.ndot) throw Error{AMG_ERR_UNSUPPORTED, "batched SpMV was given fused inner products"};
-      klaunch(k_sell<MV, VT, EPI, false, true>, plain_grid(h.lev[k]), kThreads, s, a);
+      if (ND) throw Error{AMG_ERR_UNSUPPORTED, "batched SpMV was given fused inner products"};
+      klaunch(k_sell<MV, VT, EPI, 0, true>, plain_grid(h.lev[k]), kThreads, s, a);
       check();
       return;
     }
-    const bool small = sizeof(VT) == 4 && h.lev[k].nslices <= kSmallSlices;
-    if constexpr (EPI == E_Y || EPI == E_POST || EPI == E_HORNER_LAST) {
-      if (a.ndot) {
-        if constexpr (EPI == E_Y && sizeof(VT) == 4)
-          if (small) {
-            klaunch(k_sell<MV, VT, EPI, true, false, kSmallU>, sell_grid(h.lev[k]), kThreads, s, a);
-            check();
-            return;
-          }
-        klaunch(k_sell<MV, VT, EPI, true, false>, sell_grid(h.lev[k]), kThreads, s, a);
-        check();
-        return;
-      }
-    } else {
-      if (a.ndot) throw Error{AMG_ERR_UNSUPPORTED, "SpMV epilogue without fused inner products was given some"};
-    }
+    const int grid = ND ? dot_grid(h.lev[k]) : plain_grid(h.lev[k]);
     if constexpr ((EPI == E_Y || EPI == E_RESID || EPI == E_POST) && sizeof(VT) == 4)
-      if (small) {
-        klaunch(k_sell<MV, VT, EPI, false, false, kSmallU>, plain_grid(h.lev[k]), kThreads, s, a);
+      if (h.lev[k].nslices <= kSmallSlices) {
+        klaunch(k_sell<MV, VT, EPI, ND, false, kSmallU>, grid, kThreads, s, a);
         check();
         return;
       }
-    klaunch(k_sell<MV, VT, EPI, false, false>, plain_grid(h.lev[k]), kThreads, s, a);
+    klaunch(k_sell<MV, VT, EPI, ND, false>, grid, kThreads, s, a);
     check();
   }
 
@@ -1252,17 +1298,18 @@ struct Engine {
       a.coef = V(L.poly);
       a.res = V(L.r);
     }
-    if (k == 0 && std::is_same<VT, double>::value && zq_fuse) {
-      a.ndot = 1;  // z^T q for the outer flexible CG
-      a.dop[0][0] = OP_Y;
-      a.dop[0][1] = OP_U1;
-      a.u1 = (const VT *)h.q;
-      a.partials = h.lev[0].partials + 4 * kRedBlocks;
-    }
-    if (poly)
+    if (k == 0 && zq_fuse) {  // z^T q and beta of the outer flexible CG
+      a.q64 = h.q;
+      a.fin = fin_args(0, FIN_BETA, L.partials);
+      if (poly)
+        sell<E_HORNER_LAST, 1>(a, k);
+      else
+        sell<E_POST, 1>(a, k);
+    } else if (poly) {
       sell<E_HORNER_LAST>(a, k);
-    else
+    } else {
       sell<E_POST>(a, k);
+    }
   }
   bool zq_fuse = false;
 
@@ -1317,72 +1364,68 @@ struct Engine {
       return;
     }
     Level &L = h.lev[m];
-    const int nb = sell_grid(L);
     // c = cycle(m, r)
     cycle(m, V(L.bc), V(L.c), true, pred);
-    {  // v = A c; dots
+    {  // v = A c; rho_1, alpha_1
       SellArgs<VT> a = sell_args(m, V(L.c), V(L.v), pred);
-      a.ndot = 2;
       a.u1 = V(L.bc);
-      if (gmres_variant) {  // rho1 = v^T v, alpha1 = v^T r
-        a.dop[0][0] = OP_Y; a.dop[0][1] = OP_Y; a.dop[1][0] = OP_Y; a.dop[1][1] = OP_U1;
-      } else {               // rho1 = c^T v, alpha1 = c^T r
-        a.dop[0][0] = OP_X; a.dop[0][1] = OP_Y; a.dop[1][0] = OP_X; a.dop[1][1] = OP_U1;
-      }
-      sell<E_Y>(a, m);
+      a.dot_y = gmres_variant;  // GMRES: v^T v, v^T r; CG: c^T v, c^T r
+      a.fin = fin_args(m, FIN_K1, L.partials);
+      sell<E_Y, 2>(a, m);
     }
-    // One-block kernels take the scalars: with programmatic dependent launch
-    // their launch costs less than every block of the vector kernel summing the
-    // partials itself.
-    klaunch(k_fin_k1, 1, kThreads, s, L.partials, nb, L.slots, pred);
-    check();
     const int ng = ew_grid(L.n);
-    klaunch(k_axpy_rt<VT>, ng, kThreads, s, L.n, V(L.bc), V(L.v), V(L.rt), V(L.wd), V(L.tmp), L.slots,
-            L.partials + 3 * kRedBlocks, pred);
-    check();
-    klaunch(k_decide, 1, kThreads, s, L.partials + 3 * kRedBlocks, ng, L.slots, h.p.kcycle_t, pred, L.flag);
+    klaunch(k_axpy_rt<VT>, ng, kThreads, s, L.n, (const VT *)V(L.bc), (const VT *)V(L.v), V(L.rt), (const VT *)V(L.wd),
+            V(L.tmp), h.p.kcycle_t, L.slots, L.flag, L.partials, ticket(L), pred);
     check();
     // second inner step, predicated on the decision
     cycle(m, V(L.rt), V(L.d), true, L.flag);
     {
       SellArgs<VT> a = sell_args(m, V(L.d), V(L.w), L.flag);
-      a.ndot = 3;
       a.u1 = V(L.v);
       a.u2 = V(L.rt);
-      if (gmres_variant) {  // gamma = w^T v, beta = w^T w, alpha2 = w^T r~
-        a.dop[0][0] = OP_Y; a.dop[0][1] = OP_U1;
-        a.dop[1][0] = OP_Y; a.dop[1][1] = OP_Y;
-        a.dop[2][0] = OP_Y; a.dop[2][1] = OP_U2;
-      } else {               // gamma = d^T v, beta = d^T w, alpha2 = d^T r~
-        a.dop[0][0] = OP_X; a.dop[0][1] = OP_U1;
-        a.dop[1][0] = OP_X; a.dop[1][1] = OP_Y;
-        a.dop[2][0] = OP_X; a.dop[2][1] = OP_U2;
-      }
-      sell<E_Y>(a, m);
+      a.dot_y = gmres_variant;  // GMRES: w^T w, w^T v, w^T r~; CG: d^T w, d^T v, d^T r~
+      a.fin = fin_args(m, FIN_K3, L.partials);
+      sell<E_Y, 3>(a, m);
     }
-    klaunch(k_fin_k3, 1, kThreads, s, L.partials, nb, L.slots, L.flag);
-    check();
     klaunch(k_combine<VT>, ng, kThreads, s, L.n, V(L.c), V(L.d), V(L.xc), L.slots, L.flag, pred);
     check();
   }
 
+  // flexible CG: out = M r with the smoothing start x0 of level 0 already formed
+  // (by k_to_vt or k_fcg_update), then z^T q and beta.  The result stays in VT.
+  const VT *precond_fcg(const int *pred) {
+    Level &L0 = h.lev[0];
+    constexpr bool f64 = std::is_same<VT, double>::value;
+    const VT *in = f64 ? (const VT *)h.r : V(h.pre_in);
+    VT *out = f64 ? (VT *)h.z : V(h.pre_out);
+    zq_fuse = h.L > 1;
+    cycle(0, in, out, true, pred);
+    zq_fuse = false;
+    if (h.L == 1) {
+      klaunch(k_dot_zq<VT>, ew_grid(L0.n), kThreads, s, L0.n, (const VT *)out, (const double *)h.q,
+              fin_args(0, FIN_BETA, L0.partials), pred);
+      check();
+    }
+    return out;
+  }
+
+  // the preconditioner input in VT and x0 from the FP64 residual (before the first
+  // iteration and after a restart; otherwise k_fcg_update leaves them)
+  void input_from_r(const double *r, const int *pred) {
+    Level &L0 = h.lev[0];
+    klaunch(k_to_vt<VT>, ew_grid(L0.n), kThreads, s, L0.n, r, V(h.pre_in), V(L0.wd), V(L0.tmp), pred);
+    check();
+  }
+
   // z = M r for the FP64 outer iteration
-  void precond(const double *r, double *z, const int *pred, bool with_zq) {
+  void precond(const double *r, double *z, const int *pred) {
     Level &L0 = h.lev[0];
     if (std::is_same<VT, double>::value) {
-      zq_fuse = with_zq;
       cycle(0, (const VT *)r, (VT *)z, false, pred);
-      zq_fuse = false;
-      if (with_zq && h.L == 1) {
-        klaunch(k_dot64, ew_grid(L0.n), kThreads, s, L0.n, z, h.q, L0.partials + 4 * kRedBlocks, pred);
-        check();
-      }
     } else {
-      klaunch(k_to_vt<VT>, ew_grid(L0.n), kThreads, s, L0.n, r, V(h.pre_in), V(L0.wd), V(L0.tmp), pred);
-      check();
+      input_from_r(r, pred);
       cycle(0, V(h.pre_in), V(h.pre_out), true, pred);
-      klaunch(k_from_vt_dot<VT>, ew_grid(L0.n), kThreads, s, L0.n, V(h.pre_out), z, h.q,
-                                                           L0.partials + 4 * kRedBlocks, pred);
+      klaunch(k_from_vt<VT>, ew_grid(L0.n), kThreads, s, L0.n, (const VT *)V(h.pre_out), z, pred);
       check();
     }
   }
@@ -1400,7 +1443,7 @@ struct Engine {
       ++launches;
     }
     // z = M r
-    precond(h.r, h.z, nullptr, false);
+    precond(h.r, h.z, nullptr);
     Engine<double, double> e64(h, s);
     e64.segdot(0, 1, h.z, h.q, nullptr, nullptr, nullptr, nullptr, S_ZQ, nullptr);
     launches += e64.launches;
@@ -1417,7 +1460,7 @@ struct Engine {
       a.x = h.pdir;
       a.out = h.q;
       a.live = L0.slive;
-      klaunch(k_sell<double, double, E_Y, false, true>, outer_grid(L0), kThreads, s, a);
+      klaunch(k_sell<double, double, E_Y, 0, true>, outer_grid(L0), kThreads, s, a);
     }
     launches += 3;
     e64.launches = 0;
@@ -1434,18 +1477,15 @@ struct Engine {
   }
 
   // one flexible-CG iteration, all on the device (graph-capturable)
-  void fcg_iteration(int *active, int *restart) {
+  void fcg_iteration(int *active, int *restart, volatile int *host_state) {
     Level &L0 = h.lev[0];
-    double *part = L0.partials;
     const int ng = ew_grid(L0.n);
-    const int nsg = outer_grid(L0);  // FP64 q = A p and its two inner products
-    const int nzq = (std::is_same<VT, double>::value && h.L > 1) ? sell_grid(L0) : ng;  // z^T q of the cycle
-    // z = M r (+ z^T q partials)
-    precond(h.r, h.z, active, true);
+    // z = M r, z^T q and beta
+    const VT *z = precond_fcg(active);
     // p = z + beta p
-    klaunch(k_fcg_p, ng, kThreads, s, L0.n, h.z, h.pdir, part + 4 * kRedBlocks, nzq, L0.slots, restart, active);
+    klaunch(k_fcg_p<VT>, ng, kThreads, s, L0.n, z, h.pdir, (const double *)L0.slots, (const int *)restart, active);
     check();
-    {  // q = A p (FP64), p^T q, p^T r
+    {  // q = A p (FP64), p^T q, p^T r, alpha
       SellArgs<double> a{};
       a.n = L0.n;
       a.nslices = L0.nslices;
@@ -1455,22 +1495,16 @@ struct Engine {
       a.x = h.pdir;
       a.out = h.q;
       a.u1 = h.r;
-      a.ndot = 2;
-      a.dop[0][0] = OP_X; a.dop[0][1] = OP_Y;
-      a.dop[1][0] = OP_X; a.dop[1][1] = OP_U1;
-      a.partials = part + 5 * kRedBlocks;
+      a.fin = fin_args(0, FIN_ALPHA, L0.partials);
       a.pred = active;
-      klaunch(k_sell<double, double, E_Y, true, false>, nsg, kThreads, s, a);
+      klaunch(k_sell<double, double, E_Y, 2, false>, outer_grid(L0), kThreads, s, a);
       check();
     }
-    // x, r update (+ the next preconditioner input in reduced precision)
-    const bool red = !std::is_same<VT, double>::value;
-    klaunch(k_fcg_update<VT>, ng, kThreads, s, L0.n, h.x, h.r, h.pdir, h.q, part + 5 * kRedBlocks, nsg, L0.slots,
-                                             part + 7 * kRedBlocks, nullptr, V(L0.wd), V(L0.tmp), active);
-    check();
-    (void)red;
-    klaunch(k_fcg_fin, 1, kThreads, s, part + 7 * kRedBlocks, ng, L0.slots, h.hist, h.it_dev, active, restart,
-                                     h.status_dev);
+    // x, r update, the next preconditioner input, and the end of the iteration
+    const FcgState st{h.hist, h.it_dev, active, restart, h.status_dev, host_state};
+    klaunch(k_fcg_update<VT>, ng, kThreads, s, L0.n, h.x, h.r, (const double *)h.pdir, (const double *)h.q, L0.slots,
+            L0.partials, ticket(L0), std::is_same<VT, double>::value ? (VT *)nullptr : V(h.pre_in),
+            (const VT *)V(L0.wd), V(L0.tmp), st, active);
     check();
   }
 };
@@ -1696,6 +1730,13 @@ int run_solve_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *i
     klaunch(k_set_state, 1, 32, s, h.it_dev, active, restart, h.status_dev, 0, 1, 1, 0);
     AMG_CUDA(cudaMemcpyAsync(h.hist, &hist[0], sizeof(double), cudaMemcpyHostToDevice, s));
     AMG_LAUNCH_CHECK();
+    // the state of the iteration in mapped pinned words that its last kernel writes
+    // (no copy per iteration): [0] iterations, [4] status
+    volatile int *st_host = reinterpret_cast<int *>(h.host_pinned + 32);
+    int *st_dev = nullptr;
+    AMG_CUDA(cudaHostGetDevicePointer(reinterpret_cast<void **>(&st_dev), h.host_pinned + 32, 0));
+    st_host[0] = 0;
+    st_host[4] = 0;
     // capture one outer iteration as a graph
     int64_t per_iter = 0;
     if (h.p.use_graph && h.graph_kind != 0) {
@@ -1705,7 +1746,7 @@ int run_solve_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *i
         h.graph_exec = nullptr;
       }
       AMG_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-      eng.fcg_iteration(active, restart);
+      eng.fcg_iteration(active, restart, st_dev);
       AMG_CUDA(cudaStreamEndCapture(s, &h.graph));
       AMG_CUDA(cudaGraphInstantiate(&h.graph_exec, h.graph, 0));
       h.graph_kind = 0;
@@ -1713,23 +1754,22 @@ int run_solve_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *i
       eng.launches = 0;
     }
     per_iter = h.graph_launches;
+    eng.input_from_r(h.r, nullptr);
     auto enqueue = [&]() {
       if (h.p.use_graph) {
         AMG_CUDA(cudaGraphLaunch(h.graph_exec, s));
         launches += per_iter;
       } else {
-        eng.fcg_iteration(active, restart);
+        eng.fcg_iteration(active, restart, st_dev);
       }
     };
     // The next iteration is queued before this one's state is read, so the GPU
     // does not wait for the host between iterations; once an iteration stops
     // (*active = 0) every kernel of the next one returns at once.
-    int *st_host = reinterpret_cast<int *>(h.host_pinned + 32);  // two slots of 8 ints
     EventPair ep;  // destroyed on every exit, including a throw inside the loop
     cudaEvent_t *evs = ep.e;
     auto launch_iter = [&](int slot) {
       enqueue();
-      AMG_CUDA(cudaMemcpyAsync(st_host + 8 * slot, h.it_dev, sizeof(int) * 8, cudaMemcpyDeviceToHost, s));
       AMG_CUDA(cudaEventRecord(evs[slot], s));
     };
     int slot = 0;
@@ -1737,13 +1777,13 @@ int run_solve_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *i
     for (;;) {
       launch_iter(slot ^ 1);
       AMG_CUDA(cudaEventSynchronize(evs[slot]));
-      const int dst = st_host[8 * slot + 4];
-      it = st_host[8 * slot];
+      const int dst = st_host[4];
       if (dst == 0) {  // still iterating
         slot ^= 1;
         continue;
       }
       AMG_CUDA(cudaStreamSynchronize(s));  // the queued iteration ran and did nothing
+      it = st_host[0];
       if (dst == 1) {  // updated residual meets tol: check the true residual
         true_residual(h, S_TRUE_RR, s, launches);
         AMG_CUDA(cudaMemcpyAsync(h.host_pinned, L0.slots, sizeof(double) * kNumSlots, cudaMemcpyDeviceToHost, s));
@@ -1759,7 +1799,8 @@ int run_solve_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *i
         }
         // iterative refinement: restart flexible CG from the true residual
         klaunch(k_set_state, 1, 32, s, h.it_dev, active, restart, h.status_dev, -1, 1, 1, 0);
-        AMG_LAUNCH_CHECK();
+        eng.input_from_r(h.r, nullptr);
+        st_host[4] = 0;  // the stream is idle
         slot = 0;
         launch_iter(slot);
         continue;
@@ -1844,7 +1885,7 @@ int run_fgmres_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *
     for (int j = 0; j < m; ++j) {
       double *vj = h.V + (size_t)j * n, *zj = h.Z + (size_t)j * n;
       const int64_t before = eng.launches;
-      eng.precond(vj, zj, active, false);
+      eng.precond(vj, zj, active);
       {  // w = A z_j in FP64
         SellArgs<double> a{};
         a.n = n;
@@ -1855,7 +1896,7 @@ int run_fgmres_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *
         a.x = zj;
         a.out = w;
         a.pred = active;
-        klaunch(k_sell<double, double, E_Y, false, false>, outer_grid(L0), kThreads, s, a);
+        klaunch(k_sell<double, double, E_Y, 0, false>, outer_grid(L0), kThreads, s, a);
         eng.check();
       }
       for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
@@ -2152,7 +2193,7 @@ void run_precond_t(Hierarchy &h, const double *b, double *x, cudaStream_t s) {
   const int32_t n = h.lev[0].n;
   if (!h.batched) trace_reset(h, s);
   copy_in(h.r, b, n, s);
-  eng.precond(h.r, h.z, nullptr, false);
+  eng.precond(h.r, h.z, nullptr);
   copy_out(x, h.z, n, s);
   AMG_CUDA(cudaStreamSynchronize(s));
   if (!h.batched) trace_collect(h, 1, s);
