@@ -165,6 +165,8 @@ struct Level {
                               // (set at prepare, autotuned; at most kRedBlocks)
   int32_t sell_plain_blocks = 0;  // grid of the launches without inner products (default: a
                                   // warp per slice)
+  int32_t split_log = -1;     // log2 of the warps that share a slice in the small-level product
+                              // (-1: one warp per slice, k_sell)
   int32_t seg_tile = 0;       // batch: rows per tile of the per-system inner products
   int64_t sell_entries = 0;
   int64_t *sptr = nullptr;
@@ -184,6 +186,7 @@ struct Level {
   int64_t sell64_entries = 0;
   // solve-phase vectors and per-row data in the vector type
   void *wd = nullptr, *dinv = nullptr, *pw = nullptr, *poly = nullptr;
+  void *pwm = nullptr;    // P weights in member order: pwm[m] = pw[amem[m]]
   bool poly_off = false;  // the level's polynomial was cleared: damped Jacobi
   void *r = nullptr, *bc = nullptr, *xc = nullptr, *c = nullptr, *v = nullptr, *rt = nullptr,
        *d = nullptr, *w = nullptr, *tmp = nullptr, *u0 = nullptr, *u1 = nullptr;
@@ -363,6 +366,18 @@ __device__ __forceinline__ void pdl_wait_and_trigger() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+
+// The two halves for the kernels of the cycle.  A kernel lets its successor
+// launch at its start, loads what no kernel of a solve writes (matrix entries,
+// aggregates, weights) and only then waits for its predecessor, so that the
+// chain of dependent loads behind the wait is the gather of the vector alone.
+// The order stays complete: every block of every kernel waits before it reads or
+// writes anything that changes, so a grid ends only after its predecessor has.
+// What is read before the wait is complete before any solve is queued: setup,
+// re-setup and amg_set_poly synchronise before they return.  Vectors are read
+// with plain loads (no ld.global.nc), which the compiler keeps behind the wait.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---------------------------------------------------------------- device utilities
 __device__ __forceinline__ double warp_sum(double v) {

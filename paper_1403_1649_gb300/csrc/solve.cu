@@ -236,53 +236,78 @@ constexpr int sell_min_blocks() { return sizeof(VT) == 4 ? 6 : 4; }
 // plain SpMV does not hold their accumulators in registers)
 // GATE: a batch's launch, skipping slices whose systems have all stopped
 // (compiled only into the batch instantiations)
-// UW: entries a row per step on small levels (0: the default below).  A level of
-// a few hundred slices leaves most of the GPU idle and each warp's chain of
-// dependent loads sets the time, so there every load of a coarse row (15-30
-// entries) goes out in one or two steps.
 // With fused inner products the FP32-vector kernel needs more than the 40
 // registers of six resident blocks (it spilled there): four blocks, 64 registers.
 constexpr int kDotBlocks = 4;
 template <class VT, int ND>
 constexpr int sell_launch_blocks() { return ND ? kDotBlocks : sell_min_blocks<VT>(); }
 
-template <class MV, class VT, int EPI, int ND, bool GATE, int UW = 0>
-__global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<VT, ND>()) k_sell(SellArgs<VT> a) {
-  pdl_wait_and_trigger();
-  if (a.pred && *a.pred == 0) return;
+// row `row` of the epilogue EPI with the row's product y, and the launch's inner products
+template <class VT, int EPI, int ND>
+__device__ __forceinline__ void sell_epilogue(const SellArgs<VT> &a, int32_t row, VT y, double (&acc)[ND ? ND : 1]) {
+  VT o;
+  if (EPI == E_Y) o = y;
+  else if (EPI == E_RESID) o = a.rhs[row] - y;
+  else if (EPI == E_POST) o = a.xin[row] + a.wd[row] * (a.rhs[row] - y);
+  else if (EPI == E_DSCALE) o = a.dinv[row] * y;
+  else if (EPI == E_POLYPRE)
+    o = a.coef[3 * row] * a.p0[row] + a.coef[3 * row + 1] * a.p1[row] + a.coef[3 * row + 2] * (a.dinv[row] * y);
+  else if (EPI == E_RESID_POLY) {
+    o = a.rhs[row] - y;
+    a.out2[row] = a.dinv[row] * (a.coef[3 * row + 2] * o);
+  } else if (EPI == E_HORNER)
+    o = a.dinv[row] * y + a.dinv[row] * (a.coef[3 * row + 1] * a.res[row]);
+  else
+    o = a.xin[row] + (a.dinv[row] * y + a.dinv[row] * (a.coef[3 * row] * a.res[row]));
+  a.out[row] = o;
+  if constexpr (ND == 1) {
+    acc[0] += (double)o * a.q64[row];
+  } else if constexpr (ND >= 2) {
+    const double oy = (double)o, sv = a.dot_y ? oy : (double)a.x[row];
+    acc[0] += sv * oy;
+    acc[1] += sv * (double)a.u1[row];
+    if constexpr (ND == 3) acc[2] += sv * (double)a.u2[row];
+  }
+}
+
+// y = A x over SELL-32, one warp per slice, one lane per row
+template <class MV, class VT, int EPI, int ND, bool GATE>
+__global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell(SellArgs<VT> a) {
+  pdl_trigger();
   const int lane = threadIdx.x & 31;
   const MV *__restrict__ sval = static_cast<const MV *>(a.sval);
   double acc[ND ? ND : 1] = {0.0};
   // U entries of a row per step: 6 with FP32 vectors (a 7-point row without its
   // split-off diagonal in one step, at 40 registers), 8 with FP64
-  constexpr int U = UW ? UW : (sizeof(VT) == 4 ? 6 : 8);
+  constexpr int U = sizeof(VT) == 4 ? 6 : 8;
+  bool first = true, run = true, live = true;
+  // FP32 vectors at 64 registers wait for the predecessor after the first slice's
+  // matrix loads have gone out; at 40 registers, and with FP64 vectors, that spills
+  constexpr bool kAhead = sizeof(VT) == 4 && ND > 0;
+  if constexpr (!kAhead) {
+    pdl_wait();
+    if (a.pred && *a.pred == 0) return;
+    first = false;
+  }
+  auto enter = [&](int32_t sl) {
+    if (!first) return;
+    first = false;
+    pdl_wait();
+    run = !(a.pred && *a.pred == 0);
+    if (GATE) live = sl < a.nslices && a.live[sl];
+  };
   for (int32_t sl = blockIdx.x * kWarps + (threadIdx.x >> 5); sl < a.nslices; sl += gridDim.x * kWarps) {
-    if (GATE && !a.live[sl]) continue;
+    if (GATE && !first) {
+      live = a.live[sl];
+      if (!live) continue;
+    }
     const int32_t row = sl * 32 + lane;
     VT y = VT(0), dg = VT(0), xr = VT(0);
     const bool diag = !std::is_same<MV, double>::value && a.sdiag != nullptr && row < a.n;
-    // small levels (UW): the row's own operands (split diagonal, x_row and the
-    // epilogue's rhs, wd, xin) go out before the slice pointers, so that the
-    // warp's chain of dependent loads is the matrix and the gathers only
-    VT pre_rhs = VT(0), pre_wd = VT(0), pre_xin = VT(0);
-    if constexpr (UW != 0) {
-      if (diag) {
-        dg = (VT)ld_stream(a.sdiag + row);
-        xr = __ldg(a.x + row);
-      }
-      if (row < a.n) {
-        if (EPI == E_RESID || EPI == E_POST) pre_rhs = __ldg(a.rhs + row);
-        if (EPI == E_POST) {
-          pre_wd = __ldg(a.wd + row);
-          pre_xin = __ldg(a.xin + row);
-        }
-      }
-    }
     const int64_t base = a.sptr[sl];
     const int32_t width = (int32_t)((a.sptr[sl + 1] - base) >> 5);
-    // otherwise the split diagonal (FP32 / BF16 values only) and x_row are loaded
-    // right behind the first step's matrix loads, so that their latency overlaps
-    // the gathers
+    // the split diagonal (FP32 / BF16 values only) is loaded right behind the first
+    // step's matrix loads and x_row with the gathers, so that their latency overlaps
     if constexpr (kPairs<MV> || kHalfPairs<MV>) {
       // FP32 values: a lane's entries 2j and 2j+1 come in one 16-byte load;
       // BF16 values: their columns in one 8-byte load and their values in one
@@ -315,14 +340,15 @@ __global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<VT, ND>(
             }
           }
         }
-        if (UW == 0 && e == 0 && diag) {
-          dg = (VT)ld_stream(a.sdiag + row);
-          xr = __ldg(a.x + row);
+        if (e == 0) {
+          if (diag) dg = (VT)ld_stream(a.sdiag + row);
+          enter(sl);
+          if (diag) xr = a.x[row];
         }
         VT xv[S];
 #pragma unroll
         for (int q = 0; q < S; ++q)
-          if (FULL || e + q < width) xv[q] = __ldg(a.x + c[q]);
+          if (FULL || e + q < width) xv[q] = a.x[c[q]];
 #pragma unroll
         for (int q = 0; q < S; ++q)
           if (FULL || e + q < width) y += v[q] * xv[q];
@@ -331,9 +357,9 @@ __global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<VT, ND>(
       // one step without predicates, whose loads all go out before the first gather
       using UStep = std::integral_constant<int, U>;
       using U2Step = std::integral_constant<int, U + 2>;
-      if (UW == 0 && width == U) {
+      if (width == U) {
         step(0, std::true_type{}, UStep{});
-      } else if (UW == 0 && width == U + 2) {
+      } else if (width == U + 2) {
         step(0, std::true_type{}, U2Step{});
       } else {
         for (int32_t e = 0; e < width; e += U) step(e, std::false_type{}, UStep{});
@@ -351,19 +377,19 @@ __global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<VT, ND>(
             v[q] = ld_stream(vp + 32 * (e + q));
           }
         }
-        if (UW == 0 && e == 0 && diag) {
-          dg = (VT)ld_stream(a.sdiag + row);
-          xr = __ldg(a.x + row);
-        }
+        if (e == 0) enter(sl);
         VT xv[U];
 #pragma unroll
         for (int q = 0; q < U; ++q)
-          if (e + q < width) xv[q] = __ldg(a.x + c[q]);
+          if (e + q < width) xv[q] = a.x[c[q]];
 #pragma unroll
         for (int q = 0; q < U; ++q)
           if (e + q < width) y += to_acc(v[q], VT(0)) * xv[q];
       }
     }
+    enter(sl);  // a slice without entries has not waited yet
+    if (!run) return;
+    if (GATE && !live) continue;
     if (diag) {
       if (width == 0) {  // a row without off-diagonal entries
         dg = (VT)a.sdiag[row];
@@ -371,90 +397,224 @@ __global__ void __launch_bounds__(kThreads, UW ? 1 : sell_launch_blocks<VT, ND>(
       }
       y += dg * xr;
     }
-    if (row < a.n) {
-      VT o;
-      if (EPI == E_Y) o = y;
-      else if (EPI == E_RESID) o = (UW ? pre_rhs : a.rhs[row]) - y;
-      else if (EPI == E_POST)
-        o = UW ? pre_xin + pre_wd * (pre_rhs - y) : a.xin[row] + a.wd[row] * (a.rhs[row] - y);
-      else if (EPI == E_DSCALE) o = a.dinv[row] * y;
-      else if (EPI == E_POLYPRE)
-        o = a.coef[3 * row] * a.p0[row] + a.coef[3 * row + 1] * a.p1[row] + a.coef[3 * row + 2] * (a.dinv[row] * y);
-      else if (EPI == E_RESID_POLY) {
-        o = a.rhs[row] - y;
-        a.out2[row] = a.dinv[row] * (a.coef[3 * row + 2] * o);
-      } else if (EPI == E_HORNER)
-        o = a.dinv[row] * y + a.dinv[row] * (a.coef[3 * row + 1] * a.res[row]);
-      else
-        o = a.xin[row] + (a.dinv[row] * y + a.dinv[row] * (a.coef[3 * row] * a.res[row]));
-      a.out[row] = o;
-      if constexpr (ND == 1) {
-        acc[0] += (double)o * a.q64[row];
-      } else if constexpr (ND >= 2) {
-        const double oy = (double)o, sv = a.dot_y ? oy : (double)a.x[row];
-        acc[0] += sv * oy;
-        acc[1] += sv * (double)a.u1[row];
-        if constexpr (ND == 3) acc[2] += sv * (double)a.u2[row];
+    if (row < a.n) sell_epilogue<VT, EPI, ND>(a, row, y, acc);
+  }
+  enter(a.nslices);  // a warp without a slice
+  if (!run) return;
+  if constexpr (ND > 0) grid_dots<ND>(acc, 1, a.fin);
+}
+
+// The product on a small level (at most kSmallSlices slices): 2^wl warps share a
+// slice, warp q taking its entries q, q + 2^wl, ... (pairs of entries for FP32 and
+// BF16 values), and meet in shared memory in warp order.  Such a level leaves most
+// of the GPU idle and lives in L2, so its time is one warp's chain of dependent
+// loads: splitting the rows shortens the chain to one step whose matrix loads all
+// go out before the wait for the predecessor.
+template <class MV, class VT, int EPI, int ND, bool GATE>
+__global__ void __launch_bounds__(kThreads) k_sell_small(SellArgs<VT> a, int wl) {
+  pdl_trigger();
+  __shared__ VT sh[kWarps][32];
+  constexpr int U = 8;  // entries of a warp per step
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int wps = 1 << wl, sub = wid & (wps - 1), spb = kWarps >> wl;
+  const MV *__restrict__ sval = static_cast<const MV *>(a.sval);
+  double acc[ND ? ND : 1] = {0.0};
+  bool first = true;
+  for (int32_t s0 = blockIdx.x * spb; s0 < a.nslices; s0 += gridDim.x * spb) {
+    const int32_t sl = s0 + (wid >> wl);
+    const bool in = sl < a.nslices;
+    const int32_t row = sl * 32 + lane;
+    const bool mine = sub == 0 && in && row < a.n;  // this thread finishes the row
+    const int64_t base = in ? a.sptr[sl] : 0;
+    const int32_t width = in ? (int32_t)((a.sptr[sl + 1] - base) >> 5) : 0;
+    VT dg = VT(0);
+    if (!std::is_same<MV, double>::value && mine && a.sdiag) dg = (VT)a.sdiag[row];
+    VT y = VT(0);
+    auto step = [&](int32_t e0, auto &&between) {
+      int32_t c[U];
+      VT v[U];
+      if constexpr (kPairs<MV> || kHalfPairs<MV>) {
+        const int4 *__restrict__ pp = a.spair + (base >> 1) + lane;
+        const int2 *__restrict__ cp2 = reinterpret_cast<const int2 *>(a.scol + base) + lane;
+        const __nv_bfloat162 *__restrict__ vp2 = reinterpret_cast<const __nv_bfloat162 *>(sval + base) + lane;
+#pragma unroll
+        for (int q = 0; q < U; q += 2) {
+          const int32_t pr = (e0 >> 1) + sub + (q >> 1) * wps;  // this warp's next pair
+          c[q] = c[q + 1] = -1;
+          if (2 * pr < width) {
+            if constexpr (kPairs<MV>) {
+              const int4 p4 = __ldg(pp + 32 * pr);
+              c[q] = p4.x;
+              v[q] = __int_as_float(p4.y);
+              c[q + 1] = p4.z;
+              v[q + 1] = __int_as_float(p4.w);
+            } else {
+              const int2 cc = __ldg(cp2 + 32 * pr);
+              const float2 vv = __bfloat1622float2(vp2[32 * pr]);
+              c[q] = cc.x;
+              c[q + 1] = cc.y;
+              v[q] = vv.x;
+              v[q + 1] = vv.y;
+            }
+          }
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < U; ++q) {
+          const int32_t e = e0 + sub + q * wps;
+          c[q] = -1;
+          if (e < width) {
+            c[q] = __ldg(a.scol + base + 32 * (int64_t)e + lane);
+            v[q] = to_acc(sval[base + 32 * (int64_t)e + lane], VT(0));
+          }
+        }
       }
+      between();
+      VT xv[U];
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (c[q] >= 0) xv[q] = a.x[c[q]];
+#pragma unroll
+      for (int q = 0; q < U; ++q)
+        if (c[q] >= 0) y += v[q] * xv[q];
+    };
+    bool run = true;
+    step(0, [&] {
+      if (!first) return;
+      first = false;
+      pdl_wait();
+      run = !(a.pred && *a.pred == 0);
+    });
+    if (!run) return;  // the same in every thread of the grid
+    const bool live = !GATE || (in && a.live[sl]);  // of a batch: a dead slice is not stored
+    if (live)
+      for (int32_t e0 = U * wps; e0 < width; e0 += U * wps) step(e0, [] {});
+    if (wps > 1) {
+      if (s0 != (int32_t)blockIdx.x * spb) __syncthreads();  // the last slice's sums have been read
+      if (sub) sh[wid][lane] = y;
+      __syncthreads();
+      if (sub == 0)
+        for (int q = 1; q < wps; ++q) y += sh[wid + q][lane];
+    }
+    if (mine && live) {
+      if (!std::is_same<MV, double>::value && a.sdiag) y += dg * a.x[row];
+      sell_epilogue<VT, EPI, ND>(a, row, y, acc);
     }
   }
-  if constexpr (ND > 0) grid_dots<ND>(acc, 1, a.fin);
+  if (first) {  // a block without a slice
+    pdl_wait();
+    if (a.pred && *a.pred == 0) return;
+  }
+  if constexpr (ND > 0) grid_dots<ND>(acc, wps, a.fin);
 }
 
 // out = wd * rhs: damped Jacobi from a zero initial guess
 template <class VT>
-__global__ void k_scale(int32_t n, VT *__restrict__ out, const VT *__restrict__ wd, const VT *__restrict__ rhs,
-                        const int *pred, const int32_t *sys, const int *bact) {
-  pdl_wait_and_trigger();
+__global__ void k_scale(int32_t n, VT *out, const VT *__restrict__ wd, const VT *rhs, const int *pred,
+                        const int32_t *__restrict__ sys, const int *bact) {
+  pdl_trigger();
+  const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  VT w = i0 < n ? wd[i0] : VT(0);
+  pdl_wait();
   if (pred && *pred == 0) return;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    if (!bact || bact[sys[i]]) out[i] = wd[i] * rhs[i];
-}
-
-// sum_{i in G_I} P(i, I) r(i) over the members amem[m0..m1) in their (ascending) order
-template <class VT>
-__device__ __forceinline__ VT restrict_row(int32_t m0, int32_t m1, const int32_t *__restrict__ amem,
-                                          const VT *__restrict__ pw, const VT *__restrict__ r) {
-  VT s = VT(0);
-  for (int32_t m = m0; m < m1; ++m) {
-    const int32_t i = amem[m];
-    s += pw[i] * r[i];
+  for (int32_t i = i0; i < n; i += gridDim.x * blockDim.x) {
+    if (i != i0) w = wd[i];
+    if (!bact || bact[sys[i]]) out[i] = w * rhs[i];
   }
-  return s;
 }
 
-// r_{k+1}(I) = sum_{i in G_I} P(i, I) r_k(i) in ascending fine index; also the
-// next level's smoothing start x0 = wd_{k+1} * r_{k+1} when that level smooths.
+// r_{k+1}(I) = sum_{i in G_I} P(i, I) r_k(i); also the next level's smoothing start
+// x0 = wd_{k+1} * r_{k+1} when that level smooths.  kRestrictLanes lanes share an
+// aggregate (members t, t + 4, ... and a fixed shuffle tree); the members and
+// weights of the first 16 are loaded before the wait, so that one gather is left
+// behind it.  Aggregates hold ~5 to 11 rows, at most a few dozen.
+constexpr int kRestrictLanes = 4;
+constexpr int kRestrictAhead = 4;  // members a lane loads ahead
 template <class VT>
-__global__ void k_restrict(int32_t nc, const int32_t *__restrict__ aptr, const int32_t *__restrict__ amem,
-                           const VT *__restrict__ pw, const VT *__restrict__ r, VT *__restrict__ bc,
-                           const VT *__restrict__ wdc, VT *__restrict__ x0c, const int *pred,
-                           const int32_t *sysc, const int *bact) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  for (int32_t I = blockIdx.x * blockDim.x + threadIdx.x; I < nc; I += gridDim.x * blockDim.x) {
-    if (bact && !bact[sysc[I]]) continue;
-    const VT s = restrict_row(aptr[I], aptr[I + 1], amem, pw, r);
-    bc[I] = s;
-    if (wdc) x0c[I] = wdc[I] * s;
+struct Members {
+  int32_t i[kRestrictAhead];
+  VT p[kRestrictAhead];
+  int32_t m0, m1;
+  __device__ __forceinline__ void load(bool in, int32_t I, int t, const int32_t *__restrict__ aptr,
+                                       const int32_t *__restrict__ amem, const VT *__restrict__ pwm) {
+    m0 = in ? aptr[I] : 0;
+    m1 = in ? aptr[I + 1] : 0;
+#pragma unroll
+    for (int u = 0; u < kRestrictAhead; ++u) {
+      const int32_t m = m0 + t + u * kRestrictLanes;
+      i[u] = -1;
+      if (m < m1) {
+        i[u] = amem[m];
+        p[u] = pwm[m];
+      }
+    }
+  }
+  // sum over the members, the same in the aggregate's lanes
+  __device__ __forceinline__ VT sum(int t, const int32_t *__restrict__ amem, const VT *__restrict__ pwm, const VT *r) {
+    VT v[kRestrictAhead], s = VT(0);
+#pragma unroll
+    for (int u = 0; u < kRestrictAhead; ++u)
+      if (i[u] >= 0) v[u] = r[i[u]];
+#pragma unroll
+    for (int u = 0; u < kRestrictAhead; ++u)
+      if (i[u] >= 0) s += p[u] * v[u];
+    for (int32_t m = m0 + t + kRestrictAhead * kRestrictLanes; m < m1; m += kRestrictLanes) s += pwm[m] * r[amem[m]];
+#pragma unroll
+    for (int o = kRestrictLanes / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  }
+};
+
+template <class VT>
+__global__ void __launch_bounds__(kThreads) k_restrict(int32_t nc, const int32_t *__restrict__ aptr,
+                                                       const int32_t *__restrict__ amem, const VT *__restrict__ pwm,
+                                                       const VT *r, VT *bc, const VT *__restrict__ wdc, VT *x0c,
+                                                       const int *pred, const int32_t *__restrict__ sysc,
+                                                       const int *bact) {
+  pdl_trigger();
+  const int t = threadIdx.x % kRestrictLanes;
+  const int32_t per = gridDim.x * (kThreads / kRestrictLanes);
+  const int32_t rounds = (nc + per - 1) / per;  // every lane of a warp runs the same rounds
+  int32_t I = blockIdx.x * (kThreads / kRestrictLanes) + threadIdx.x / kRestrictLanes;
+  for (int32_t q = 0; q < rounds; ++q, I += per) {
+    const bool in = I < nc;
+    Members<VT> mb;
+    mb.load(in, I, t, aptr, amem, pwm);
+    const VT w = in && wdc ? wdc[I] : VT(0);
+    if (q == 0) {
+      pdl_wait();
+      if (pred && *pred == 0) return;
+    }
+    const VT s = mb.sum(t, amem, pwm, r);
+    if (in && t == 0 && (!bact || bact[sysc[I]])) {
+      bc[I] = s;
+      if (wdc) x0c[I] = w * s;
+    }
   }
 }
 
 // x_k += P_k x_{k+1}: a gather through the aggregate map
 template <class VT>
-__global__ void k_prolong(int32_t n, const int32_t *__restrict__ agg, const VT *__restrict__ pw,
-                          const VT *__restrict__ xc, VT *__restrict__ x, const int *pred, const int32_t *sys,
-                          const int *bact) {
-  pdl_wait_and_trigger();
+__global__ void k_prolong(int32_t n, const int32_t *__restrict__ agg, const VT *__restrict__ pw, const VT *xc, VT *x,
+                          const int *pred, const int32_t *__restrict__ sys, const int *bact) {
+  pdl_trigger();
+  const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  int32_t g = i0 < n ? agg[i0] : 0;
+  VT p = i0 < n ? pw[i0] : VT(0);
+  pdl_wait();
   if (pred && *pred == 0) return;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    if (!bact || bact[sys[i]]) x[i] += pw[i] * xc[agg[i]];
+  for (int32_t i = i0; i < n; i += gridDim.x * blockDim.x) {
+    if (i != i0) {
+      g = agg[i];
+      p = pw[i];
+    }
+    if (!bact || bact[sys[i]]) x[i] += p * xc[g];
+  }
 }
 
 // exact coarsest solve x = A_L^-1 b (one warp per row, FP64 accumulation)
 template <class VT>
-__global__ void k_coarse(int32_t nL, const double *__restrict__ Ainv, const VT *__restrict__ b, VT *__restrict__ x,
-                         const VT *__restrict__ wdc_unused, const int *pred) {
+__global__ void k_coarse(int32_t nL, const double *__restrict__ Ainv, const VT *b, VT *x, const int *pred) {
   pdl_wait_and_trigger();
   if (pred && *pred == 0) return;
   const int lane = threadIdx.x & 31;
@@ -468,21 +628,48 @@ __global__ void k_coarse(int32_t nL, const double *__restrict__ Ainv, const VT *
 
 // restriction to the coarsest level and its exact solve in one launch: every
 // block forms r_L = R r (as k_restrict does) in shared memory, then its warps
-// take rows of x = A_L^-1 r_L (as k_coarse does)
+// take rows of x = A_L^-1 r_L.  The rows go round the blocks, one block an SM:
+// an FP64 warp instruction takes 16 cycles of an SM, so the rows' dot products
+// are spread over all of them.  The members of the first two passes of the
+// restriction and a warp's first 256 entries of A_L^-1 are loaded before the wait.
 constexpr int kFusedCoarseMax = 2048;
+constexpr int kCoarseThreads = 512;
 template <class VT>
-__global__ void k_restrict_coarse(int32_t nL, const int32_t *__restrict__ aptr, const int32_t *__restrict__ amem,
-                                  const VT *__restrict__ pw, const VT *__restrict__ r, const double *__restrict__ Ainv,
-                                  VT *__restrict__ x, const int *pred) {
+__global__ void __launch_bounds__(kCoarseThreads, 1) k_restrict_coarse(
+    int32_t nL, const int32_t *__restrict__ aptr, const int32_t *__restrict__ amem, const VT *__restrict__ pwm,
+    const VT *r, const double *__restrict__ Ainv, VT *x, const int *pred) {
   __shared__ VT bsh[kFusedCoarseMax];
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  constexpr int kPer = kCoarseThreads / kRestrictLanes;  // aggregates per pass
+  const int t = threadIdx.x % kRestrictLanes, lane = threadIdx.x & 31;
+  int32_t I = threadIdx.x / kRestrictLanes;
+  Members<VT> m0, m1;
+  m0.load(I < nL, I, t, aptr, amem, pwm);
+  m1.load(I + kPer < nL, I + kPer, t, aptr, amem, pwm);
+  int32_t i = blockIdx.x + gridDim.x * (threadIdx.x >> 5);
+  double ar[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int32_t j = lane + 32 * u;
+    ar[u] = i < nL && j < nL ? Ainv[(int64_t)i * nL + j] : 0.0;
+  }
+  pdl_wait();
   if (pred && *pred == 0) return;
-  for (int32_t I = threadIdx.x; I < nL; I += blockDim.x) bsh[I] = restrict_row(aptr[I], aptr[I + 1], amem, pw, r);
+  for (int32_t p = 0; p * kPer < nL; ++p, I += kPer) {
+    if (p == 1) m0 = m1;
+    if (p > 1) m0.load(I < nL, I, t, aptr, amem, pwm);
+    const VT s = m0.sum(t, amem, pwm, r);
+    if (t == 0 && I < nL) bsh[I] = s;
+  }
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  for (int32_t i = blockIdx.x * kWarps + (threadIdx.x >> 5); i < nL; i += gridDim.x * kWarps) {
+  for (bool ahead = true; i < nL; i += gridDim.x * (kCoarseThreads / 32), ahead = false) {
     double s = 0.0;
-    for (int32_t j = lane; j < nL; j += 32) s += Ainv[(int64_t)i * nL + j] * (double)bsh[j];
+    if (ahead) {
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (32 * u < nL) s += ar[u] * (lane + 32 * u < nL ? (double)bsh[lane + 32 * u] : 0.0);
+    }
+    for (int32_t j = lane + (ahead ? 256 : 0); j < nL; j += 32) s += Ainv[(int64_t)i * nL + j] * (double)bsh[j];
     s = warp_sum(s);
     if (lane == 0) x[i] = (VT)s;
   }
@@ -511,23 +698,25 @@ __device__ __forceinline__ double sum_partials(const double *__restrict__ part, 
 // test of Alg. 5 in the last block: the second inner step runs iff the enclosing
 // step runs and ||r~|| > t ||r||.  A skipped enclosing step clears the flag.
 template <class VT>
-__global__ void __launch_bounds__(kThreads) k_axpy_rt(int32_t n, const VT *__restrict__ r, const VT *__restrict__ v,
-                                                      VT *__restrict__ rt, const VT *__restrict__ wd,
-                                                      VT *__restrict__ x0, double t, double *__restrict__ slots,
-                                                      int *__restrict__ flag, double *part, unsigned *ticket,
-                                                      const int *pred) {
-  pdl_wait_and_trigger();
+__global__ void __launch_bounds__(kThreads) k_axpy_rt(int32_t n, const VT *r, const VT *v, VT *rt,
+                                                      const VT *__restrict__ wd, VT *x0, double t, double *slots,
+                                                      int *flag, double *part, unsigned *ticket, const int *pred) {
+  pdl_trigger();
+  const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  VT w = i0 < n ? wd[i0] : VT(0);
+  pdl_wait();
   if (pred && *pred == 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
     return;
   }
   const VT s1 = (VT)slots[S_S1];
   double acc[2] = {0.0, 0.0};
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  for (int32_t i = i0; i < n; i += gridDim.x * blockDim.x) {
+    if (i != i0) w = wd[i];
     const VT ri = r[i];
     const VT ti = ri - s1 * v[i];
     rt[i] = ti;
-    if (wd) x0[i] = wd[i] * ti;
+    x0[i] = w * ti;
     acc[0] += (double)ti * (double)ti;
     acc[1] += (double)ri * (double)ri;
   }
@@ -545,7 +734,8 @@ __global__ void __launch_bounds__(kThreads) k_axpy_rt(int32_t n, const VT *__res
 template <class VT>
 __global__ void k_combine(int32_t n, const VT *__restrict__ c, const VT *__restrict__ d, VT *__restrict__ x,
                           const double *__restrict__ slots, const int *__restrict__ flag, const int *pred) {
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   const bool two = *flag != 0;
   const VT cc = (VT)(two ? slots[S_CC] : slots[S_S1]);
@@ -558,7 +748,8 @@ __global__ void k_combine(int32_t n, const VT *__restrict__ c, const VT *__restr
 template <class VT>
 __global__ void k_to_vt(int32_t n, const double *__restrict__ in, VT *__restrict__ out, const VT *__restrict__ wd,
                         VT *__restrict__ x0, const int *pred) {
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const VT v = (VT)in[i];
@@ -570,7 +761,8 @@ __global__ void k_to_vt(int32_t n, const double *__restrict__ in, VT *__restrict
 // z = (double) zin
 template <class VT>
 __global__ void k_from_vt(int32_t n, const VT *__restrict__ zin, double *__restrict__ z, const int *pred) {
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) z[i] = (double)zin[i];
 }
@@ -580,7 +772,8 @@ __global__ void k_from_vt(int32_t n, const VT *__restrict__ zin, double *__restr
 template <class VT>
 __global__ void __launch_bounds__(kThreads) k_dot_zq(int32_t n, const VT *__restrict__ z, const double *__restrict__ q,
                                                      FinArgs fin, const int *pred) {
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   double acc[1] = {0.0};
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
@@ -592,7 +785,8 @@ __global__ void __launch_bounds__(kThreads) k_dot_zq(int32_t n, const VT *__rest
 template <class VT>
 __global__ void k_fcg_p(int32_t n, const VT *__restrict__ z, double *__restrict__ p, const double *__restrict__ slots,
                         const int *__restrict__ restart, const int *pred) {
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   const bool rs = *restart != 0;
   const double beta = slots[S_BETA];
@@ -616,7 +810,8 @@ __global__ void __launch_bounds__(kThreads) k_fcg_update(int32_t n, double *__re
                                                          double *__restrict__ slots, double *part, unsigned *ticket,
                                                          VT *__restrict__ rvt, const VT *__restrict__ wd,
                                                          VT *__restrict__ x0, FcgState st, const int *pred) {
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   const double alpha = slots[S_ALPHA];
   double acc[1] = {0.0};
@@ -993,7 +1188,8 @@ template <class VT>
 __global__ void k_bcoarse(int32_t nL, const int32_t *__restrict__ sys, const int32_t *__restrict__ off,
                           const double *__restrict__ binv, const int64_t *__restrict__ boff, const VT *__restrict__ b,
                           VT *__restrict__ x, const int *pred) {
-  pdl_wait_and_trigger();
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   const int lane = threadIdx.x & 31;
   for (int32_t i = blockIdx.x * kWarps + (threadIdx.x >> 5); i < nL; i += gridDim.x * kWarps) {
@@ -1091,13 +1287,17 @@ __global__ void k_bfcg_fin(int32_t nsys, double *__restrict__ bslots, int *__res
 template <class VT>
 __global__ void k_convert_row_data(int32_t n, const double *__restrict__ diag, double omega_host,
                                    const double *__restrict__ omega_dev, const double *__restrict__ pw64,
-                                   VT *__restrict__ wd, VT *__restrict__ dinv, VT *__restrict__ pw) {
+                                   VT *__restrict__ wd, VT *__restrict__ dinv, VT *__restrict__ pw,
+                                   const int32_t *__restrict__ amem, VT *__restrict__ pwm) {
   pdl_wait_and_trigger();
   const double omega = omega_dev ? *omega_dev : omega_host;
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     wd[i] = (VT)(omega / diag[i]);
     dinv[i] = (VT)(1.0 / diag[i]);
-    if (pw64) pw[i] = (VT)pw64[i];
+    if (pw64) {
+      pw[i] = (VT)pw64[i];
+      pwm[i] = (VT)pw64[amem[i]];
+    }
   }
 }
 
@@ -1132,11 +1332,20 @@ inline int dot_grid(const Level &L) { return std::min(L.sell_blocks, kDotBlocks 
 // level 0: 34.4 against 27.4 us under ncu)
 inline int full_plain_grid(const Level &L) { return grid_for((int64_t)L.nslices, kWarps, 1 << 30); }
 inline int plain_grid(const Level &L) { return L.sell_plain_blocks; }
-// levels of at most kSmallSlices slices (fewer warps than the GPU holds at a
-// quarter of its occupancy) run the products with kSmallU entries a step, with
-// FP32 vectors (measured: no gain with FP64 vectors)
+// Levels of at most kSmallSlices slices (fewer warps than the GPU holds at a
+// quarter of its occupancy) run the product with 2^split_log warps a slice: enough
+// that a warp takes its entries in one step of eight, or until the level has
+// kSplitWarps warps (the GPU's at three quarters of its occupancy), beyond which
+// more warps only wait for each other.
 constexpr int32_t kSmallSlices = 2048;
-constexpr int kSmallU = 16;
+constexpr int32_t kSplitWarps = 152 * 48;
+inline int split_log_for(const Level &L) {
+  if (L.nslices > kSmallSlices || L.nslices == 0) return -1;
+  const int64_t width = L.sell_entries / (32 * (int64_t)L.nslices);  // average entries a row
+  int wl = 0;
+  while (wl < 3 && (width >> wl) > 6 && ((int64_t)L.nslices << (wl + 1)) <= kSplitWarps) ++wl;
+  return wl;
+}
 inline int outer_grid(const Level &L0) { return default_sell_grid<double>(L0); }
 
 template <class MV, class VT>
@@ -1185,20 +1394,23 @@ struct Engine {
   // post-smoothing step of level 0 (z^T q of the outer flexible CG)
   template <int EPI, int ND = 0>
   void sell(const SellArgs<VT> &a, int k) {
-    if (h.batched) {  // no fused inner products in a batch: they are per system (segdot)
-      if (ND) throw Error{AMG_ERR_UNSUPPORTED, "batched SpMV was given fused inner products"};
-      klaunch(k_sell<MV, VT, EPI, 0, true>, plain_grid(h.lev[k]), kThreads, s, a);
-      check();
-      return;
-    }
-    const int grid = ND ? dot_grid(h.lev[k]) : plain_grid(h.lev[k]);
-    if constexpr ((EPI == E_Y || EPI == E_RESID || EPI == E_POST) && sizeof(VT) == 4)
-      if (h.lev[k].nslices <= kSmallSlices) {
-        klaunch(k_sell<MV, VT, EPI, ND, false, kSmallU>, grid, kThreads, s, a);
+    const Level &L = h.lev[k];
+    if (h.batched && ND)  // inner products of a batch are per system (segdot)
+      throw Error{AMG_ERR_UNSUPPORTED, "batched SpMV was given fused inner products"};
+    if constexpr (EPI == E_Y || EPI == E_RESID || EPI == E_POST)
+      if (L.split_log >= 0) {
+        const int grid = grid_for(L.nslices, kWarps >> L.split_log, kRedBlocks);
+        if (h.batched)
+          klaunch(k_sell_small<MV, VT, EPI, 0, true>, grid, kThreads, s, a, (int)L.split_log);
+        else
+          klaunch(k_sell_small<MV, VT, EPI, ND, false>, grid, kThreads, s, a, (int)L.split_log);
         check();
         return;
       }
-    klaunch(k_sell<MV, VT, EPI, ND, false>, grid, kThreads, s, a);
+    if (h.batched)
+      klaunch(k_sell<MV, VT, EPI, 0, true>, plain_grid(L), kThreads, s, a);
+    else
+      klaunch(k_sell<MV, VT, EPI, ND, false>, ND ? dot_grid(L) : plain_grid(L), kThreads, s, a);
     check();
   }
 
@@ -1211,7 +1423,7 @@ struct Engine {
         klaunch(k_bcoarse<VT>, grid_for(h.nL, kWarps, 152 * 8), kThreads, s, h.nL, (const int32_t *)L.sys_of,
                 (const int32_t *)L.sys_off, (const double *)h.binv, (const int64_t *)h.binv_off, rhs, out, pred);
       else
-        klaunch(k_coarse<VT>, grid_for(h.nL, kWarps, 152), kThreads, s, h.nL, h.coarse_inv, rhs, out, nullptr, pred);
+        klaunch(k_coarse<VT>, grid_for(h.nL, kWarps, 152), kThreads, s, h.nL, h.coarse_inv, rhs, out, pred);
       check();
       return;
     }
@@ -1244,13 +1456,14 @@ struct Engine {
     // single systems: the restriction to the coarsest level and its solve in one launch
     const bool fuse_coarse = coarse_is_last && !tail && !h.batched && h.nL <= kFusedCoarseMax;
     if (fuse_coarse) {
-      klaunch(k_restrict_coarse<VT>, grid_for(h.nL, kWarps, 152), kThreads, s, h.nL, L.aptr, L.amem, V(L.pw),
-              V(L.r), h.coarse_inv, V(C.xc), pred);
+      klaunch(k_restrict_coarse<VT>, std::min(h.nL, 152), kCoarseThreads, s, h.nL, L.aptr, L.amem,
+              (const VT *)V(L.pwm), (const VT *)V(L.r), h.coarse_inv, V(C.xc), pred);
       check();
     } else {
       // r_{k+1} = R_k r_k  (and x0 of level k+1 when it smooths)
-      klaunch(k_restrict<VT>, ew_grid(L.nc), kThreads, s, L.nc, L.aptr, L.amem, V(L.pw), V(L.r), V(C.bc),
-              (coarse_is_last || tail) ? nullptr : V(C.wd), V(C.tmp), pred, bsys(C), bact());
+      klaunch(k_restrict<VT>, grid_for((int64_t)L.nc * kRestrictLanes, kThreads, 152 * 32), kThreads, s, L.nc, L.aptr,
+              L.amem, (const VT *)V(L.pwm), (const VT *)V(L.r), V(C.bc),
+              (const VT *)((coarse_is_last || tail) ? nullptr : V(C.wd)), V(C.tmp), pred, bsys(C), bact());
       check();
     }
     if (tail) {  // levels k+1..L-1 in one cluster launch
@@ -1528,6 +1741,7 @@ void alloc_level_vectors(Hierarchy &h, Level &L, int k) {
   }
   if (L.sell_blocks <= 0) L.sell_blocks = default_sell_grid<VT>(L);
   if (L.sell_plain_blocks <= 0) L.sell_plain_blocks = L.sell_blocks;
+  L.split_log = split_log_for(L);
   L.slots = h.arena.get<double>(kNumSlots);
   L.flag = h.arena.get<int>(4);
   L.partials = h.arena.get<double>((size_t)kRedBlocks * 8);
@@ -1623,9 +1837,10 @@ void make_row_data_t(Hierarchy &h, Level &L, const double *diag, cudaStream_t s)
     L.wd = h.arena.get<VT>((size_t)L.n + 1);
     L.dinv = h.arena.get<VT>((size_t)L.n + 1);
     L.pw = h.arena.get<VT>((size_t)L.n + 1);
+    L.pwm = h.arena.get<VT>((size_t)L.n + 1);
   }
   klaunch(k_convert_row_data<VT>, ew_grid(L.n), kThreads, s, L.n, diag, L.omega, (const double *)L.omega_dev,
-          L.pw64, (VT *)L.wd, (VT *)L.dinv, (VT *)L.pw);
+          L.pw64, (VT *)L.wd, (VT *)L.dinv, (VT *)L.pw, (const int32_t *)L.amem, (VT *)L.pwm);
   AMG_LAUNCH_CHECK();
 }
 
@@ -2154,10 +2369,12 @@ void autotune_t(Hierarchy &h, cudaStream_t s) {
       DevBuf<VT> x((size_t)L.n + 1), y((size_t)L.n + 1);
       AMG_CUDA(cudaMemsetAsync(x.p, 0, sizeof(VT) * (L.n + 1), s));
       // the plain product at each grid; launches with fused inner products take
-      // the best grid within the partial-sum capacity
+      // the best grid within the partial-sum capacity.  The split-row kernel of
+      // the small levels covers its slices in one pass and has no grid to choose.
       const int gfull = full_plain_grid(L);
       std::vector<std::pair<int, float>> t, tr;
-      for (int g : {152, 304, 608, 912, 1216, 2432, 4864, 1 << 30}) {
+      if (L.split_log >= 0) tr = t = {{L.sell_blocks, 0.f}};
+      else for (int g : {152, 304, 608, 912, 1216, 2432, 4864, 1 << 30}) {
         const int gg = std::min(g, gfull);
         if (!t.empty() && t.back().first == gg) continue;
         L.sell_plain_blocks = gg;
