@@ -178,6 +178,17 @@ struct Level {
   // one 16-byte load; slice widths are even.
   int4 *spair = nullptr;
   float *sdiag = nullptr;
+  // A_k P_k with the solve-phase matrix, SELL-32 without the entry of the row's own
+  // aggregate, which is in ap_own: the post-smoothing step takes the residual after
+  // the coarse correction as r - (A P) x_{k+1}, so that it reads neither A_k nor the
+  // corrected iterate of the neighbours.  Entries as {column, value} pairs with FP32
+  // vectors (layout of spair), as ap_col / ap_val with FP64.
+  int64_t *ap_ptr = nullptr;
+  int64_t ap_entries = 0;
+  int4 *ap_pair = nullptr;
+  int32_t *ap_col = nullptr;
+  double *ap_val = nullptr;
+  void *ap_own = nullptr;
   // level 0 only: every entry in FP64 for the outer Krylov method and the true
   // residual (the same arrays as sptr / scol / sval in FP64 mode)
   int64_t *sptr64 = nullptr;

@@ -582,6 +582,17 @@ int amg_validate_hierarchy(const amg_hierarchy *H) {
         expect(L.nc == h.lev[k + 1].n, k, "coarse size");
         for (int32_t a : agg) expect(a >= 0 && a < L.nc, k, "aggregate id out of range");
         expect(ap[0] == 0 && ap[L.nc] == L.n, k, "member pointer ends");
+        auto pp = fetch(L.ap_ptr, (size_t)L.nslices + 1);
+        expect(pp[0] == 0 && pp[L.nslices] == L.ap_entries, k, "A P pointer ends");
+        for (int32_t q = 0; q < L.nslices; ++q)
+          expect(pp[q] <= pp[q + 1] && (pp[q + 1] - pp[q]) % unit == 0, k, "A P slice");
+        if (L.ap_pair) {
+          auto pw = fetch(reinterpret_cast<const int32_t *>(L.ap_pair), 2 * (size_t)L.ap_entries);
+          for (size_t q = 0; q < pw.size(); q += 2) expect(pw[q] >= 0 && pw[q] < L.nc, k, "A P column out of range");
+        } else {
+          for (int32_t c : fetch(L.ap_col, (size_t)L.ap_entries))
+            expect(c >= 0 && c < L.nc, k, "A P column out of range");
+        }
         std::vector<char> seen(L.n, 0);
         for (int32_t I = 0; I < L.nc; ++I)
           for (int32_t m = ap[I]; m < ap[I + 1]; ++m) {

@@ -955,6 +955,161 @@ __global__ void k_build_sell(int32_t n, int32_t nslices, const int32_t *__restri
   if (sdiag && row < n) sdiag[row] = __double2float_rn(__dadd_rn(dii, comp));
 }
 
+// ---- A P of a level, from its solve-phase matrix ------------------------------
+// entry e of the lane's row in the SELL layout of the value type
+template <class MV>
+struct SellRow {
+  const int32_t *__restrict__ scol;
+  const void *sval;
+  const int4 *__restrict__ spair;
+  int64_t base;
+  int lane;
+  __device__ __forceinline__ int64_t at(int32_t e) const {
+    return std::is_same<MV, __nv_bfloat16>::value ? base + (int64_t)(e >> 1) * (2 * kSlice) + 2 * lane + (e & 1)
+                                                  : base + (int64_t)e * kSlice + lane;
+  }
+  __device__ __forceinline__ const int2 *pair(int32_t e) const {
+    return reinterpret_cast<const int2 *>(spair + (base >> 1) + (int64_t)(e >> 1) * kSlice + lane) + (e & 1);
+  }
+  __device__ __forceinline__ int32_t col(int32_t e) const {
+    if constexpr (std::is_same<MV, float>::value) return pair(e)->x;
+    else return scol[at(e)];
+  }
+  __device__ __forceinline__ auto val(int32_t e) const {
+    if constexpr (std::is_same<MV, float>::value) return __int_as_float(pair(e)->y);
+    else if constexpr (std::is_same<MV, __nv_bfloat16>::value)
+      return __bfloat162float(static_cast<const __nv_bfloat16 *>(sval)[at(e)]);
+    else return static_cast<const double *>(sval)[at(e)];
+  }
+};
+
+// The aggregates J != own of the row's neighbours, once each in order of first
+// occurrence: f(e, same) for the first entry e of each, same(q) telling whether
+// entry q > e belongs to it.  Up to K entries with their aggregates in registers.
+template <int K, class Row, class F>
+__device__ __forceinline__ void ap_row_regs(const Row &r, int32_t width, int32_t own, const int32_t *__restrict__ agg,
+                                            F &&f) {
+  int32_t J[K];
+#pragma unroll
+  for (int e = 0; e < K; ++e) J[e] = e < width ? agg[r.col(e)] : own;
+#pragma unroll
+  for (int e = 0; e < K; ++e) {
+    bool first = J[e] != own;
+#pragma unroll
+    for (int q = 0; q < e; ++q) first = first && J[q] != J[e];
+    if (first) {
+      unsigned mask = 0;  // the entries of this aggregate
+#pragma unroll
+      for (int q = e; q < K; ++q) mask |= J[q] == J[e] ? 1u << q : 0u;
+      f(J[e], mask);
+    }
+  }
+}
+
+// entries of A P per row without the row's own aggregate; slice width = the longest
+// row's, rounded up to even for the pair layout
+template <class MV>
+__global__ void k_ap_width(int32_t n, int32_t nslices, const int64_t *__restrict__ sptr,
+                           const int32_t *__restrict__ scol, const int4 *__restrict__ spair,
+                           const int32_t *__restrict__ agg, bool pairs, int64_t *__restrict__ width32) {
+  pdl_wait_and_trigger();
+  const int lane = threadIdx.x & 31;
+  const int32_t sl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (sl >= nslices) return;
+  const int32_t row = sl * kSlice + lane;
+  const SellRow<MV> r{scol, nullptr, spair, sptr[sl], lane};
+  const int32_t width = (int32_t)((sptr[sl + 1] - r.base) / kSlice);
+  int32_t cnt = 0;
+  if (row < n) {
+    const int32_t own = agg[row];
+    auto count = [&](int32_t, unsigned) { ++cnt; };
+    if (width <= 8) {
+      ap_row_regs<8>(r, width, own, agg, count);
+    } else if (width <= 24) {
+      ap_row_regs<24>(r, width, own, agg, count);
+    } else {
+      for (int32_t e = 0; e < width; ++e) {
+        const int32_t J = agg[r.col(e)];
+        bool first = J != own;
+        for (int32_t q = 0; first && q < e; ++q) first = agg[r.col(q)] != J;
+        cnt += first ? 1 : 0;
+      }
+    }
+  }
+  cnt = __reduce_max_sync(0xffffffffu, cnt);
+  if (pairs) cnt = (cnt + 1) & ~1;
+  if (lane == 0) width32[sl] = (int64_t)cnt * kSlice;
+}
+
+// the entries sum_{j in J} a_ij P_j in the vector type, a_ij as the solve-phase
+// matrix holds them (rounded values, compensated diagonal), so that the residual
+// update is that of the same operator
+template <class MV, class VT>
+__global__ void k_ap_fill(int32_t n, int32_t nslices, const int64_t *__restrict__ sptr,
+                          const int32_t *__restrict__ scol, const MV *__restrict__ sval,
+                          const int4 *__restrict__ spair, const float *__restrict__ sdiag,
+                          const int32_t *__restrict__ agg, const VT *__restrict__ pw,
+                          const int64_t *__restrict__ apptr, int4 *__restrict__ appair, int32_t *__restrict__ apcol,
+                          double *__restrict__ apval, VT *__restrict__ apown) {
+  pdl_wait_and_trigger();
+  const int lane = threadIdx.x & 31;
+  const int32_t sl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (sl >= nslices) return;
+  const int32_t row = sl * kSlice + lane;
+  const SellRow<MV> r{scol, sval, spair, sptr[sl], lane};
+  const int32_t width = (int32_t)((sptr[sl + 1] - r.base) / kSlice);
+  const int64_t base = apptr[sl];
+  const int32_t apw = (int32_t)((apptr[sl + 1] - base) / kSlice);
+  const int32_t own = agg[row < n ? row : n - 1];
+  int32_t cnt = 0;
+  auto put = [&](int32_t c, VT v) {
+    if constexpr (std::is_same<VT, float>::value) {
+      int2 *w = reinterpret_cast<int2 *>(appair + (base >> 1) + (int64_t)(cnt >> 1) * kSlice + lane) + (cnt & 1);
+      *w = make_int2(c, __float_as_int(v));
+    } else {
+      apcol[base + (int64_t)cnt * kSlice + lane] = c;
+      apval[base + (int64_t)cnt * kSlice + lane] = v;
+    }
+    ++cnt;
+  };
+  if (row < n) {
+    VT o = VT(0);
+    if (sdiag) o = (VT)sdiag[row] * pw[row];
+    for (int32_t e = 0; e < width; ++e) {
+      const int32_t c = r.col(e);
+      if (agg[c] == own) o += (VT)r.val(e) * pw[c];
+    }
+    apown[row] = o;
+    auto add = [&](int32_t J, unsigned mask) {
+      VT s = VT(0);
+      for (; mask; mask &= mask - 1) {
+        const int32_t e = __ffs(mask) - 1;
+        s += (VT)r.val(e) * pw[r.col(e)];
+      }
+      put(J, s);
+    };
+    if (width <= 8) {
+      ap_row_regs<8>(r, width, own, agg, add);
+    } else if (width <= 24) {
+      ap_row_regs<24>(r, width, own, agg, add);
+    } else {
+      for (int32_t e = 0; e < width; ++e) {
+        const int32_t J = agg[r.col(e)];
+        bool first = J != own;
+        for (int32_t q = 0; first && q < e; ++q) first = agg[r.col(q)] != J;
+        if (!first) continue;
+        VT s = VT(0);
+        for (int32_t q = e; q < width; ++q) {
+          const int32_t c = r.col(q);
+          if (agg[c] == J) s += (VT)r.val(q) * pw[c];
+        }
+        put(J, s);
+      }
+    }
+  }
+  while (cnt < apw) put(own, VT(0));
+}
+
 // ============================================================== Arnoldi omega
 // ---- Arnoldi on M = |D|^-1/2 A |D|^-1/2 with three kernels per step --------
 // Every kernel ends with a last-block reduction: blocks publish their partial
@@ -2083,6 +2238,50 @@ void build_solve_matrix(Hierarchy &h, Level &L, cudaStream_t s, bool fresh) {
   }
 }
 
+// A P of level q (not the coarsest).  widths: slice widths and their scan, the
+// entry count on its way to the pinned word of the level (read at the caller's
+// next synchronisation); fill: the entries
+template <class MV, class VT>
+void ap_widths_t(Hierarchy &h, int q, cudaStream_t s) {
+  Level &L = h.lev[q];
+  DevBuf<int64_t> w32(L.nslices + 1);
+  AMG_COUNT(), klaunch_sm(k_ap_width<MV>, blocks_for((int64_t)L.nslices * 32), 256, 0, s, L.n, L.nslices, L.sptr, L.scol,
+                          L.spair, L.agg, std::is_same<VT, float>::value, w32.p);
+  AMG_LAUNCH_CHECK();
+  L.ap_ptr = h.arena.get<int64_t>(L.nslices + 1);
+  exclusive_scan<int64_t, int64_t>(w32.p, L.ap_ptr, L.nslices, s);
+  AMG_CUDA(cudaMemcpyAsync(reinterpret_cast<int64_t *>(h.host_pinned + kPinnedSellEntries) + q, L.ap_ptr + L.nslices,
+                           sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+}
+template <class MV, class VT>
+void ap_fill_t(Hierarchy &h, int q, cudaStream_t s, bool fresh) {
+  Level &L = h.lev[q];
+  if (fresh) {
+    L.ap_entries = reinterpret_cast<const int64_t *>(h.host_pinned + kPinnedSellEntries)[q];
+    L.ap_own = h.arena.get<VT>((size_t)L.n + 1);
+    if (std::is_same<VT, float>::value) {
+      L.ap_pair = h.arena.get<int4>(L.ap_entries / 2);
+    } else {
+      L.ap_col = h.arena.get<int32_t>(L.ap_entries);
+      L.ap_val = h.arena.get<double>(L.ap_entries);
+    }
+  }
+  AMG_COUNT(), klaunch_sm(k_ap_fill<MV, VT>, blocks_for((int64_t)L.nslices * 32), 256, 0, s, L.n, L.nslices, L.sptr,
+                          L.scol, (const MV *)L.sval, L.spair, L.sdiag, L.agg, (const VT *)L.pw, L.ap_ptr, L.ap_pair,
+                          L.ap_col, L.ap_val, (VT *)L.ap_own);
+  AMG_LAUNCH_CHECK();
+}
+void ap_widths(Hierarchy &h, int q, cudaStream_t s) {
+  if (h.p.precision == AMG_PREC_F64) ap_widths_t<double, double>(h, q, s);
+  else if (h.p.precision == AMG_PREC_F32) ap_widths_t<float, float>(h, q, s);
+  else ap_widths_t<__nv_bfloat16, float>(h, q, s);
+}
+void ap_fill(Hierarchy &h, int q, cudaStream_t s, bool fresh) {
+  if (h.p.precision == AMG_PREC_F64) ap_fill_t<double, double>(h, q, s, fresh);
+  else if (h.p.precision == AMG_PREC_F32) ap_fill_t<float, float>(h, q, s, fresh);
+  else ap_fill_t<__nv_bfloat16, float>(h, q, s, fresh);
+}
+
 // m = 5 Arnoldi steps on D^-1/2 A D^-1/2 for omega of Eq. (damped Jacobi):
 // three kernels per step; the Hessenberg matrix goes to H (9 x 8) and the
 // norms ||M q_j|| to wn (8), for k_omega_from_H.  Returns m.
@@ -2383,6 +2582,8 @@ void finish_levels(Hierarchy &h, cudaStream_t s, bool fresh) {
     AMG_LAUNCH_CHECK();
   }
   for (int q = 0; q < h.L; ++q) make_row_data(h, h.lev[q], diag[q].p, s);  // per-row smoother data
+  if (fresh)
+    for (int q = 0; q + 1 < h.L; ++q) ap_widths(h, q, s);
   {  // the estimated weights back to the host, one synchronisation for all levels
     for (int q = 0; q < h.L - 1; ++q)
       if (h.lev[q].omega_dev)
@@ -2391,6 +2592,7 @@ void finish_levels(Hierarchy &h, cudaStream_t s, bool fresh) {
     for (int q = 0; q < h.L - 1; ++q)
       if (h.lev[q].omega_dev) h.lev[q].omega = h.host_pinned[q];
   }
+  for (int q = 0; q + 1 < h.L; ++q) ap_fill(h, q, s, fresh);
 
   // ---- coarsest level: dense factorisation and inverse
   Level &Lc = h.lev[h.L - 1];

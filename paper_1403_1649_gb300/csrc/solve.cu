@@ -48,9 +48,8 @@ struct SellArgs {
   const unsigned char *live;  // batch: 0 for slices whose systems all stopped (skipped); else null
   const VT *x;    // SpMV input
   VT *out;        // output vector
-  const VT *rhs;  // right-hand side (residual / smoothing epilogues)
-  const VT *wd;   // omega / A_ii
-  const VT *xin;  // the iterate that the post-smoothing step updates
+  const VT *rhs;  // right-hand side (residual epilogues)
+  const VT *xin;  // the iterate that the last Horner step updates
   // fused inner products with left operand s = x (dot_y: the output): ND = 2:
   // {s.out, s.u1}, ND = 3: {s.out, s.u1, s.u2}, ND = 1: {out.q64}; then fin
   const VT *u1, *u2;
@@ -69,13 +68,12 @@ struct SellArgs {
 // epilogues of the SELL kernel (y = A x):
 //   E_Y            out = y
 //   E_RESID        out = rhs - y
-//   E_POST         out = xin + wd (rhs - y)                  damped Jacobi after prolongation
 //   E_DSCALE       out = D^-1 y                               polynomial pre-smoother, term 1
 //   E_POLYPRE      out = c0 p0 + c1 p1 + c2 D^-1 y            polynomial pre-smoother, sum
 //   E_RESID_POLY   out = rhs - y, out2 = D^-1 (c2 out)        post-smoother: residual, Horner start
 //   E_HORNER       out = D^-1 y + D^-1 (c1 res)               Horner middle step
 //   E_HORNER_LAST  out = xin + D^-1 y + D^-1 (c0 res)         Horner last step, update
-enum Epi { E_Y = 0, E_RESID = 1, E_POST = 2, E_DSCALE = 3, E_POLYPRE = 4, E_RESID_POLY = 5, E_HORNER = 6,
+enum Epi { E_Y = 0, E_RESID = 1, E_DSCALE = 3, E_POLYPRE = 4, E_RESID_POLY = 5, E_HORNER = 6,
            E_HORNER_LAST = 7 };
 
 template <class MV> __device__ __forceinline__ MV ld_stream(const MV *p) { return __ldcs(p); }
@@ -248,7 +246,6 @@ __device__ __forceinline__ void sell_epilogue(const SellArgs<VT> &a, int32_t row
   VT o;
   if (EPI == E_Y) o = y;
   else if (EPI == E_RESID) o = a.rhs[row] - y;
-  else if (EPI == E_POST) o = a.xin[row] + a.wd[row] * (a.rhs[row] - y);
   else if (EPI == E_DSCALE) o = a.dinv[row] * y;
   else if (EPI == E_POLYPRE)
     o = a.coef[3 * row] * a.p0[row] + a.coef[3 * row + 1] * a.p1[row] + a.coef[3 * row + 2] * (a.dinv[row] * y);
@@ -610,6 +607,118 @@ __global__ void k_prolong(int32_t n, const int32_t *__restrict__ agg, const VT *
     }
     if (!bact || bact[sys[i]]) x[i] += p * xc[g];
   }
+}
+
+// Post-smoothing after the coarse correction (Alg. 4/5): with x the iterate and r
+// its residual before the correction,
+//   out = x + P x_{k+1} + wd (r - (A P) x_{k+1}).
+// A P has one entry per neighbouring aggregate (3-6 off the row's own, for 6-25 in
+// a row of A) and gathers from the small vector x_{k+1}; the prolongation needs no
+// launch of its own and A is not read again.
+template <class VT>
+struct PostArgs {
+  int32_t n, nslices;
+  const int64_t *ptr;
+  const int4 *pair;    // FP32 vectors
+  const int32_t *col;  // FP64 vectors
+  const double *val;
+  const VT *own, *pw, *wd;
+  const int32_t *agg;
+  const unsigned char *live;  // batch
+  const VT *x, *r, *xc;
+  VT *out;
+  const double *q64;  // ND = 1: out . q64
+  FinArgs fin;
+  const int *pred;
+};
+
+template <class VT>
+constexpr int post_blocks() { return sizeof(VT) == 4 ? 3 : 2; }  // resident blocks per SM
+
+template <class VT, int ND, bool GATE>
+__global__ void __launch_bounds__(kThreads, post_blocks<VT>()) k_post(PostArgs<VT> a) {
+  pdl_trigger();
+  const int lane = threadIdx.x & 31;
+  double acc[ND ? ND : 1] = {0.0};
+  bool first = true, run = true;
+  constexpr int U = 8;
+  for (int32_t sl = blockIdx.x * kWarps + (threadIdx.x >> 5); sl < a.nslices; sl += gridDim.x * kWarps) {
+    if (GATE && !first && !a.live[sl]) continue;
+    const int32_t row = sl * 32 + lane;
+    const int32_t rr = min(row, a.n - 1);
+    const int64_t base = a.ptr[sl];
+    const int32_t width = (int32_t)((a.ptr[sl + 1] - base) >> 5);
+    const int32_t g = __ldcs(a.agg + rr);
+    const VT own = __ldcs(a.own + rr), p = __ldcs(a.pw + rr), w = __ldcs(a.wd + rr);
+    VT y = VT(0);
+    auto step = [&](int32_t e, auto size, auto full, auto &&between) {
+      constexpr int S = decltype(size)::value;
+      constexpr bool FULL = decltype(full)::value;
+      int32_t c[S];
+      VT v[S];
+      if constexpr (sizeof(VT) == 4) {
+        const int4 *__restrict__ pp = a.pair + (base >> 1) + lane;
+#pragma unroll
+        for (int q = 0; q < S; q += 2)
+          if (FULL || e + q < width) {
+            const int4 p4 = ld_stream(pp + 16 * (e + q));
+            c[q] = p4.x;
+            v[q] = __int_as_float(p4.y);
+            c[q + 1] = p4.z;
+            v[q + 1] = __int_as_float(p4.w);
+          }
+      } else {
+#pragma unroll
+        for (int q = 0; q < S; ++q)
+          if (FULL || e + q < width) {
+            c[q] = ld_stream(a.col + base + 32 * (int64_t)(e + q) + lane);
+            v[q] = ld_stream(a.val + base + 32 * (int64_t)(e + q) + lane);
+          }
+      }
+      between();
+      VT xv[S];
+#pragma unroll
+      for (int q = 0; q < S; ++q)
+        if (FULL || e + q < width) xv[q] = a.xc[c[q]];
+#pragma unroll
+      for (int q = 0; q < S; ++q)
+        if (FULL || e + q < width) y += v[q] * xv[q];
+    };
+    bool live = true;
+    VT xg = VT(0), ri = VT(0), xi = VT(0);
+    auto enter = [&] {  // wait (first slice), then the row's own operands
+      if (first) {
+        first = false;
+        pdl_wait();
+        run = !(a.pred && *a.pred == 0);
+        if (GATE) live = a.live[sl];
+      }
+      xg = a.xc[g];
+      ri = a.r[rr];
+      xi = a.x[rr];
+    };
+    using S4 = std::integral_constant<int, 4>;
+    using S6 = std::integral_constant<int, 6>;
+    using SU = std::integral_constant<int, U>;
+    if (width == 4) step(0, S4{}, std::true_type{}, enter);
+    else if (width == 6) step(0, S6{}, std::true_type{}, enter);
+    else {
+      step(0, SU{}, std::false_type{}, enter);
+      for (int32_t e = U; e < width; e += U) step(e, SU{}, std::false_type{}, [] {});
+    }
+    if (!run) return;  // the same in every thread of the grid
+    if (GATE && !live) continue;
+    if (row < a.n) {
+      const VT o = (xi + p * xg) + w * (ri - (own * xg + y));
+      a.out[row] = o;
+      if constexpr (ND == 1) acc[0] += (double)o * a.q64[row];
+    }
+  }
+  if (first) {  // a warp without a slice
+    pdl_wait();
+    if (a.pred && *a.pred == 0) return;
+  }
+  if constexpr (ND > 0) grid_dots<ND>(acc, 1, a.fin);
 }
 
 // exact coarsest solve x = A_L^-1 b (one warp per row, FP64 accumulation)
@@ -1397,7 +1506,7 @@ struct Engine {
     const Level &L = h.lev[k];
     if (h.batched && ND)  // inner products of a batch are per system (segdot)
       throw Error{AMG_ERR_UNSUPPORTED, "batched SpMV was given fused inner products"};
-    if constexpr (EPI == E_Y || EPI == E_RESID || EPI == E_POST)
+    if constexpr (EPI == E_Y || EPI == E_RESID)
       if (L.split_log >= 0) {
         const int grid = grid_for(L.nslices, kWarps >> L.split_log, kRedBlocks);
         if (h.batched)
@@ -1486,42 +1595,63 @@ struct Engine {
     } else {
       cycle(k + 1, V(C.bc), V(C.xc), true, pred);  // Alg. 4 recursion
     }
+    if (!poly) {  // x_k += P_k x_{k+1}, then the post-smoothing step on the updated residual
+      PostArgs<VT> a{};
+      a.n = L.n;
+      a.nslices = L.nslices;
+      a.ptr = L.ap_ptr;
+      a.pair = L.ap_pair;
+      a.col = L.ap_col;
+      a.val = L.ap_val;
+      a.own = V(L.ap_own);
+      a.pw = V(L.pw);
+      a.wd = V(L.wd);
+      a.agg = L.agg;
+      a.x = tmp;
+      a.r = V(L.r);
+      a.xc = V(C.xc);
+      a.out = out;
+      a.pred = pred;
+      const int grid = grid_for(L.nslices, kWarps, post_blocks<VT>() * 152);
+      if (h.batched) {
+        a.live = L.slive;
+        klaunch(k_post<VT, 0, true>, grid, kThreads, s, a);
+      } else if (k == 0 && zq_fuse) {  // z^T q and beta of the outer flexible CG
+        a.q64 = h.q;
+        a.fin = fin_args(0, FIN_BETA, L.partials);
+        klaunch(k_post<VT, 1, false>, grid, kThreads, s, a);
+      } else {
+        klaunch(k_post<VT, 0, false>, grid, kThreads, s, a);
+      }
+      check();
+      return;
+    }
     // x_k += P_k x_{k+1}
     klaunch(k_prolong<VT>, ew_grid(L.n), kThreads, s, L.n, L.agg, V(L.pw), V(C.xc), tmp, pred, bsys(L), bact());
     check();
-    // r_k = b_k - A_k x_k;  x_k += omega D^-1 r_k  (or the transposed polynomial)
-    SellArgs<VT> a = sell_args(k, tmp, out, pred);
-    a.rhs = rhs;
-    a.wd = V(L.wd);
+    // r_k = b_k - A_k x_k, then the transposed polynomial in Horner form
+    SellArgs<VT> b = sell_args(k, tmp, V(L.r), pred);
+    b.rhs = rhs;
+    b.dinv = V(L.dinv);
+    b.coef = V(L.poly);
+    b.out2 = V(L.u0);
+    sell<E_RESID_POLY>(b, k);
+    b = sell_args(k, V(L.u0), V(L.u1), pred);
+    b.dinv = V(L.dinv);
+    b.coef = V(L.poly);
+    b.res = V(L.r);
+    sell<E_HORNER>(b, k);
+    SellArgs<VT> a = sell_args(k, V(L.u1), out, pred);
     a.xin = tmp;
-    if (poly) {
-      SellArgs<VT> b = sell_args(k, tmp, V(L.r), pred);
-      b.rhs = rhs;
-      b.dinv = V(L.dinv);
-      b.coef = V(L.poly);
-      b.out2 = V(L.u0);
-      sell<E_RESID_POLY>(b, k);
-      b = sell_args(k, V(L.u0), V(L.u1), pred);
-      b.dinv = V(L.dinv);
-      b.coef = V(L.poly);
-      b.res = V(L.r);
-      sell<E_HORNER>(b, k);
-      a.x = V(L.u1);
-      a.dinv = V(L.dinv);
-      a.coef = V(L.poly);
-      a.res = V(L.r);
-    }
-    if (k == 0 && zq_fuse) {  // z^T q and beta of the outer flexible CG
+    a.dinv = V(L.dinv);
+    a.coef = V(L.poly);
+    a.res = V(L.r);
+    if (k == 0 && zq_fuse) {
       a.q64 = h.q;
       a.fin = fin_args(0, FIN_BETA, L.partials);
-      if (poly)
-        sell<E_HORNER_LAST, 1>(a, k);
-      else
-        sell<E_POST, 1>(a, k);
-    } else if (poly) {
-      sell<E_HORNER_LAST>(a, k);
+      sell<E_HORNER_LAST, 1>(a, k);
     } else {
-      sell<E_POST>(a, k);
+      sell<E_HORNER_LAST>(a, k);
     }
   }
   bool zq_fuse = false;
