@@ -246,10 +246,10 @@ int amg_mlp_backward(int32_t n, const float *w, const float *feat, const float *
  * their steady state, and hosts that have handed the whole device memory
  * budget to another framework.  The paper has no counterpart; this is a
  * service of the library.
- *  - No cudaMalloc, cudaFree or allocating library call: the work arrays live
- *    in a fixed device array of about 4.2 MB (2048 rows x (3 + 4 x 64) floats
- *    plus 64 x 4096 doubles) that every GPU loading this library keeps until
- *    the process exits.
+ *  - No cudaMalloc, cudaFree or allocating library call: the work array lives
+ *    in a fixed device array of about 1.4 MB (the weight-gradient sums of 32
+ *    tiles of 64 rows) that every GPU loading this library keeps until the
+ *    process exits.
  *  - n may be at most 2048; larger n returns AMG_ERR_BAD_INPUT with a message.
  *  - Each call looks up that array's device address on the current device
  *    (no allocation); the first call on a device also loads the module that

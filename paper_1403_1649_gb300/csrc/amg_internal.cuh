@@ -315,8 +315,7 @@ void twogrid_loss(Hierarchy &h, const double *coef, int nvec, uint64_t seed, dou
                   cudaStream_t s);
 void features(const Hierarchy &h, int level, float *feat_dev, cudaStream_t s);
 void mlp_forward_half(int32_t n, const uint16_t *w16_dev, const float *feat, float *out, cudaStream_t s);
-void mlp_backward(int32_t n, const float *w, const float *feat, const float *dout, double *dparam, cudaStream_t s,
-                  bool zero);
+void mlp_backward(int32_t n, const float *w, const float *feat, const float *dout, double *dparam, cudaStream_t s);
 void apply_learned(Hierarchy &h, const uint16_t *w16_dev, cudaStream_t s);
 void train_smoother(Hierarchy *const *hs, int nh, int steps, double lr, int nvec, uint64_t seed, float *w_host,
                     double *loss_hist, cudaStream_t s);

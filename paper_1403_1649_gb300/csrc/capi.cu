@@ -447,7 +447,7 @@ int amg_mlp_backward(int32_t n, const float *w, const float *feat, const float *
   if (n < 0 || !w || !feat || !dout || !dparam) return AMG_ERR_BAD_INPUT;
   return guarded([&]() {
     amg::current_stream() = (cudaStream_t)stream;
-    amg::mlp_backward(n, w, feat, dout, dparam, (cudaStream_t)stream, true);
+    amg::mlp_backward(n, w, feat, dout, dparam, (cudaStream_t)stream);
     return AMG_OK;
   });
 }
