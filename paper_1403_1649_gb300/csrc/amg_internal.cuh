@@ -211,8 +211,10 @@ struct Level {
   std::vector<int32_t> sys_off_host;
   int32_t ntiles = 0;
   int32_t *tile_row = nullptr, *sys_tile = nullptr;  // ntiles+1 row starts; nsys+1 first tiles
+  int32_t *tile_sys = nullptr;                       // system of each tile
   double *bslots = nullptr;   // kNumSlots x nsys per-system scalars
   int *bflag = nullptr;       // nsys second-step flags, then "any"
+  int *bticket = nullptr;     // per system: tiles finished by the running launch
   double *tpart = nullptr;    // 3 x ntiles tile partial sums
 };
 

@@ -211,17 +211,26 @@ __device__ __forceinline__ void block_store_dot(double a, double *partials) {
 // batch: live[sl] = 1 when some system with rows in slice sl still iterates.
 // Rows of a stopped system are only ever read by that system, so its work can
 // be skipped; a restarted system starts again from its recomputed residual.
-__global__ void k_slice_live(int32_t n, int32_t nslices, const int32_t *__restrict__ sys,
-                             const int *__restrict__ bact, unsigned char *__restrict__ live) {
-  pdl_wait_and_trigger();
-  for (int32_t sl = blockIdx.x * blockDim.x + threadIdx.x; sl < nslices; sl += gridDim.x * blockDim.x) {
+// blockIdx.y is the level.
+struct LiveArgs {
+  int32_t n[kMaxLevels], nslices[kMaxLevels];
+  const int32_t *sys[kMaxLevels];
+  unsigned char *live[kMaxLevels];
+};
+__global__ void k_slice_live(const __grid_constant__ LiveArgs a, const int *bact) {
+  pdl_trigger();
+  pdl_wait();
+  const int k = blockIdx.y;
+  const int32_t n = a.n[k];
+  const int32_t *__restrict__ sys = a.sys[k];
+  for (int32_t sl = blockIdx.x * blockDim.x + threadIdx.x; sl < a.nslices[k]; sl += gridDim.x * blockDim.x) {
     unsigned char v = 0;
     for (int32_t q = sys[sl * 32]; q <= sys[min(sl * 32 + 31, n - 1)]; ++q)
       if (bact[q]) {
         v = 1;
         break;
       }
-    live[sl] = v;
+    a.live[k][sl] = v;
   }
 }
 
@@ -1174,55 +1183,6 @@ __global__ void k_sys_of(int32_t n, int32_t nsys, const int32_t *__restrict__ of
   }
 }
 
-// tile partials of up to three inner products a_d . b_d (nullptr b: a . a)
-template <class VT>
-__global__ void k_segdot(int32_t ntiles, const int32_t *__restrict__ tile_row, int ndot, const VT *a0,
-                         const VT *b0, const VT *a1, const VT *b1, const VT *a2, const VT *b2,
-                         double *__restrict__ tpart, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  for (int32_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    for (int32_t i = tile_row[t] + threadIdx.x; i < tile_row[t + 1]; i += blockDim.x) {
-      s0 += (double)a0[i] * (double)b0[i];
-      if (ndot > 1) s1 += (double)a1[i] * (double)b1[i];
-      if (ndot > 2) s2 += (double)a2[i] * (double)b2[i];
-    }
-    __shared__ double sh[3][kWarps];
-    s0 = warp_sum(s0);
-    s1 = warp_sum(s1);
-    s2 = warp_sum(s2);
-    if ((threadIdx.x & 31) == 0) {
-      sh[0][threadIdx.x >> 5] = s0;
-      sh[1][threadIdx.x >> 5] = s1;
-      sh[2][threadIdx.x >> 5] = s2;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-      double v = 0.0;
-      for (int w = 0; w < kWarps; ++w) v += sh[threadIdx.x][w];
-      if ((int)threadIdx.x < ndot) tpart[(int64_t)threadIdx.x * ntiles + t] = v;
-    }
-    __syncthreads();
-  }
-}
-
-// dot d of system s = sum of its tiles' partials; out[(slot0 + d) * nsys + s]
-__global__ void k_segfin(int32_t nsys, int32_t ntiles, const int32_t *__restrict__ sys_tile, int ndot,
-                         const double *__restrict__ tpart, double *__restrict__ bslots, int slot0, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  const int lane = threadIdx.x & 31;
-  for (int32_t s = blockIdx.x * kWarps + (threadIdx.x >> 5); s < nsys; s += gridDim.x * kWarps) {
-    for (int d = 0; d < ndot; ++d) {
-      double v = 0.0;
-      for (int32_t t = sys_tile[s] + lane; t < sys_tile[s + 1]; t += 32) v += tpart[(int64_t)d * ntiles + t];
-      v = warp_sum(v);
-      if (lane == 0) bslots[(int64_t)(slot0 + d) * nsys + s] = v;
-    }
-  }
-}
-
 #define BS(slot, s) bslots[(int64_t)(slot)*nsys + (s)]
 
 // per-system status of a batch while it runs: kIterating, kUpdatedConverged
@@ -1231,63 +1191,168 @@ __global__ void k_segfin(int32_t nsys, int32_t ntiles, const int32_t *__restrict
 constexpr int kIterating = 2;
 constexpr int kUpdatedConverged = 1;
 
-// Alg. 5 per system: s1 = alpha_1 / rho_1 (dots in S_RHO1, S_A1)
-__global__ void k_bfin_k1(int32_t nsys, double *__restrict__ bslots, const int *pred) {
-  pdl_wait_and_trigger();
+// Per-system inner products and the scalars they lead to, in one launch: a block
+// takes a row tile of one system, and the block that finishes a system's last tile
+// sums the system's tiles in tile order and takes its scalar step.  Tiles of stopped
+// systems are skipped (bact; null: all systems).  As separate launches the sums over
+// tiles and the scalar steps were 21 of a pass's ~100 kernels.
+enum BFin { BF_STORE = 0, BF_K1 = 1, BF_DECIDE = 2, BF_K3 = 3, BF_BETA = 4, BF_ALPHA = 5 };
+
+struct SegArgs {
+  int32_t ntiles, nsys;
+  const int32_t *tile_row, *tile_sys, *sys_tile;
+  const int *bact;
+  double *tpart;  // 3 x ntiles
+  int *ticket;    // nsys, 0 between launches
+  double *bslots;
+  int kind, slot0;  // BF_STORE: totals to slots slot0, slot0 + 1, ...
+  int *flag;        // BF_K1 clears, BF_DECIDE sets the level's second-step flags (flag[nsys]: any)
+  double t;         // BF_DECIDE
+  const int *brs;   // BF_BETA: restart flags
+};
+
+constexpr int kSegThreads = 512;
+
+__device__ __forceinline__ void run_bfin(const SegArgs &g, int32_t s, int nd, const double *tot) {
+  double *bslots = g.bslots;
+  const int32_t nsys = g.nsys;
+  switch (g.kind) {
+    case BF_STORE:
+      for (int d = 0; d < nd; ++d) BS(g.slot0 + d, s) = tot[d];
+      break;
+    case BF_K1:  // Alg. 5 after v = A c: c^T v, c^T r
+      BS(S_RHO1, s) = tot[0];
+      BS(S_A1, s) = tot[1];
+      BS(S_S1, s) = tot[1] / tot[0];
+      break;
+    case BF_DECIDE: {  // ||r~|| > t ||r|| (squared): this system needs the second inner step
+      const bool second = !(tot[0] <= g.t * g.t * tot[1]);
+      g.flag[s] = second ? 1 : 0;
+      if (second) g.flag[nsys] = 1;
+      break;
+    }
+    case BF_K3: {  // after w = A d: gamma = d^T v, beta = d^T w, alpha_2 = d^T r~
+      const double gam = tot[0], g1 = gam / BS(S_RHO1, s), cd = tot[2] / (tot[1] - gam * g1);
+      BS(S_CC, s) = BS(S_S1, s) - g1 * cd;
+      BS(S_CD, s) = cd;
+      break;
+    }
+    case BF_BETA:  // outer flexible CG: z^T q_old
+      BS(S_ZQ, s) = tot[0];
+      BS(S_BETA, s) = g.brs[s] ? 0.0 : -tot[0] / BS(S_PQ, s);
+      break;
+    default:  // p^T q, p^T r
+      BS(S_PQ, s) = tot[0];
+      BS(S_PR, s) = tot[1];
+      BS(S_ALPHA, s) = tot[1] / tot[0];
+  }
+}
+
+// the tile's sums; the block that completes system s runs its scalar step.  Every
+// thread of the block calls it (tile t lies in system s).
+template <int ND>
+__device__ __forceinline__ void seg_finish(const double (&acc)[ND], const SegArgs &g, int32_t t, int32_t s) {
+  __shared__ double sh[ND][kSegThreads];
+  __shared__ double tot[ND];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int32_t t0 = g.sys_tile[s], nt = g.sys_tile[s + 1] - t0;
+#pragma unroll
+  for (int k = 0; k < ND; ++k) sh[k][threadIdx.x] = acc[k];
+  __syncthreads();
+  if (wid < ND) {
+    double v = sh[wid][lane];
+#pragma unroll
+    for (int q = 1; q < kSegThreads / 32; ++q) v += sh[wid][q * 32 + lane];
+    v = warp_sum(v);
+    if (lane == 0) {
+      if (nt == 1) {
+        tot[wid] = v;
+      } else {
+        g.tpart[(int64_t)wid * g.ntiles + t] = v;
+        __threadfence();
+      }
+    }
+  }
+  __syncthreads();
+  if (nt > 1) {
+    if (threadIdx.x == 0) last = atomicAdd(g.ticket + s, 1) == nt - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    if (wid < ND) {
+      const double *p = g.tpart + (int64_t)wid * g.ntiles + t0;
+      double v = 0.0;
+      for (int32_t q = lane; q < nt; q += 32) v += __ldcg(p + q);
+      v = warp_sum(v);
+      if (lane == 0) tot[wid] = v;
+    }
+    if (threadIdx.x == 0) g.ticket[s] = 0;
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) run_bfin(g, s, ND, tot);
+}
+
+// s . y0 (, s . y1, s . y2) of every system
+template <class VS, class VY, int ND>
+__global__ void __launch_bounds__(kSegThreads) k_segdot(SegArgs g, const VS *sv, const VY *y0, const VY *y1,
+                                                        const VY *y2, const int *pred) {
+  pdl_trigger();
+  pdl_wait();
+  if (g.kind == BF_K1 && blockIdx.x == 0 && threadIdx.x == 0) g.flag[g.nsys] = 0;  // also when the step is skipped
   if (pred && *pred == 0) return;
-  for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x)
-    BS(S_S1, s) = BS(S_A1, s) / BS(S_RHO1, s);
+  for (int32_t t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
+    const int32_t s = g.tile_sys[t];
+    if (g.bact && !g.bact[s]) continue;
+    double acc[ND] = {0.0};
+    const int32_t r1 = g.tile_row[t + 1];
+#pragma unroll 4
+    for (int32_t i = g.tile_row[t] + threadIdx.x; i < r1; i += kSegThreads) {
+      const double x = (double)sv[i];
+      acc[0] += x * (double)y0[i];
+      if constexpr (ND > 1) acc[1] += x * (double)y1[i];
+      if constexpr (ND > 2) acc[2] += x * (double)y2[i];
+    }
+    seg_finish<ND>(acc, g, t, s);
+    __syncthreads();  // the shared sums are rewritten by the next tile
+  }
+}
+
+// r~ = r - (alpha_1/rho_1) v and x0 = wd r~ per system, and the test of Alg. 5
+template <class VT>
+__global__ void __launch_bounds__(kSegThreads) k_baxpy_rt(SegArgs g, const VT *r, const VT *v, VT *rt,
+                                                          const VT *__restrict__ wd, VT *x0, const int *pred) {
+  pdl_trigger();
+  pdl_wait();
+  if (pred && *pred == 0) return;
+  for (int32_t t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
+    const int32_t s = g.tile_sys[t];
+    if (g.bact && !g.bact[s]) continue;
+    const VT s1 = (VT)g.bslots[(int64_t)S_S1 * g.nsys + s];
+    double acc[2] = {0.0, 0.0};
+    const int32_t i1 = g.tile_row[t + 1];
+#pragma unroll 4
+    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kSegThreads) {
+      const VT ri = r[i], ti = ri - s1 * v[i];
+      rt[i] = ti;
+      x0[i] = wd[i] * ti;
+      acc[0] += (double)ti * (double)ti;
+      acc[1] += (double)ri * (double)ri;
+    }
+    seg_finish<2>(acc, g, t, s);
+    __syncthreads();
+  }
 }
 
 template <class VT>
-__global__ void k_baxpy_rt(int32_t n, const int32_t *__restrict__ sys, int32_t nsys, const VT *__restrict__ r,
-                           const VT *__restrict__ v, VT *__restrict__ rt, const VT *__restrict__ wd,
-                           VT *__restrict__ x0, const double *__restrict__ bslots, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const VT t = r[i] - (VT)BS(S_S1, sys[i]) * v[i];
-    rt[i] = t;
-    x0[i] = wd[i] * t;
-  }
-}
-
-// per-system test ||r~|| <= t ||r|| (norms squared in S_NRT2, S_NR2); flag[nsys] = any
-__global__ void k_bdecide(int32_t nsys, const double *__restrict__ bslots, double t, const int *parent,
-                          int *__restrict__ flag) {
-  pdl_wait_and_trigger();
-  __shared__ int any;
-  if (threadIdx.x == 0) any = 0;
-  __syncthreads();
-  const int active = parent ? *parent : 1;
-  for (int32_t s = threadIdx.x; s < nsys; s += blockDim.x) {
-    const bool second = active && !(sqrt(BS(S_NRT2, s)) <= t * sqrt(BS(S_NR2, s)));
-    flag[s] = second ? 1 : 0;
-    if (second) any = 1;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) flag[nsys] = any;
-}
-
-__global__ void k_bfin_k3(int32_t nsys, double *__restrict__ bslots, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x) {
-    const double rho1 = BS(S_RHO1, s), gam = BS(S_GAM, s), bet = BS(S_BET, s), a2 = BS(S_A2, s);
-    const double rho2 = bet - gam * gam / rho1;
-    BS(S_CC, s) = BS(S_S1, s) - gam * a2 / (rho1 * rho2);
-    BS(S_CD, s) = a2 / rho2;
-  }
-}
-
-template <class VT>
-__global__ void k_bcombine(int32_t n, const int32_t *__restrict__ sys, int32_t nsys, const VT *__restrict__ c,
-                           const VT *__restrict__ d, VT *__restrict__ x, const double *__restrict__ bslots,
-                           const int *__restrict__ flag, const int *pred) {
-  pdl_wait_and_trigger();
+__global__ void k_bcombine(int32_t n, const int32_t *__restrict__ sys, int32_t nsys, const VT *c, const VT *d, VT *x,
+                           const double *bslots, const int *flag, const int *bact, const int *pred) {
+  pdl_trigger();
+  pdl_wait();
   if (pred && *pred == 0) return;
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int32_t s = sys[i];
+    if (!bact[s]) continue;
     x[i] = flag[s] ? (VT)BS(S_CC, s) * c[i] + (VT)BS(S_CD, s) * d[i] : (VT)BS(S_S1, s) * c[i];
   }
 }
@@ -1296,13 +1361,15 @@ __global__ void k_bcombine(int32_t n, const int32_t *__restrict__ sys, int32_t n
 template <class VT>
 __global__ void k_bcoarse(int32_t nL, const int32_t *__restrict__ sys, const int32_t *__restrict__ off,
                           const double *__restrict__ binv, const int64_t *__restrict__ boff, const VT *__restrict__ b,
-                          VT *__restrict__ x, const int *pred) {
+                          VT *__restrict__ x, const int *bact, const int *pred) {
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
   const int lane = threadIdx.x & 31;
   for (int32_t i = blockIdx.x * kWarps + (threadIdx.x >> 5); i < nL; i += gridDim.x * kWarps) {
-    const int32_t s = sys[i], r0 = off[s], m = off[s + 1] - r0;
+    const int32_t s = sys[i];
+    if (!bact[s]) continue;
+    const int32_t r0 = off[s], m = off[s + 1] - r0;
     const double *Bi = binv + boff[s] + (int64_t)(i - r0) * m;
     double acc = 0.0;
     for (int32_t j = lane; j < m; j += 32) acc += Bi[j] * (double)b[r0 + j];
@@ -1311,45 +1378,53 @@ __global__ void k_bcoarse(int32_t nL, const int32_t *__restrict__ sys, const int
   }
 }
 
-// flexible CG per system.  bact[s]: still iterating; brs[s]: restart (beta = 0)
-__global__ void k_bfcg_beta(int32_t nsys, double *__restrict__ bslots, const int *__restrict__ brs) {
-  pdl_wait_and_trigger();
-  for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x)
-    BS(S_BETA, s) = brs[s] ? 0.0 : -BS(S_ZQ, s) / BS(S_PQ, s);
-}
-
-__global__ void k_bfcg_p(int32_t n, const int32_t *__restrict__ sys, int32_t nsys, const double *__restrict__ z,
-                         double *__restrict__ p, const double *__restrict__ bslots) {
-  pdl_wait_and_trigger();
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = z[i] + BS(S_BETA, sys[i]) * p[i];
-}
-
-__global__ void k_bfcg_alpha(int32_t nsys, double *__restrict__ bslots) {
-  pdl_wait_and_trigger();
-  for (int32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x)
-    BS(S_ALPHA, s) = BS(S_PR, s) / BS(S_PQ, s);
-}
-
-__global__ void k_bfcg_update(int32_t n, const int32_t *__restrict__ sys, int32_t nsys, double *__restrict__ x,
-                              double *__restrict__ r, const double *__restrict__ p, const double *__restrict__ q,
-                              const double *__restrict__ bslots, const int *__restrict__ bact) {
-  pdl_wait_and_trigger();
+// flexible CG per system.  bact[s]: still iterating
+template <class VT>
+__global__ void k_bfcg_p(int32_t n, const int32_t *__restrict__ sys, int32_t nsys, const VT *z, double *p,
+                         const double *bslots, const int *bact) {
+  pdl_trigger();
+  pdl_wait();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int32_t s = sys[i];
-    if (!bact[s]) continue;  // converged systems keep x and r untouched
-    const double a = BS(S_ALPHA, s);
-    x[i] += a * p[i];
-    r[i] -= a * q[i];
+    if (bact[s]) p[i] = (double)z[i] + BS(S_BETA, s) * p[i];
+  }
+}
+
+// x += alpha p, r -= alpha q, the next preconditioner input and its smoothing start,
+// ||r||^2; stopped systems keep x and r untouched
+template <class VT>
+__global__ void __launch_bounds__(kSegThreads) k_bfcg_update(SegArgs g, double *x, double *r, const double *p,
+                                                             const double *q, VT *rvt, const VT *__restrict__ wd,
+                                                             VT *x0) {
+  pdl_trigger();
+  pdl_wait();
+  for (int32_t t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
+    const int32_t s = g.tile_sys[t];
+    if (!g.bact[s]) continue;
+    const double a = g.bslots[(int64_t)S_ALPHA * g.nsys + s];
+    double acc[1] = {0.0};
+    const int32_t i1 = g.tile_row[t + 1];
+#pragma unroll 4
+    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kSegThreads) {
+      x[i] += a * p[i];
+      const double ri = r[i] - a * q[i];
+      r[i] = ri;
+      acc[0] += ri * ri;
+      const VT v = (VT)ri;
+      if (rvt) rvt[i] = v;
+      x0[i] = wd[i] * v;
+    }
+    seg_finish<1>(acc, g, t, s);
+    __syncthreads();
   }
 }
 
 // end of an iteration: per-system relative residual, iteration count, status;
-// bact[nsys] = number of systems still iterating; hist[k] (k < hist_len) gets
-// the largest relative residual of pass k
+// bact[nsys] = number of systems still iterating, also in the mapped pinned word
+// host; hist[k] (k < hist_len) gets the largest relative residual of pass k
 __global__ void k_bfcg_fin(int32_t nsys, double *__restrict__ bslots, int *__restrict__ bact, int *__restrict__ brs,
                            int *__restrict__ bit, int *__restrict__ bstat, double tol, int max_iter,
-                           double *__restrict__ hist, int hist_len, int *__restrict__ it) {
+                           double *__restrict__ hist, int hist_len, int *__restrict__ it, volatile int *host) {
   pdl_wait_and_trigger();
   __shared__ int nact;
   __shared__ double worst;
@@ -1388,6 +1463,8 @@ __global__ void k_bfcg_fin(int32_t nsys, double *__restrict__ bslots, int *__res
     const int k = *it + 1;
     *it = k;
     if (k < hist_len) hist[k] = worst;
+    *host = nact;
+    __threadfence_system();
   }
 }
 
@@ -1530,7 +1607,8 @@ struct Engine {
     if (k == h.L - 1) {
       if (h.batched)
         klaunch(k_bcoarse<VT>, grid_for(h.nL, kWarps, 152 * 8), kThreads, s, h.nL, (const int32_t *)L.sys_of,
-                (const int32_t *)L.sys_off, (const double *)h.binv, (const int64_t *)h.binv_off, rhs, out, pred);
+                (const int32_t *)L.sys_off, (const double *)h.binv, (const int64_t *)h.binv_off, rhs, out,
+                (const int *)h.bactive, pred);
       else
         klaunch(k_coarse<VT>, grid_for(h.nL, kWarps, 152), kThreads, s, h.nL, h.coarse_inv, rhs, out, pred);
       check();
@@ -1656,16 +1734,32 @@ struct Engine {
   }
   bool zq_fuse = false;
 
-  // per-system inner products of the batch into bslots[slot0 ..]
-  void segdot(int k, int ndot, const VT *a0, const VT *b0, const VT *a1, const VT *b1, const VT *a2, const VT *b2,
-              int slot0, const int *pred) {
+  // tiles of level k and the scalar step that ends its per-system inner products;
+  // gate: systems still iterating only
+  SegArgs seg_args(int k, BFin kind, bool gate, int slot0 = 0) {
     Level &L = h.lev[k];
-    klaunch(k_segdot<VT>, grid_for(L.ntiles, 1, 152 * 8), kThreads, s, L.ntiles, (const int32_t *)L.tile_row, ndot,
-            a0, b0, a1, b1, a2, b2, L.tpart, pred);
-    klaunch(k_segfin, grid_for(h.nsys, kWarps, 152), kThreads, s, (int32_t)h.nsys, L.ntiles,
-            (const int32_t *)L.sys_tile, ndot, (const double *)L.tpart, L.bslots, slot0, pred);
-    launches += 2;
-    AMG_LAUNCH_CHECK();
+    SegArgs g{};
+    g.ntiles = L.ntiles;
+    g.nsys = h.nsys;
+    g.tile_row = L.tile_row;
+    g.tile_sys = L.tile_sys;
+    g.sys_tile = L.sys_tile;
+    g.bact = gate ? h.bactive : nullptr;
+    g.tpart = L.tpart;
+    g.ticket = L.bticket;
+    g.bslots = L.bslots;
+    g.kind = kind;
+    g.slot0 = slot0;
+    g.flag = L.bflag;
+    g.t = h.p.kcycle_t;
+    g.brs = h.bactive + h.nsys + 1;
+    return g;
+  }
+  static int seg_grid(const SegArgs &g) { return grid_for(g.ntiles, 1, 152 * 4); }
+  template <int ND, class VS, class VY>
+  void segdot(const SegArgs &g, const VS *sv, const VY *y0, const VY *y1, const VY *y2, const int *pred) {
+    klaunch(k_segdot<VS, VY, ND>, seg_grid(g), kSegThreads, s, g, sv, y0, y1, y2, pred);
+    check();
   }
 
   // Alg. 5 coarse part at level m for every system of a batch, with per-system
@@ -1673,31 +1767,22 @@ struct Engine {
   void krylov2_batched(int m, const int *pred) {
     Level &L = h.lev[m];
     const int32_t ns = h.nsys;
+    const VT *nil = nullptr;
     cycle(m, V(L.bc), V(L.c), true, pred);
     sell<E_Y>(sell_args(m, V(L.c), V(L.v), pred), m);
-    if (gmres_variant)
-      segdot(m, 2, V(L.v), V(L.v), V(L.v), V(L.bc), nullptr, nullptr, S_RHO1, pred);
-    else
-      segdot(m, 2, V(L.c), V(L.v), V(L.c), V(L.bc), nullptr, nullptr, S_RHO1, pred);
-    klaunch(k_bfin_k1, grid_for(ns, kThreads, 152), kThreads, s, ns, L.bslots, pred);
-    klaunch(k_baxpy_rt<VT>, ew_grid(L.n), kThreads, s, L.n, (const int32_t *)L.sys_of, ns, (const VT *)V(L.bc),
-            (const VT *)V(L.v), V(L.rt), (const VT *)V(L.wd), V(L.tmp), (const double *)L.bslots, pred);
-    segdot(m, 2, V(L.rt), V(L.rt), V(L.bc), V(L.bc), nullptr, nullptr, S_NRT2, pred);
-    klaunch(k_bdecide, 1, 1024, s, ns, (const double *)L.bslots, h.p.kcycle_t, pred, L.bflag);
-    launches += 3;
-    AMG_LAUNCH_CHECK();
+    segdot<2>(seg_args(m, BF_K1, true), (const VT *)V(L.c), (const VT *)V(L.v), (const VT *)V(L.bc), nil, pred);
+    const SegArgs g = seg_args(m, BF_DECIDE, true);
+    klaunch(k_baxpy_rt<VT>, seg_grid(g), kSegThreads, s, g, (const VT *)V(L.bc), (const VT *)V(L.v), V(L.rt),
+            (const VT *)V(L.wd), V(L.tmp), pred);
+    check();
     const int *any = L.bflag + ns;
     cycle(m, V(L.rt), V(L.d), true, any);
     sell<E_Y>(sell_args(m, V(L.d), V(L.w), any), m);
-    if (gmres_variant)
-      segdot(m, 3, V(L.w), V(L.v), V(L.w), V(L.w), V(L.w), V(L.rt), S_GAM, any);
-    else
-      segdot(m, 3, V(L.d), V(L.v), V(L.d), V(L.w), V(L.d), V(L.rt), S_GAM, any);
-    klaunch(k_bfin_k3, grid_for(ns, kThreads, 152), kThreads, s, ns, L.bslots, any);
+    segdot<3>(seg_args(m, BF_K3, true), (const VT *)V(L.d), (const VT *)V(L.v), (const VT *)V(L.w),
+              (const VT *)V(L.rt), any);
     klaunch(k_bcombine<VT>, ew_grid(L.n), kThreads, s, L.n, (const int32_t *)L.sys_of, ns, (const VT *)V(L.c),
-            (const VT *)V(L.d), V(L.xc), (const double *)L.bslots, (const int *)L.bflag, pred);
-    launches += 2;
-    AMG_LAUNCH_CHECK();
+            (const VT *)V(L.d), V(L.xc), (const double *)L.bslots, (const int *)L.bflag, (const int *)h.bactive, pred);
+    check();
   }
 
   // Alg. 5 coarse part at level m: rhs = bc[m], result in xc[m]; lev[m].tmp holds wd*bc.
@@ -1774,25 +1859,34 @@ struct Engine {
   }
 
   // one flexible-CG iteration of every system of a batch (graph-capturable)
-  void fcg_iteration_batched(double tol) {
+  void fcg_iteration_batched(double tol, volatile int *host_active) {
     Level &L0 = h.lev[0];
     const int32_t ns = h.nsys, n = L0.n;
     const int ng = ew_grid(n);
     int *bact = h.bactive, *brs = h.bactive + ns + 1;
-    for (int k = 0; k < h.L; ++k) {  // slices of the systems still iterating
-      Level &L = h.lev[k];
-      klaunch(k_slice_live, grid_for(L.nslices, kThreads, 152 * 4), kThreads, s, L.n, L.nslices,
-              (const int32_t *)L.sys_of, (const int *)bact, L.slive);
-      ++launches;
+    {  // slices of the systems still iterating, on every level
+      LiveArgs la{};
+      for (int k = 0; k < h.L; ++k) {
+        const Level &L = h.lev[k];
+        la.n[k] = L.n;
+        la.nslices[k] = L.nslices;
+        la.sys[k] = L.sys_of;
+        la.live[k] = L.slive;
+      }
+      klaunch(k_slice_live, dim3((unsigned)grid_for(L0.nslices, kThreads, 152 * 4), (unsigned)h.L), kThreads, s, la,
+              (const int *)bact);
+      check();
     }
-    // z = M r
-    precond(h.r, h.z, nullptr);
-    Engine<double, double> e64(h, s);
-    e64.segdot(0, 1, h.z, h.q, nullptr, nullptr, nullptr, nullptr, S_ZQ, nullptr);
-    launches += e64.launches;
-    klaunch(k_bfcg_beta, grid_for(ns, kThreads, 152), kThreads, s, ns, L0.bslots, (const int *)brs);
-    klaunch(k_bfcg_p, ng, kThreads, s, n, (const int32_t *)L0.sys_of, ns, (const double *)h.z, h.pdir,
-            (const double *)L0.bslots);
+    // z = M r from the input and smoothing start left by k_bfcg_update
+    constexpr bool f64 = std::is_same<VT, double>::value;
+    const VT *in = f64 ? (const VT *)h.r : V(h.pre_in);
+    VT *z = f64 ? (VT *)h.z : V(h.pre_out);
+    cycle(0, in, z, true, nullptr);
+    const double *nil = nullptr;
+    segdot<1>(seg_args(0, BF_BETA, true), (const VT *)z, (const double *)h.q, nil, nil, nullptr);
+    klaunch(k_bfcg_p<VT>, ng, kThreads, s, n, (const int32_t *)L0.sys_of, ns, (const VT *)z, h.pdir,
+            (const double *)L0.bslots, (const int *)bact);
+    check();
     {  // q = A p in FP64
       SellArgs<double> a{};
       a.n = n;
@@ -1804,19 +1898,17 @@ struct Engine {
       a.out = h.q;
       a.live = L0.slive;
       klaunch(k_sell<double, double, E_Y, 0, true>, outer_grid(L0), kThreads, s, a);
+      check();
     }
-    launches += 3;
-    e64.launches = 0;
-    e64.segdot(0, 2, h.pdir, h.q, h.pdir, h.r, nullptr, nullptr, S_PQ, nullptr);
-    klaunch(k_bfcg_alpha, grid_for(ns, kThreads, 152), kThreads, s, ns, L0.bslots);
-    klaunch(k_bfcg_update, ng, kThreads, s, n, (const int32_t *)L0.sys_of, ns, h.x, h.r, (const double *)h.pdir,
-            (const double *)h.q, (const double *)L0.bslots, (const int *)bact);
-    e64.segdot(0, 1, h.r, h.r, nullptr, nullptr, nullptr, nullptr, S_RR, nullptr);
-    launches += e64.launches + 2;
+    segdot<2>(seg_args(0, BF_ALPHA, true), (const double *)h.pdir, (const double *)h.q, (const double *)h.r, nil,
+              nullptr);
+    const SegArgs g = seg_args(0, BF_STORE, true, S_RR);
+    klaunch(k_bfcg_update<VT>, seg_grid(g), kSegThreads, s, g, h.x, h.r, (const double *)h.pdir, (const double *)h.q,
+            f64 ? (VT *)nullptr : V(h.pre_in), (const VT *)V(L0.wd), V(L0.tmp));
+    check();
     klaunch(k_bfcg_fin, 1, 1024, s, ns, L0.bslots, bact, brs, h.bit, h.bit + ns, tol, h.p.max_iter, h.hist,
-            h.p.max_iter + 8, h.it_dev);
-    ++launches;
-    AMG_LAUNCH_CHECK();
+            h.p.max_iter + 8, h.it_dev, host_active);
+    check();
   }
 
   // one flexible-CG iteration, all on the device (graph-capturable)
@@ -2345,16 +2437,25 @@ int run_solve_batch_t(Hierarchy &h, const double *b, double *x, double tol, int3
   int64_t launches = 0;
   copy_in(h.b, b, n, s);
   copy_in(h.x, x, n, s);
-  e64.segdot(0, 1, h.b, h.b, nullptr, nullptr, nullptr, nullptr, S_NB2, nullptr);
+  const double *nil = nullptr;
+  e64.segdot<1>(e64.seg_args(0, BF_STORE, false, S_NB2), (const double *)h.b, (const double *)h.b, nil, nil, nullptr);
   klaunch(k_fix_zero_norm, grid_for(ns, kThreads, 152), kThreads, s, ns, L0.bslots);
-  klaunch(k_residual64, outer_grid(L0), kThreads, s, n, L0.nslices, (const int64_t *)L0.sptr64,
-          (const int32_t *)L0.scol64, (const double *)L0.sval64, (const double *)h.x, (const double *)h.b, h.r,
-          L0.partials + 7 * kRedBlocks);
-  e64.segdot(0, 1, h.r, h.r, nullptr, nullptr, nullptr, nullptr, S_RR, nullptr);
+  auto residual = [&](int slot) {  // r = b - A x and ||r||^2 of every system
+    klaunch(k_residual64, outer_grid(L0), kThreads, s, n, L0.nslices, (const int64_t *)L0.sptr64,
+            (const int32_t *)L0.scol64, (const double *)L0.sval64, (const double *)h.x, (const double *)h.b, h.r,
+            L0.partials + 7 * kRedBlocks);
+    e64.segdot<1>(e64.seg_args(0, BF_STORE, false, slot), (const double *)h.r, (const double *)h.r, nil, nil, nullptr);
+    ++launches;
+  };
+  residual(S_RR);
   klaunch(k_bset, 1, 1024, s, ns, (const double *)L0.bslots, tol, h.bactive, h.bit);
   AMG_CUDA(cudaMemsetAsync(h.it_dev, 0, sizeof(int), s));
-  launches += 3;
+  launches += 2;
   AMG_LAUNCH_CHECK();
+  // number of systems still iterating, in a mapped pinned word that a pass's last kernel writes
+  volatile int *active = reinterpret_cast<int *>(h.host_pinned + 32);
+  int *active_dev = nullptr;
+  AMG_CUDA(cudaHostGetDevicePointer(reinterpret_cast<void **>(&active_dev), h.host_pinned + 32, 0));
   // capture one iteration of all systems
   if (h.graph_exec) {
     cudaGraphExecDestroy(h.graph_exec);
@@ -2363,35 +2464,47 @@ int run_solve_batch_t(Hierarchy &h, const double *b, double *x, double tol, int3
   }
   if (h.p.use_graph) {
     AMG_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
-    eng.fcg_iteration_batched(tol);
+    eng.fcg_iteration_batched(tol, active_dev);
     AMG_CUDA(cudaStreamEndCapture(s, &h.graph));
     AMG_CUDA(cudaGraphInstantiate(&h.graph_exec, h.graph, 0));
     h.graph_launches = eng.launches;
     eng.launches = 0;
     h.graph_kind = -1;  // not the single-system iteration
   }
-  int *pin = reinterpret_cast<int *>(h.host_pinned + 32);
+  int *pin = reinterpret_cast<int *>(h.host_pinned + 36);
+  EventPair ep;
   int rounds = 0;
+  auto launch_pass = [&](int slot) {
+    if (h.p.use_graph) {
+      AMG_CUDA(cudaGraphLaunch(h.graph_exec, s));
+      launches += h.graph_launches;
+    } else {
+      eng.fcg_iteration_batched(tol, active_dev);
+    }
+    AMG_CUDA(cudaEventRecord(ep.e[slot], s));
+    ++rounds;
+  };
   for (;;) {
     AMG_CUDA(cudaMemcpyAsync(pin, h.bactive + ns, sizeof(int), cudaMemcpyDeviceToHost, s));
     AMG_CUDA(cudaStreamSynchronize(s));
     if (pin[0] > 0 && rounds < 100 * h.p.max_iter) {
-      if (h.p.use_graph) {
-        AMG_CUDA(cudaGraphLaunch(h.graph_exec, s));
-        launches += h.graph_launches;
-      } else {
-        eng.fcg_iteration_batched(tol);
+      eng.input_from_r(h.r, nullptr);
+      // the next pass is queued before this one's count is read (a pass after the
+      // last system stopped changes nothing)
+      *active = pin[0];
+      int slot = 0;
+      launch_pass(slot);
+      while (rounds < 100 * h.p.max_iter) {
+        launch_pass(slot ^ 1);
+        AMG_CUDA(cudaEventSynchronize(ep.e[slot]));
+        if (*active == 0) break;
+        slot ^= 1;
       }
-      ++rounds;
-      continue;
     }
     // every system stopped: check the true residuals, restart those that miss tol
-    klaunch(k_residual64, outer_grid(L0), kThreads, s, n, L0.nslices, (const int64_t *)L0.sptr64,
-            (const int32_t *)L0.scol64, (const double *)L0.sval64, (const double *)h.x, (const double *)h.b, h.r,
-            L0.partials + 7 * kRedBlocks);
-    e64.segdot(0, 1, h.r, h.r, nullptr, nullptr, nullptr, nullptr, S_TRUE_RR, nullptr);
+    residual(S_TRUE_RR);
     klaunch(k_brestart, 1, 1024, s, ns, (const double *)L0.bslots, tol, h.p.max_iter, h.bactive, h.bit);
-    launches += 2;
+    ++launches;
     AMG_CUDA(cudaMemcpyAsync(pin, h.bactive + ns, sizeof(int), cudaMemcpyDeviceToHost, s));
     AMG_CUDA(cudaStreamSynchronize(s));
     if (pin[0] == 0 || rounds >= 100 * h.p.max_iter) break;
@@ -2425,27 +2538,39 @@ int run_solve_batch_t(Hierarchy &h, const double *b, double *x, double tol, int3
 // one system and holds at most `tile` rows
 void build_tiles(Hierarchy &h, Level &L, int32_t tile, cudaStream_t s) {
   const int32_t ns = h.nsys;
-  std::vector<int32_t> trow, stile(ns + 1, 0);
+  std::vector<int32_t> trow, tsys, stile(ns + 1, 0);
   for (int32_t q = 0; q < ns; ++q) {
     stile[q] = (int32_t)trow.size();
-    for (int32_t r = L.sys_off_host[q]; r < L.sys_off_host[q + 1]; r += tile) trow.push_back(r);
+    for (int32_t r = L.sys_off_host[q]; r < L.sys_off_host[q + 1]; r += tile) {
+      trow.push_back(r);
+      tsys.push_back(q);
+    }
   }
   stile[ns] = (int32_t)trow.size();
   L.ntiles = (int32_t)trow.size();
   L.seg_tile = tile;
   trow.push_back(L.n);
   L.tile_row = h.arena.get<int32_t>(trow.size());
+  L.tile_sys = h.arena.get<int32_t>(tsys.size());
   L.sys_tile = h.arena.get<int32_t>(ns + 1);
   L.tpart = h.arena.get<double>(3 * (size_t)L.ntiles + 1);
   AMG_CUDA(cudaMemcpyAsync(L.tile_row, trow.data(), sizeof(int32_t) * trow.size(), cudaMemcpyHostToDevice, s));
+  AMG_CUDA(cudaMemcpyAsync(L.tile_sys, tsys.data(), sizeof(int32_t) * tsys.size(), cudaMemcpyHostToDevice, s));
   AMG_CUDA(cudaMemcpyAsync(L.sys_tile, stile.data(), sizeof(int32_t) * (ns + 1), cudaMemcpyHostToDevice, s));
-  AMG_CUDA(cudaStreamSynchronize(s));  // trow / stile leave scope
+  AMG_CUDA(cudaStreamSynchronize(s));  // trow, tsys and stile leave scope
 }
 
 // per-level system map, row tiles and per-system scalars of a batch
 void prepare_batched(Hierarchy &h, cudaStream_t s) {
   const int32_t ns = h.nsys;
   constexpr int32_t kTile = 2048;
+  h.bit = h.arena.get<int>(2 * (size_t)ns);
+  h.bactive = h.arena.get<int>(2 * (size_t)ns + 2);
+  {  // before the first solve (amg_precond, the autotuner) every system counts as iterating
+    const std::vector<int> one((size_t)ns + 1, 1);
+    AMG_CUDA(cudaMemcpyAsync(h.bactive, one.data(), sizeof(int) * (ns + 1), cudaMemcpyHostToDevice, s));
+    AMG_CUDA(cudaStreamSynchronize(s));
+  }
   for (int k = 0; k < h.L; ++k) {
     Level &L = h.lev[k];
     L.sys_of = h.arena.get<int32_t>((size_t)L.n + 1);
@@ -2455,11 +2580,11 @@ void prepare_batched(Hierarchy &h, cudaStream_t s) {
     build_tiles(h, L, kTile, s);
     L.bslots = h.arena.get<double>((size_t)kNumSlots * ns);
     L.bflag = h.arena.get<int>((size_t)ns + 1);
+    L.bticket = h.arena.get<int>((size_t)ns);
+    AMG_CUDA(cudaMemsetAsync(L.bticket, 0, sizeof(int) * ns, s));
     AMG_CUDA(cudaMemsetAsync(L.bslots, 0, sizeof(double) * kNumSlots * ns, s));
     AMG_CUDA(cudaMemsetAsync(L.bflag, 0, sizeof(int) * (ns + 1), s));
   }
-  h.bit = h.arena.get<int>(2 * (size_t)ns);
-  h.bactive = h.arena.get<int>(2 * (size_t)ns + 2);
   AMG_LAUNCH_CHECK();
 }
 
@@ -2519,7 +2644,9 @@ void autotune_t(Hierarchy &h, cudaStream_t s) {
         for (int tile : {1024, 2048, 4096, 8192}) {
           build_tiles(h, L, tile, s);
           tt.push_back({tile, time_it([&] {
-                          eng.segdot(k, 2, x.p, x.p, y.p, y.p, nullptr, nullptr, S_RHO1, nullptr);
+                          const VT *nil = nullptr;
+                          eng.template segdot<2>(eng.seg_args(k, BF_STORE, false, S_RHO1), (const VT *)x.p,
+                                                 (const VT *)y.p, (const VT *)y.p, nil, nullptr);
                         })});
         }
         build_tiles(h, L, pick(tt), s);
@@ -2539,6 +2666,10 @@ void run_precond_t(Hierarchy &h, const double *b, double *x, cudaStream_t s) {
   Engine<MV, VT> eng(h, s);
   const int32_t n = h.lev[0].n;
   if (!h.batched) trace_reset(h, s);
+  else {  // every system takes part, also after a solve that stopped them
+    AMG_CUDA(cudaMemsetAsync(h.bactive, 1, sizeof(int) * h.nsys, s));
+    for (int k = 0; k < h.L; ++k) AMG_CUDA(cudaMemsetAsync(h.lev[k].slive, 1, (size_t)h.lev[k].nslices + 1, s));
+  }
   copy_in(h.r, b, n, s);
   eng.precond(h.r, h.z, nullptr);
   copy_out(x, h.z, n, s);
