@@ -812,6 +812,39 @@ __device__ __forceinline__ double sum_partials(const double *__restrict__ part, 
   return result;
 }
 
+// Vector kernels take kRows rows a thread and round, their loads issued before the
+// first store: the compiler cannot move a load over a store that may alias, so a
+// plain loop has one row's loads in flight (a batch's tiles, one block each: 116.3 ->
+// 111.3 ms a pass of 40 systems with the tile sizes of build_tiles; the single-system
+// kernels, a full wave of blocks, run the same either way).
+constexpr int kRows = 4;
+// kRows rows i, i + step, ... < end of r~ = r - s1 v, x0 = wd r~, ||r~||^2 and ||r||^2
+template <class VT>
+__device__ __forceinline__ void axpy_rt_rows(int32_t i, int32_t step, int32_t end, VT s1, const VT *r, const VT *v,
+                                             VT *rt, const VT *__restrict__ wd, VT *x0, double (&acc)[2]) {
+  VT rv[kRows], vv[kRows], wv[kRows];
+#pragma unroll
+  for (int u = 0; u < kRows; ++u) {
+    const int32_t k = i + u * step;
+    if (k < end) {
+      rv[u] = r[k];
+      vv[u] = v[k];
+      wv[u] = wd[k];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kRows; ++u) {
+    const int32_t k = i + u * step;
+    if (k < end) {
+      const VT ti = rv[u] - s1 * vv[u];
+      rt[k] = ti;
+      x0[k] = wv[u] * ti;
+      acc[0] += (double)ti * (double)ti;
+      acc[1] += (double)rv[u] * (double)rv[u];
+    }
+  }
+}
+
 // r~ = r - (alpha_1/rho_1) v, the next smoothing start x0 = wd * r~, and the
 // test of Alg. 5 in the last block: the second inner step runs iff the enclosing
 // step runs and ||r~|| > t ||r||.  A skipped enclosing step clears the flag.
@@ -820,8 +853,6 @@ __global__ void __launch_bounds__(kThreads) k_axpy_rt(int32_t n, const VT *r, co
                                                       const VT *__restrict__ wd, VT *x0, double t, double *slots,
                                                       int *flag, double *part, unsigned *ticket, const int *pred) {
   pdl_trigger();
-  const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x;
-  VT w = i0 < n ? wd[i0] : VT(0);
   pdl_wait();
   if (pred && *pred == 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
@@ -829,15 +860,9 @@ __global__ void __launch_bounds__(kThreads) k_axpy_rt(int32_t n, const VT *r, co
   }
   const VT s1 = (VT)slots[S_S1];
   double acc[2] = {0.0, 0.0};
-  for (int32_t i = i0; i < n; i += gridDim.x * blockDim.x) {
-    if (i != i0) w = wd[i];
-    const VT ri = r[i];
-    const VT ti = ri - s1 * v[i];
-    rt[i] = ti;
-    x0[i] = w * ti;
-    acc[0] += (double)ti * (double)ti;
-    acc[1] += (double)ri * (double)ri;
-  }
+  const int32_t step = gridDim.x * blockDim.x;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kRows * step)
+    axpy_rt_rows<VT>(i, step, n, s1, r, v, rt, wd, x0, acc);
   double tot[2];
   if (grid_totals<2>(acc, 1, part, ticket, tot)) {
     slots[S_NRT2] = tot[0];
@@ -901,15 +926,27 @@ __global__ void __launch_bounds__(kThreads) k_dot_zq(int32_t n, const VT *__rest
 
 // p = z + beta p (beta = 0 right after a restart); z in the cycle's vector type
 template <class VT>
-__global__ void k_fcg_p(int32_t n, const VT *__restrict__ z, double *__restrict__ p, const double *__restrict__ slots,
-                        const int *__restrict__ restart, const int *pred) {
+__global__ void k_fcg_p(int32_t n, const VT *z, double *p, const double *slots, const int *restart,
+                        const int *pred) {
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
   const bool rs = *restart != 0;
   const double beta = slots[S_BETA];
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = rs ? (double)z[i] : (double)z[i] + beta * p[i];
+  const int32_t step = gridDim.x * blockDim.x;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kRows * step) {
+    VT zv[kRows];
+    double pv[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (i + u * step < n) {
+        zv[u] = z[i + u * step];
+        pv[u] = p[i + u * step];
+      }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (i + u * step < n) p[i + u * step] = rs ? (double)zv[u] : (double)zv[u] + beta * pv[u];
+  }
 }
 
 struct FcgState {
@@ -918,30 +955,57 @@ struct FcgState {
   volatile int *host;  // mapped pinned words: [0] iterations, [4] status
 };
 
+// kRows rows i, i + step, ... < end of the update of x and r, of the next
+// preconditioner input rvt (nullable) and its smoothing start x0, and of ||r||^2
+template <class VT>
+__device__ __forceinline__ void fcg_update_rows(int32_t i, int32_t step, int32_t end, double alpha, double *x,
+                                                double *r, const double *p, const double *q, VT *rvt,
+                                                const VT *__restrict__ wd, VT *x0, double &acc) {
+  double xv[kRows], rv[kRows], pv[kRows], qv[kRows];
+  VT wv[kRows];
+#pragma unroll
+  for (int u = 0; u < kRows; ++u) {
+    const int32_t k = i + u * step;
+    if (k < end) {
+      xv[u] = x[k];
+      pv[u] = p[k];
+      rv[u] = r[k];
+      qv[u] = q[k];
+      wv[u] = wd[k];
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < kRows; ++u) {
+    const int32_t k = i + u * step;
+    if (k < end) {
+      x[k] = xv[u] + alpha * pv[u];
+      const double ri = rv[u] - alpha * qv[u];
+      r[k] = ri;
+      acc += ri * ri;
+      const VT v = (VT)ri;
+      if (rvt) rvt[k] = v;
+      x0[k] = wv[u] * v;
+    }
+  }
+}
+
 // x += alpha p;  r -= alpha q;  the preconditioner input (in reduced precision
 // also rounded to VT) and its smoothing start x0 = wd r.  The last block ends the
 // outer iteration: relative residual into the history, iteration count,
 // convergence / breakdown status (deactivates the following launches).
 template <class VT>
-__global__ void __launch_bounds__(kThreads) k_fcg_update(int32_t n, double *__restrict__ x, double *__restrict__ r,
-                                                         const double *__restrict__ p, const double *__restrict__ q,
-                                                         double *__restrict__ slots, double *part, unsigned *ticket,
-                                                         VT *__restrict__ rvt, const VT *__restrict__ wd,
-                                                         VT *__restrict__ x0, FcgState st, const int *pred) {
+__global__ void __launch_bounds__(kThreads) k_fcg_update(int32_t n, double *x, double *r, const double *p,
+                                                         const double *q, double *slots, double *part,
+                                                         unsigned *ticket, VT *rvt, const VT *__restrict__ wd,
+                                                         VT *x0, FcgState st, const int *pred) {
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
   const double alpha = slots[S_ALPHA];
   double acc[1] = {0.0};
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    x[i] += alpha * p[i];
-    const double ri = r[i] - alpha * q[i];
-    r[i] = ri;
-    acc[0] += ri * ri;
-    const VT v = (VT)ri;
-    if (rvt) rvt[i] = v;
-    x0[i] = wd[i] * v;
-  }
+  const int32_t step = gridDim.x * blockDim.x;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kRows * step)
+    fcg_update_rows<VT>(i, step, n, alpha, x, r, p, q, rvt, wd, x0, acc[0]);
   double tot[1];
   if (grid_totals<1>(acc, 1, part, ticket, tot)) {
     const double rel = sqrt(tot[0]) / sqrt(slots[S_NB2]);
@@ -1211,7 +1275,7 @@ struct SegArgs {
   const int *brs;   // BF_BETA: restart flags
 };
 
-constexpr int kSegThreads = 512;
+constexpr int kSegThreads = 256;
 
 __device__ __forceinline__ void run_bfin(const SegArgs &g, int32_t s, int nd, const double *tot) {
   double *bslots = g.bslots;
@@ -1331,14 +1395,8 @@ __global__ void __launch_bounds__(kSegThreads) k_baxpy_rt(SegArgs g, const VT *r
     const VT s1 = (VT)g.bslots[(int64_t)S_S1 * g.nsys + s];
     double acc[2] = {0.0, 0.0};
     const int32_t i1 = g.tile_row[t + 1];
-#pragma unroll 4
-    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kSegThreads) {
-      const VT ri = r[i], ti = ri - s1 * v[i];
-      rt[i] = ti;
-      x0[i] = wd[i] * ti;
-      acc[0] += (double)ti * (double)ti;
-      acc[1] += (double)ri * (double)ri;
-    }
+    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kRows * kSegThreads)
+      axpy_rt_rows<VT>(i, kSegThreads, i1, s1, r, v, rt, wd, x0, acc);
     seg_finish<2>(acc, g, t, s);
     __syncthreads();
   }
@@ -1384,9 +1442,25 @@ __global__ void k_bfcg_p(int32_t n, const int32_t *__restrict__ sys, int32_t nsy
                          const double *bslots, const int *bact) {
   pdl_trigger();
   pdl_wait();
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int32_t s = sys[i];
-    if (bact[s]) p[i] = (double)z[i] + BS(S_BETA, s) * p[i];
+  const int32_t step = gridDim.x * blockDim.x;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kRows * step) {
+    int32_t sv[kRows];
+    VT zv[kRows];
+    double pv[kRows];
+#pragma unroll
+    for (int u = 0; u < kRows; ++u) sv[u] = i + u * step < n ? sys[i + u * step] : -1;
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (sv[u] >= 0 && !bact[sv[u]]) sv[u] = -1;
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (sv[u] >= 0) {
+        zv[u] = z[i + u * step];
+        pv[u] = p[i + u * step];
+      }
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (sv[u] >= 0) p[i + u * step] = (double)zv[u] + BS(S_BETA, sv[u]) * pv[u];
   }
 }
 
@@ -1404,16 +1478,8 @@ __global__ void __launch_bounds__(kSegThreads) k_bfcg_update(SegArgs g, double *
     const double a = g.bslots[(int64_t)S_ALPHA * g.nsys + s];
     double acc[1] = {0.0};
     const int32_t i1 = g.tile_row[t + 1];
-#pragma unroll 4
-    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kSegThreads) {
-      x[i] += a * p[i];
-      const double ri = r[i] - a * q[i];
-      r[i] = ri;
-      acc[0] += ri * ri;
-      const VT v = (VT)ri;
-      if (rvt) rvt[i] = v;
-      x0[i] = wd[i] * v;
-    }
+    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kRows * kSegThreads)
+      fcg_update_rows<VT>(i, kSegThreads, i1, a, x, r, p, q, rvt, wd, x0, acc[0]);
     seg_finish<1>(acc, g, t, s);
     __syncthreads();
   }
@@ -1755,7 +1821,7 @@ struct Engine {
     g.brs = h.bactive + h.nsys + 1;
     return g;
   }
-  static int seg_grid(const SegArgs &g) { return grid_for(g.ntiles, 1, 152 * 4); }
+  static int seg_grid(const SegArgs &g) { return grid_for(g.ntiles, 1, 152 * 8); }
   template <int ND, class VS, class VY>
   void segdot(const SegArgs &g, const VS *sv, const VY *y0, const VY *y1, const VY *y2, const int *pred) {
     klaunch(k_segdot<VS, VY, ND>, seg_grid(g), kSegThreads, s, g, sv, y0, y1, y2, pred);
@@ -2534,10 +2600,15 @@ int run_solve_batch_t(Hierarchy &h, const double *b, double *x, double tol, int3
   return status;
 }
 
-// row tiles of level L for the per-system inner products: every tile lies in
-// one system and holds at most `tile` rows
-void build_tiles(Hierarchy &h, Level &L, int32_t tile, cudaStream_t s) {
+// Row tiles of level L for the per-system inner products, every tile in one system.
+// `tile` rows suit a level that fills the GPU with kSegWave of them; smaller levels
+// take smaller tiles (two rows a thread at least) so that their FP64 work meets more
+// SMs, larger ones up to four times larger tiles with fewer sums to finish.
+constexpr int32_t kSegWave = 152 * 4;
+void build_tiles(Hierarchy &h, Level &L, int32_t seg_tile, cudaStream_t s) {
   const int32_t ns = h.nsys;
+  const int64_t fit = (int64_t)L.n * seg_tile / ((int64_t)kSegWave * 2048);
+  const int32_t tile = (int32_t)std::max<int64_t>(2 * kSegThreads, std::min<int64_t>(4 * (int64_t)seg_tile, (fit + 255) / 256 * 256));
   std::vector<int32_t> trow, tsys, stile(ns + 1, 0);
   for (int32_t q = 0; q < ns; ++q) {
     stile[q] = (int32_t)trow.size();
@@ -2548,7 +2619,7 @@ void build_tiles(Hierarchy &h, Level &L, int32_t tile, cudaStream_t s) {
   }
   stile[ns] = (int32_t)trow.size();
   L.ntiles = (int32_t)trow.size();
-  L.seg_tile = tile;
+  L.seg_tile = seg_tile;
   trow.push_back(L.n);
   L.tile_row = h.arena.get<int32_t>(trow.size());
   L.tile_sys = h.arena.get<int32_t>(tsys.size());
