@@ -1076,158 +1076,271 @@ __global__ void k_residual64(int32_t n, int32_t nslices, const int64_t *__restri
 // ---------------------------------------------------------------- outer FGMRES (FP64)
 constexpr int kMaxRestart = 32;
 
-// partial dot products of w with the basis vectors V_0..V_{ncol-1}, eight
-// columns per sweep over the rows
-__global__ void k_mdot(int32_t n, const double *__restrict__ V, int ncol, const double *__restrict__ w,
-                       double *__restrict__ part, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  __shared__ double sh[kWarps][8];
-  for (int c0 = 0; c0 < ncol; c0 += 8) {
-    double acc[8];
-#pragma unroll
-    for (int l = 0; l < 8; ++l) acc[l] = 0.0;
-    for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-      const double wi = w[i];
-#pragma unroll
-      for (int l = 0; l < 8; ++l)
-        if (c0 + l < ncol) acc[l] += V[(int64_t)(c0 + l) * n + i] * wi;
-    }
-#pragma unroll
-    for (int l = 0; l < 8; ++l) {
-      const double v = warp_sum(acc[l]);
-      if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][l] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < 8 && c0 + (int)threadIdx.x < ncol) {
-      double v = 0.0;
-      for (int wq = 0; wq < kWarps; ++wq) v += sh[wq][threadIdx.x];
-      part[(int64_t)(c0 + threadIdx.x) * kRedBlocks + blockIdx.x] = v;
-    }
-    __syncthreads();
-  }
-}
+// One Arnoldi step is the cycle, the product w = A z_j and four launches: the
+// classical Gram-Schmidt coefficients (GS_DOT), the update and the coefficients of
+// the reorthogonalisation (GS_AGAIN), its update with ||w|| and the Givens step
+// (GS_LAST), and the next basis vector with the preconditioner's input.  The step
+// number is a device word, so that one captured graph serves every step of a
+// restart.  Bound by L2 up to a few 10^5 rows, by HBM beyond; what the separate
+// sums, norm, scalar and conversion kernels cost was their launches' latency, and the
+// host's wait for every step: 301^2 convection-diffusion in FP64, 19.1 -> 14.6 ms a solve.
+struct FgArgs {
+  int32_t n;
+  int m;            // restart length (leading dimension of H)
+  double *V, *Z;    // basis and preconditioned vectors, column by column
+  double *w;        // A z_j
+  const double *z;  // z_j, copied to Z by GS_DOT
+  double *H, *fg;   // fg[0..m] = g, fg[m+1..2m] = cos, fg[2m+1..3m] = sin
+  double *hc;       // coefficients of the running pass; hc[kMaxRestart + 1] = 1 / ||w||
+  double *part;     // (kMaxRestart + 1) x kRedBlocks
+  unsigned *ticket;
+  int *step;        // j
+  double *slots, *hist;
+  int *it, *active, *status;
+  volatile int *host;  // mapped pinned words: [0] iterations, [4] status
+};
+enum GsPass { GS_DOT = 0, GS_AGAIN = 1, GS_LAST = 2 };
 
-// h_l = sum of the partials of column l; H(l, j) += h_l; hc = h
-__global__ void k_fin_mdot(const double *__restrict__ part, int nb, int ncol, double *__restrict__ H, int ldh,
-                           int j, double *__restrict__ hc, int accumulate, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int l = wid; l < ncol; l += blockDim.x >> 5) {
-    double v = 0.0;
-    for (int b = lane; b < nb; b += 32) v += part[(int64_t)l * kRedBlocks + b];
-    v = warp_sum(v);
-    if (lane == 0) {
-      hc[l] = v;
-      H[l * ldh + j] = accumulate ? H[l * ldh + j] + v : v;
-    }
-  }
-}
-
-// w -= sum_l hc_l V_l
-__global__ void k_maxpy(int32_t n, const double *__restrict__ V, int ncol, const double *__restrict__ hc,
-                        double *__restrict__ w, const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  __shared__ double h[kMaxRestart + 1];
-  for (int l = threadIdx.x; l < ncol; l += blockDim.x) h[l] = hc[l];
-  __syncthreads();
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    double t = w[i];
-    for (int l = 0; l < ncol; ++l) t -= h[l] * V[(int64_t)l * n + i];
-    w[i] = t;
-  }
-}
-
-// v_{j+1} = w / ||w||, H(j+1, j) = ||w||   (norm from the partials, same in every block)
-__global__ void k_fg_normalize(int32_t n, const double *__restrict__ w, double *__restrict__ vnext,
-                               const double *__restrict__ part, int nb, double *__restrict__ H, int ldh, int j,
-                               const int *pred) {
-  pdl_wait_and_trigger();
-  if (pred && *pred == 0) return;
-  const double nrm = sqrt(sum_partials(part, 0, nb));
-  if (blockIdx.x == 0 && threadIdx.x == 0) H[(j + 1) * ldh + j] = nrm;
-  const double inv = nrm != 0.0 ? 1.0 / nrm : 0.0;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) vnext[i] = w[i] * inv;
-}
-
-// Givens rotations on column j of H, residual estimate |g_{j+1}| / ||b||
-// into the history; deactivates the following steps when done.
-// fg[0..m] = g, fg[m+1..2m] = cos, fg[2m+1..3m] = sin
-__global__ void k_fg_givens(double *__restrict__ H, int ldh, int j, int m, double *__restrict__ fg,
-                            double *__restrict__ slots, double *__restrict__ hist, int *__restrict__ it,
-                            int *__restrict__ active, int *__restrict__ status) {
-  pdl_wait_and_trigger();
-  if (threadIdx.x != 0 || blockIdx.x != 0 || *active == 0) return;
-  double *g = fg, *cs = fg + m + 1, *sn = fg + 2 * m + 1;
+// Givens rotations on column j of H (in shared memory), the residual estimate
+// |g_{j+1}| / ||b|| into the history; deactivates the following steps when done
+__device__ __forceinline__ void fg_givens(const FgArgs &a, int j, double *col, const double *cs, const double *sn,
+                                          double nrm) {
   for (int l = 0; l < j; ++l) {
-    const double a = H[l * ldh + j], b = H[(l + 1) * ldh + j];
-    H[l * ldh + j] = cs[l] * a + sn[l] * b;
-    H[(l + 1) * ldh + j] = -sn[l] * a + cs[l] * b;
+    const double p = col[l], q = col[l + 1];
+    col[l] = cs[l] * p + sn[l] * q;
+    col[l + 1] = -sn[l] * p + cs[l] * q;
   }
-  const double a = H[j * ldh + j], b = H[(j + 1) * ldh + j];
-  const double den = sqrt(a * a + b * b);
-  cs[j] = a / den;
-  sn[j] = b / den;
-  H[j * ldh + j] = den;
-  const double hn = H[(j + 1) * ldh + j];
-  H[(j + 1) * ldh + j] = 0.0;
-  g[j + 1] = -sn[j] * g[j];
-  g[j] = cs[j] * g[j];
-  const int k = *it + 1;
-  *it = k;
-  const double rel = fabs(g[j + 1]) / sqrt(slots[S_NB2]);
-  hist[k] = rel;
-  slots[S_REL] = rel;
-  if (!isfinite(rel)) {
-    *status = AMG_ERR_NAN;
-    *active = 0;
-  } else if (rel <= slots[S_TOL] || hn == 0.0) {
-    *status = 1;
-    *active = 0;
-  } else if (k >= (int)slots[S_MAXIT]) {
-    *status = AMG_ERR_NOT_CONVERGED;
-    *active = 0;
+  const double p = col[j], den = sqrt(p * p + nrm * nrm), c = p / den, s = nrm / den;
+  col[j] = den;
+  a.fg[a.m + 1 + j] = c;
+  a.fg[2 * a.m + 1 + j] = s;
+  const double g = a.fg[j];
+  a.fg[j + 1] = -s * g;
+  a.fg[j] = c * g;
+  a.hc[kMaxRestart + 1] = nrm != 0.0 ? 1.0 / nrm : 0.0;
+  *a.step = j + 1;
+  const int k = *a.it + 1;
+  *a.it = k;
+  const double rel = fabs(s * g) / sqrt(a.slots[S_NB2]);
+  a.hist[k] = rel;
+  a.slots[S_REL] = rel;
+  int status = 0;
+  if (!isfinite(rel)) status = AMG_ERR_NAN;
+  else if (rel <= a.slots[S_TOL] || nrm == 0.0) status = 1;
+  else if (k >= (int)a.slots[S_MAXIT]) status = AMG_ERR_NOT_CONVERGED;
+  if (status != 0) {
+    *a.status = status;
+    *a.active = 0;
   }
+  a.host[0] = k;
+  __threadfence_system();
+  a.host[4] = status;
+  __threadfence_system();
 }
 
-// y = H(0:j, 0:j)^-1 g by back substitution (one thread), into fg[3m+1 ..]
-__global__ void k_fg_trisolve(const double *__restrict__ H, int ldh, int j, int m, double *__restrict__ fg) {
-  pdl_wait_and_trigger();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const double *g = fg;
-  double *y = fg + 3 * m + 1;
-  for (int l = j - 1; l >= 0; --l) {
-    double t = g[l];
-    for (int q = l + 1; q < j; ++q) t -= H[l * ldh + q] * y[q];
-    y[l] = t / H[l * ldh + l];
+// The columns go by eight: a thread keeps eight sums over its rows, the block's 256
+// values of a column meet in one warp, and the last block sums the blocks' partials
+// in block order (a warp holds up to four columns at a time).
+template <int PASS>
+__global__ void __launch_bounds__(kThreads) k_fg_gs(FgArgs a) {
+  static_assert(kWarps == 8, "a warp per column of a group");
+  __shared__ double sh[PASS == GS_LAST ? 1 : 8][kThreads];
+  __shared__ double h[kMaxRestart + 1];
+  __shared__ double cs[PASS == GS_LAST ? kMaxRestart : 1], sn[PASS == GS_LAST ? kMaxRestart : 1];
+  __shared__ bool last;
+  pdl_trigger();
+  pdl_wait();
+  if (*a.active == 0) return;
+  const int j = *a.step, ncol = j + 1;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t n = a.n;
+  const int32_t i0 = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
+  double *w = a.w;
+  const double *V = a.V;
+  double norm2 = 0.0;
+  if (PASS == GS_DOT) {
+    for (int32_t i = i0; i < a.n; i += stride) a.Z[j * n + i] = a.z[i];
+  } else {  // w -= sum_l h_l V_l
+    if (threadIdx.x < ncol) h[threadIdx.x] = a.hc[threadIdx.x];
+    __syncthreads();
+    for (int32_t i = i0; i < a.n; i += stride) {
+      double t = w[i];
+      int l = 0;
+      for (; l + 8 <= ncol; l += 8) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = V[(l + q) * n + i];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) t -= h[l + q] * v[q];
+      }
+      for (; l < ncol; ++l) t -= h[l] * V[l * n + i];
+      w[i] = t;
+      if (PASS == GS_LAST) norm2 += t * t;
+    }
   }
-}
-
-// x += sum_l y_l Z_l
-__global__ void k_fg_xupdate(int32_t n, double *__restrict__ x, const double *__restrict__ Z, int ncol,
-                             const double *__restrict__ y) {
-  pdl_wait_and_trigger();
-  __shared__ double ys[kMaxRestart + 1];
-  for (int l = threadIdx.x; l < ncol; l += blockDim.x) ys[l] = y[l];
+  if constexpr (PASS == GS_LAST) {
+    sh[0][threadIdx.x] = norm2;
+    __syncthreads();
+    if (wid == 0) {
+      double v = sh[0][lane];
+#pragma unroll
+      for (int q = 1; q < kWarps; ++q) v += sh[0][q * 32 + lane];
+      v = warp_sum(v);
+      if (lane == 0) {
+        a.part[blockIdx.x] = v;
+        __threadfence();
+      }
+    }
+  } else {
+    for (int c0 = 0; c0 < ncol; c0 += 8) {
+      double acc[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[q] = 0.0;
+      for (int32_t i = i0; i < a.n; i += stride) {
+        const double wi = w[i];
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = c0 + q < ncol ? V[(c0 + q) * n + i] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          if (c0 + q < ncol) acc[q] += v[q] * wi;
+      }
+      __syncthreads();  // the previous group's sums have been read
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        if (c0 + q < ncol) sh[q][threadIdx.x] = acc[q];
+      __syncthreads();
+      if (c0 + wid < ncol) {
+        double v = sh[wid][lane];
+#pragma unroll
+        for (int q = 1; q < kWarps; ++q) v += sh[wid][q * 32 + lane];
+        v = warp_sum(v);
+        if (lane == 0) {
+          a.part[(c0 + wid) * kRedBlocks + blockIdx.x] = v;
+          __threadfence();
+        }
+      }
+    }
+  }
   __syncthreads();
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  if (threadIdx.x == 0) last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int nb = gridDim.x;
+  if constexpr (PASS != GS_LAST) {
+    for (int c0 = wid; c0 < ncol; c0 += 4 * kWarps) {
+      double v[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+      for (int b = lane; b < nb; b += 32)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (c0 + u * kWarps < ncol) v[u] += __ldcg(a.part + (c0 + u * kWarps) * kRedBlocks + b);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int l = c0 + u * kWarps;
+        if (l >= ncol) break;
+        const double t = warp_sum(v[u]);
+        if (lane == 0) {
+          a.hc[l] = t;
+          a.H[l * a.m + j] = PASS == GS_AGAIN ? a.H[l * a.m + j] + t : t;
+        }
+      }
+    }
+    if (threadIdx.x == 0) *a.ticket = 0;
+  } else {
+    double v = 0.0;
+    for (int b = threadIdx.x; b < nb; b += kThreads) v += __ldcg(a.part + b);
+    sh[0][threadIdx.x] = v;
+    if (threadIdx.x < ncol) h[threadIdx.x] = a.H[threadIdx.x * a.m + j];
+    if (threadIdx.x < j) {
+      cs[threadIdx.x] = a.fg[a.m + 1 + threadIdx.x];
+      sn[threadIdx.x] = a.fg[2 * a.m + 1 + threadIdx.x];
+    }
+    __syncthreads();
+    if (wid == 0) {
+      double t = sh[0][lane];
+#pragma unroll
+      for (int q = 1; q < kWarps; ++q) t += sh[0][q * 32 + lane];
+      t = warp_sum(t);
+      if (lane == 0) {
+        *a.ticket = 0;
+        fg_givens(a, j, h, cs, sn, sqrt(t));
+      }
+      __syncwarp();
+      for (int l = lane; l < ncol; l += 32) a.H[l * a.m + j] = h[l];
+    }
+  }
+}
+
+// V_j = v * scale with the preconditioner's input and smoothing start.  START: V_0 =
+// r / ||r||, g = (||r||, 0, ...); else V_j = w / ||w|| of the step just ended (the
+// last step of a restart needs no next vector).
+template <class VT, bool START>
+__global__ void __launch_bounds__(kThreads) k_fg_basis(FgArgs a, const double *v, VT *in, const VT *__restrict__ wd,
+                                                       VT *x0) {
+  pdl_trigger();
+  pdl_wait();
+  int j = 0;
+  double inv;
+  if (START) {
+    const double beta = sqrt(a.slots[S_RR]);
+    if (blockIdx.x == 0) {
+      for (int l = threadIdx.x; l <= a.m; l += blockDim.x) a.fg[l] = (l == 0) ? beta : 0.0;
+      if (threadIdx.x == 0) *a.step = 0;
+    }
+    inv = beta != 0.0 ? 1.0 / beta : 0.0;
+  } else {
+    if (*a.active == 0) return;
+    j = *a.step;
+    if (j >= a.m) return;
+    inv = a.hc[kMaxRestart + 1];
+  }
+  double *out = a.V + (int64_t)j * a.n;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
+    const double t = v[i] * inv;
+    out[i] = t;
+    in[i] = (VT)t;
+    x0[i] = wd[i] * (VT)t;
+  }
+}
+
+// x += sum_l y_l Z_l with y = H(0:j, 0:j)^-1 g, j the steps taken: every block solves
+// the triangular system in its first warp (lane l holds row l; at most 32 rows)
+__global__ void __launch_bounds__(kThreads) k_fg_xupdate(FgArgs a, double *__restrict__ x) {
+  static_assert(kMaxRestart <= 32, "a lane per row");
+  __shared__ double Hs[kMaxRestart][kMaxRestart + 1];
+  __shared__ double y[kMaxRestart];
+  pdl_trigger();
+  pdl_wait();
+  const int j = *a.step;
+  for (int q = threadIdx.x; q < j * j; q += kThreads) Hs[q / j][q % j] = a.H[(q / j) * a.m + q % j];
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    const int l = threadIdx.x;
+    double t = l < j ? a.fg[l] : 0.0;
+    for (int q = j - 1; q >= 0; --q) {
+      if (l == q) t /= Hs[q][q];
+      const double yq = __shfl_sync(0xffffffffu, t, q);
+      if (l < q) t -= Hs[l][q] * yq;
+    }
+    if (l < j) y[l] = t;
+  }
+  __syncthreads();
+  const int64_t n = a.n;
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += gridDim.x * blockDim.x) {
     double t = x[i];
-    for (int l = 0; l < ncol; ++l) t += ys[l] * Z[(int64_t)l * n + i];
+    int l = 0;
+    for (; l + 8 <= j; l += 8) {
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = a.Z[(l + q) * n + i];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) t += y[l + q] * v[q];
+    }
+    for (; l < j; ++l) t += y[l] * a.Z[l * n + i];
     x[i] = t;
   }
-}
-
-// V_0 = r / ||r||, g = (||r||, 0, ...)
-__global__ void k_fg_start(int32_t n, const double *__restrict__ r, double *__restrict__ v0,
-                           const double *__restrict__ slots, int slot_rr, double *__restrict__ fg, int m) {
-  pdl_wait_and_trigger();
-  const double beta = sqrt(slots[slot_rr]);
-  if (blockIdx.x == 0)
-    for (int l = threadIdx.x; l <= m; l += blockDim.x) fg[l] = (l == 0) ? beta : 0.0;
-  const double inv = beta != 0.0 ? 1.0 / beta : 0.0;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) v0[i] = r[i] * inv;
 }
 
 // ---------------------------------------------------------------- batched systems
@@ -2008,6 +2121,63 @@ struct Engine {
             (const VT *)V(L0.wd), V(L0.tmp), st, active);
     check();
   }
+
+  // FGMRES: basis passes take two rows a thread at least (fewer partial sums for the
+  // last block) and four blocks an SM at most
+  int gs_grid() const { return grid_for(h.lev[0].n, 2 * kThreads, 152 * 4); }
+  FgArgs fg_args(volatile int *host_state) {
+    Level &L0 = h.lev[0];
+    FgArgs a{};
+    a.n = L0.n;
+    a.m = h.p.restart;
+    a.V = h.V;
+    a.Z = h.Z;
+    a.w = h.q;
+    a.z = std::is_same<VT, double>::value ? (const double *)h.pre_out : h.z;
+    a.H = h.H;
+    a.fg = h.fg;
+    a.hc = h.hc;
+    a.part = h.gpart;
+    a.ticket = ticket(L0);
+    a.step = h.it_dev + 3;
+    a.slots = L0.slots;
+    a.hist = h.hist;
+    a.it = h.it_dev;
+    a.active = h.it_dev + 1;
+    a.status = h.status_dev;
+    a.host = host_state;
+    return a;
+  }
+
+  // one Arnoldi step from the preconditioner input left by k_fg_basis (graph-capturable)
+  void fgmres_step(const FgArgs &f) {
+    Level &L0 = h.lev[0];
+    cycle(0, V(h.pre_in), V(h.pre_out), true, f.active);
+    if (!std::is_same<VT, double>::value) {
+      klaunch(k_from_vt<VT>, ew_grid(L0.n), kThreads, s, L0.n, (const VT *)V(h.pre_out), h.z, (const int *)f.active);
+      check();
+    }
+    {  // w = A z_j in FP64
+      SellArgs<double> a{};
+      a.n = L0.n;
+      a.nslices = L0.nslices;
+      a.sptr = L0.sptr64;
+      a.scol = L0.scol64;
+      a.sval = L0.sval64;
+      a.x = f.z;
+      a.out = f.w;
+      a.pred = f.active;
+      klaunch(k_sell<double, double, E_Y, 0, false>, outer_grid(L0), kThreads, s, a);
+      check();
+    }
+    klaunch(k_fg_gs<GS_DOT>, gs_grid(), kThreads, s, f);
+    klaunch(k_fg_gs<GS_AGAIN>, gs_grid(), kThreads, s, f);
+    klaunch(k_fg_gs<GS_LAST>, gs_grid(), kThreads, s, f);
+    klaunch(k_fg_basis<VT, false>, ew_grid(L0.n), kThreads, s, f, (const double *)f.w, V(h.pre_in),
+            (const VT *)V(L0.wd), V(L0.tmp));
+    launches += 3;
+    check();
+  }
 };
 
 template <class MV, class VT>
@@ -2356,12 +2526,25 @@ int run_fgmres_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *
   klaunch(k_set_state, 1, 32, s, h.it_dev, active, h.it_dev + 2, h.status_dev, 0, 1, 0, 0);
   launches += 5;
   AMG_LAUNCH_CHECK();
-  double *w = h.q;
   int it = 0, status = AMG_ERR_NOT_CONVERGED;
   std::vector<double> hist;
   double nb2 = 1.0;
   bool first = true;
-  int *st_host = reinterpret_cast<int *>(h.host_pinned + 32);
+  // state of the iteration in mapped pinned words: [0] iterations, [4] status
+  volatile int *st_host = reinterpret_cast<int *>(h.host_pinned + 32);
+  int *st_dev = nullptr;
+  AMG_CUDA(cudaHostGetDevicePointer(reinterpret_cast<void **>(&st_dev), h.host_pinned + 32, 0));
+  const FgArgs f = eng.fg_args(st_dev);
+  EventPair ep;
+  auto launch_step = [&](int slot) {
+    if (h.p.use_graph) {
+      AMG_CUDA(cudaGraphLaunch(h.graph_exec, s));
+      launches += h.graph_launches;
+    } else {
+      eng.fgmres_step(f);
+    }
+    AMG_CUDA(cudaEventRecord(ep.e[slot], s));
+  };
   for (;;) {
     true_residual(h, S_RR, s, launches);
     AMG_CUDA(cudaMemcpyAsync(h.host_pinned, L0.slots, sizeof(double) * kNumSlots, cudaMemcpyDeviceToHost, s));
@@ -2380,53 +2563,40 @@ int run_fgmres_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *
     if (!std::isfinite(rel)) { status = AMG_ERR_NAN; break; }
     if (rel <= tol) { status = AMG_OK; break; }
     if (it >= h.p.max_iter) { status = AMG_ERR_NOT_CONVERGED; break; }
-    klaunch(k_fg_start, ng, kThreads, s, n, h.r, h.V, L0.slots, S_RR, h.fg, m);
-    klaunch(k_set_state, 1, 32, s, h.it_dev, active, h.it_dev + 2, h.status_dev, -1, 1, 0, 0);
-    launches += 2;
-    AMG_LAUNCH_CHECK();
-    int jused = 0, dst = 0;
-    for (int j = 0; j < m; ++j) {
-      double *vj = h.V + (size_t)j * n, *zj = h.Z + (size_t)j * n;
-      const int64_t before = eng.launches;
-      eng.precond(vj, zj, active);
-      {  // w = A z_j in FP64
-        SellArgs<double> a{};
-        a.n = n;
-        a.nslices = L0.nslices;
-        a.sptr = L0.sptr64;
-        a.scol = L0.scol64;
-        a.sval = L0.sval64;
-        a.x = zj;
-        a.out = w;
-        a.pred = active;
-        klaunch(k_sell<double, double, E_Y, 0, false>, outer_grid(L0), kThreads, s, a);
-        eng.check();
+    if (h.p.use_graph && h.graph_kind != 1) {  // capture one Arnoldi step
+      if (h.graph_exec) {
+        cudaGraphExecDestroy(h.graph_exec);
+        cudaGraphDestroy(h.graph);
+        h.graph_exec = nullptr;
       }
-      for (int pass = 0; pass < 2; ++pass) {  // classical Gram-Schmidt, twice
-        klaunch(k_mdot, ng, kThreads, s, n, h.V, j + 1, w, h.gpart, active);
-        klaunch(k_fin_mdot, 1, 1024, s, h.gpart, ng, j + 1, h.H, m, j, h.hc, pass, active);
-        klaunch(k_maxpy, ng, kThreads, s, n, h.V, j + 1, h.hc, w, active);
-        eng.launches += 3;
-        AMG_LAUNCH_CHECK();
-      }
-      klaunch(k_dot64, ng, kThreads, s, n, w, w, L0.partials + 6 * kRedBlocks, active);
-      klaunch(k_fg_normalize, ng, kThreads, s, n, w, h.V + (size_t)(j + 1) * n, L0.partials + 6 * kRedBlocks, ng,
-                                             h.H, m, j, active);
-      klaunch(k_fg_givens, 1, 32, s, h.H, m, j, m, h.fg, L0.slots, h.hist, h.it_dev, active, h.status_dev);
-      eng.launches += 3;
-      AMG_LAUNCH_CHECK();
-      (void)before;
-      AMG_CUDA(cudaMemcpyAsync(st_host, h.it_dev, sizeof(int) * 8, cudaMemcpyDeviceToHost, s));
-      AMG_CUDA(cudaStreamSynchronize(s));
-      it = st_host[0];
-      dst = st_host[4];
-      jused = j + 1;
-      if (dst != 0) break;
+      AMG_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
+      eng.fgmres_step(f);
+      AMG_CUDA(cudaStreamEndCapture(s, &h.graph));
+      AMG_CUDA(cudaGraphInstantiate(&h.graph_exec, h.graph, 0));
+      h.graph_kind = 1;
+      h.graph_launches = eng.launches;
+      eng.launches = 0;
     }
-    klaunch(k_fg_trisolve, 1, 32, s, h.H, m, jused, m, h.fg);
-    klaunch(k_fg_xupdate, ng, kThreads, s, n, h.x, h.Z, jused, h.fg + 3 * m + 1);
+    klaunch(k_set_state, 1, 32, s, h.it_dev, active, h.it_dev + 2, h.status_dev, -1, 1, 0, 0);
+    klaunch(k_fg_basis<VT, true>, ng, kThreads, s, f, (const double *)h.r, eng.V(h.pre_in), (const VT *)eng.V(L0.wd),
+            eng.V(L0.tmp));
     launches += 2;
     AMG_LAUNCH_CHECK();
+    // the next step is queued before this one's state is read (within a restart);
+    // once a step stops (*active = 0) every kernel of the next one returns at once
+    int dst = 0;
+    st_host[4] = 0;  // the stream was waited for above
+    launch_step(0);
+    for (int j = 0; j < m && dst == 0; ++j) {
+      if (j + 1 < m) launch_step((j + 1) & 1);
+      AMG_CUDA(cudaEventSynchronize(ep.e[j & 1]));
+      dst = st_host[4];
+    }
+    klaunch(k_fg_xupdate, eng.gs_grid(), kThreads, s, f, h.x);
+    ++launches;
+    AMG_LAUNCH_CHECK();
+    AMG_CUDA(cudaStreamSynchronize(s));
+    it = st_host[0];
     if (dst == AMG_ERR_NAN) { status = AMG_ERR_NAN; break; }
   }
   hist.resize((size_t)it + 1);
