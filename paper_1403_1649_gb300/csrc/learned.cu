@@ -456,15 +456,20 @@ __global__ void __launch_bounds__(256) k_grad_adam(const double *__restrict__ pa
 // evaluation to FP32 rounding, where FP16 activations alone would lose three
 // decimal digits.  The accumulator fragment of one layer (rows g, g+8; columns
 // 2t, 2t+1 of each 8-column tile) is the A-operand fragment of the next, so the
-// hidden activations never leave registers.
+// hidden activations never leave registers.  The weights lie in shared memory as the
+// lanes' fragments, one 16-byte word for two k-tiles: read from their rows (128 bytes
+// apart) the eight rows of a fragment met in the same banks.  2^20 rows: 166 -> 129 us;
+// bound by issue (17 of 24 instructions an activation are tanhf's), the tensor pipe at 30 %.
 __device__ __forceinline__ uint32_t pack_h2(__half x, __half y) {
   __half2 v = __halves2half2(x, y);
   return *reinterpret_cast<uint32_t *>(&v);
 }
 __device__ __forceinline__ void split_h2(float x, float y, uint32_t &hi, uint32_t &lo) {
-  const __half xh = __float2half_rn(x), yh = __float2half_rn(y);
-  hi = pack_h2(xh, yh);
-  lo = pack_h2(__float2half_rn(x - __half2float(xh)), __float2half_rn(y - __half2float(yh)));
+  const __half2 h = __floats2half2_rn(x, y);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(x - f.x, y - f.y);
+  hi = *reinterpret_cast<const uint32_t *>(&h);
+  lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 // c += A (16x16, row) * B (16x8, col)
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -478,17 +483,36 @@ constexpr int kTcWarps = 4;
 __global__ void __launch_bounds__(32 * kTcWarps) k_mlp_forward_tc(int32_t n, const __half *__restrict__ wg,
                                                                   const float *__restrict__ feat,
                                                                   float *__restrict__ out) {
-  __shared__ __align__(16) __half w[NP + 1];
-  __shared__ float bias[2 * NH + NO];
-  for (int k = threadIdx.x; k < NP; k += blockDim.x) w[k] = wg[k];
-  for (int k = threadIdx.x; k < NH; k += blockDim.x) {
-    bias[k] = __half2float(wg[B1O + k]);
-    bias[NH + k] = __half2float(wg[B2O + k]);
-  }
-  if (threadIdx.x < NO) bias[2 * NH + threadIdx.x] = __half2float(wg[B3O + threadIdx.x]);
-  __syncthreads();
+  // the B fragments of every lane, two k-tiles (layer 1: two n-tiles) per 16-byte word:
+  // {b0, b1} of the first, {b0, b1} of the second
+  __shared__ uint4 f1[NH / 16][32], f2[NH / 8][NH / 32][32], f3[NH / 32][32];
+  __shared__ float2 bias[NH + 2];
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  auto wpair = [&](int idx) { return *reinterpret_cast<const uint32_t *>(&w[idx]); };
+  {
+    const int wid = threadIdx.x >> 5;
+    auto wpair = [&](int idx) { return pack_h2(wg[idx], wg[idx + 1]); };
+    for (int q = wid; q < NH / 16; q += kTcWarps) {
+      const int at = W1O + (16 * q + g) * NF + 2 * t, at2 = at + 8 * NF;
+      f1[q][lane] = make_uint4(wpair(at), wpair(at + 8), wpair(at2), wpair(at2 + 8));
+    }
+    for (int q = wid; q < NH / 8 * (NH / 32); q += kTcWarps) {
+      const int at = W2O + (8 * (q >> 1) + g) * NH + 32 * (q & 1) + 2 * t;
+      f2[q >> 1][q & 1][lane] = make_uint4(wpair(at), wpair(at + 8), wpair(at + 16), wpair(at + 24));
+    }
+    for (int q = wid; q < NH / 32; q += kTcWarps) {  // three outputs in an 8-column tile
+      const int at = W3O + g * NH + 32 * q + 2 * t;
+      f3[q][lane] = g < NO ? make_uint4(wpair(at), wpair(at + 8), wpair(at + 16), wpair(at + 24)) : make_uint4(0, 0, 0, 0);
+    }
+    for (int k = threadIdx.x; k < NH / 2; k += blockDim.x) {
+      bias[k] = make_float2(__half2float(wg[B1O + 2 * k]), __half2float(wg[B1O + 2 * k + 1]));
+      bias[NH / 2 + k] = make_float2(__half2float(wg[B2O + 2 * k]), __half2float(wg[B2O + 2 * k + 1]));
+    }
+    if (threadIdx.x == 0) {
+      bias[NH] = make_float2(__half2float(wg[B3O]), __half2float(wg[B3O + 1]));
+      bias[NH + 1] = make_float2(__half2float(wg[B3O + 2]), 0.0f);
+    }
+  }
+  __syncthreads();
   for (int32_t tile = blockIdx.x * kTcWarps + (threadIdx.x >> 5); (int64_t)tile * 16 < n;
        tile += gridDim.x * kTcWarps) {
     const int32_t ra = tile * 16 + g, rb = ra + 8;
@@ -503,14 +527,16 @@ __global__ void __launch_bounds__(32 * kTcWarps) k_mlp_forward_tc(int32_t n, con
     }
     float c[8][4];
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int col = 8 * nt + 2 * t;
-      c[nt][0] = c[nt][2] = bias[col];
-      c[nt][1] = c[nt][3] = bias[col + 1];
-      const int wrow = W1O + (8 * nt + g) * NF + 2 * t;
-      const uint32_t b0 = wpair(wrow), b1 = wpair(wrow + 8);
-      mma_16816(c[nt], ah, b0, b1);
-      mma_16816(c[nt], al, b0, b1);
+    for (int nt = 0; nt < 8; nt += 2) {
+      const uint4 w = f1[nt / 2][lane];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float2 bv = bias[4 * (nt + q) + t];
+        c[nt + q][0] = c[nt + q][2] = bv.x;
+        c[nt + q][1] = c[nt + q][3] = bv.y;
+        mma_16816(c[nt + q], ah, q ? w.z : w.x, q ? w.w : w.y);
+        mma_16816(c[nt + q], al, q ? w.z : w.x, q ? w.w : w.y);
+      }
     }
     // tanh, then the accumulators as the A operand of the next layer (4 k-tiles)
     uint32_t hh[4][4], hl[4][4];
@@ -524,15 +550,16 @@ __global__ void __launch_bounds__(32 * kTcWarps) k_mlp_forward_tc(int32_t n, con
     // layer 2: 64 x 64
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-      const int col = 8 * nt + 2 * t;
-      c[nt][0] = c[nt][2] = bias[NH + col];
-      c[nt][1] = c[nt][3] = bias[NH + col + 1];
+      const float2 bv = bias[NH / 2 + 4 * nt + t];
+      c[nt][0] = c[nt][2] = bv.x;
+      c[nt][1] = c[nt][3] = bv.y;
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const int wrow = W2O + (8 * nt + g) * NH + 16 * kk + 2 * t;
-        const uint32_t b0 = wpair(wrow), b1 = wpair(wrow + 8);
-        mma_16816(c[nt], hh[kk], b0, b1);
-        mma_16816(c[nt], hl[kk], b0, b1);
+      for (int kk = 0; kk < 4; kk += 2) {
+        const uint4 w = f2[nt][kk / 2][lane];
+        mma_16816(c[nt], hh[kk], w.x, w.y);
+        mma_16816(c[nt], hl[kk], w.x, w.y);
+        mma_16816(c[nt], hh[kk + 1], w.z, w.w);
+        mma_16816(c[nt], hl[kk + 1], w.z, w.w);
       }
     }
 #pragma unroll
@@ -544,14 +571,16 @@ __global__ void __launch_bounds__(32 * kTcWarps) k_mlp_forward_tc(int32_t n, con
     }
     // layer 3: 3 outputs in the first 8-column tile (columns 3..7 zero)
     float o[4];
-    o[0] = o[2] = 2 * t < NO ? bias[2 * NH + 2 * t] : 0.0f;
-    o[1] = o[3] = 2 * t + 1 < NO ? bias[2 * NH + 2 * t + 1] : 0.0f;
+    const float2 bv = t < 2 ? bias[NH + t] : make_float2(0.0f, 0.0f);
+    o[0] = o[2] = bv.x;
+    o[1] = o[3] = bv.y;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const int wrow = W3O + g * NH + 16 * kk + 2 * t;
-      const uint32_t b0 = g < NO ? wpair(wrow) : 0u, b1 = g < NO ? wpair(wrow + 8) : 0u;
-      mma_16816(o, hh[kk], b0, b1);
-      mma_16816(o, hl[kk], b0, b1);
+    for (int kk = 0; kk < 4; kk += 2) {
+      const uint4 w = f3[kk / 2][lane];
+      mma_16816(o, hh[kk], w.x, w.y);
+      mma_16816(o, hl[kk], w.x, w.y);
+      mma_16816(o, hh[kk + 1], w.z, w.w);
+      mma_16816(o, hl[kk + 1], w.z, w.w);
     }
     if (ra < n) {
       if (2 * t < NO) out[(size_t)ra * NO + 2 * t] = o[0];
@@ -886,7 +915,7 @@ void features(const Hierarchy &h, int level, float *feat_dev, cudaStream_t s) {
 
 void mlp_forward_half(int32_t n, const uint16_t *w16_dev, const float *feat, float *out, cudaStream_t s) {
   if (n <= 0) return;
-  const int blocks = grid_for(((int64_t)n + 15) / 16, kTcWarps, 152 * 16);
+  const int blocks = grid_for(((int64_t)n + 15) / 16, kTcWarps, 152 * 20);  // four waves of resident blocks
   AMG_COUNT(), k_mlp_forward_tc<<<blocks, 32 * kTcWarps, 0, s>>>(n, reinterpret_cast<const __half *>(w16_dev), feat,
                                                                  out);
   AMG_LAUNCH_CHECK();
