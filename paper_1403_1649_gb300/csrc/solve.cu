@@ -243,36 +243,74 @@ constexpr int sell_min_blocks() { return sizeof(VT) == 4 ? 6 : 4; }
 // plain SpMV does not hold their accumulators in registers)
 // GATE: a batch's launch, skipping slices whose systems have all stopped
 // (compiled only into the batch instantiations)
-// With fused inner products the FP32-vector kernel needs more than the 40
-// registers of six resident blocks (it spilled there): four blocks, 64 registers.
-constexpr int kDotBlocks = 4;
+// With fused inner products: FP32 vectors need more than the 40 registers of six
+// resident blocks (they spilled there), four blocks of 64; FP64 vectors hold ten
+// entries and the row's operands in 80 registers, three blocks.  Ten entries: an FEM
+// slice has nine with the diagonal, which took two steps of eight (q = A p on 1024^2
+// rows; with the operands ahead the FEM solve went from 28.4 to 27.5 ms).
+template <class VT>
+constexpr int dot_blocks() { return sizeof(VT) == 4 ? 4 : 3; }
 template <class VT, int ND>
-constexpr int sell_launch_blocks() { return ND ? kDotBlocks : sell_min_blocks<VT>(); }
+constexpr int sell_launch_blocks() { return ND ? dot_blocks<VT>() : sell_min_blocks<VT>(); }
+
+// The row's own operands of the epilogue EPI and of the inner products.  They are
+// loaded with the first gathers: behind them, each was one more trip to L2 or HBM in
+// the chain of a slice (ops_ahead; not where the registers do not reach: the
+// polynomial's steps of several operands).
+template <class VT, int EPI, int ND>
+constexpr bool ops_ahead() { return EPI <= 1 || (sizeof(VT) == 4 && ND > 0); }
+template <class VT>
+struct RowOps {
+  VT rhs, dinv, c0, c1, c2, p0, p1, res, xin, s, u1, u2;
+  double q;
+};
+template <class VT, int EPI, int ND>
+__device__ __forceinline__ RowOps<VT> load_row_ops(const SellArgs<VT> &a, int32_t row) {
+  RowOps<VT> o;
+  if constexpr (EPI == E_RESID || EPI == E_RESID_POLY) o.rhs = a.rhs[row];
+  if constexpr (EPI >= E_DSCALE) o.dinv = a.dinv[row];
+  if constexpr (EPI == E_POLYPRE || EPI == E_HORNER_LAST) o.c0 = a.coef[3 * row];
+  if constexpr (EPI == E_POLYPRE || EPI == E_HORNER) o.c1 = a.coef[3 * row + 1];
+  if constexpr (EPI == E_POLYPRE || EPI == E_RESID_POLY) o.c2 = a.coef[3 * row + 2];
+  if constexpr (EPI == E_POLYPRE) {
+    o.p0 = a.p0[row];
+    o.p1 = a.p1[row];
+  }
+  if constexpr (EPI == E_HORNER || EPI == E_HORNER_LAST) o.res = a.res[row];
+  if constexpr (EPI == E_HORNER_LAST) o.xin = a.xin[row];
+  if constexpr (ND == 1) o.q = a.q64[row];
+  if constexpr (ND >= 2) {
+    o.s = a.x[row];
+    o.u1 = a.u1[row];
+  }
+  if constexpr (ND == 3) o.u2 = a.u2[row];
+  return o;
+}
 
 // row `row` of the epilogue EPI with the row's product y, and the launch's inner products
 template <class VT, int EPI, int ND>
-__device__ __forceinline__ void sell_epilogue(const SellArgs<VT> &a, int32_t row, VT y, double (&acc)[ND ? ND : 1]) {
+__device__ __forceinline__ void sell_epilogue(const SellArgs<VT> &a, int32_t row, VT y, const RowOps<VT> &w,
+                                              double (&acc)[ND ? ND : 1]) {
   VT o;
   if (EPI == E_Y) o = y;
-  else if (EPI == E_RESID) o = a.rhs[row] - y;
-  else if (EPI == E_DSCALE) o = a.dinv[row] * y;
-  else if (EPI == E_POLYPRE)
-    o = a.coef[3 * row] * a.p0[row] + a.coef[3 * row + 1] * a.p1[row] + a.coef[3 * row + 2] * (a.dinv[row] * y);
+  else if (EPI == E_RESID) o = w.rhs - y;
+  else if (EPI == E_DSCALE) o = w.dinv * y;
+  else if (EPI == E_POLYPRE) o = w.c0 * w.p0 + w.c1 * w.p1 + w.c2 * (w.dinv * y);
   else if (EPI == E_RESID_POLY) {
-    o = a.rhs[row] - y;
-    a.out2[row] = a.dinv[row] * (a.coef[3 * row + 2] * o);
+    o = w.rhs - y;
+    a.out2[row] = w.dinv * (w.c2 * o);
   } else if (EPI == E_HORNER)
-    o = a.dinv[row] * y + a.dinv[row] * (a.coef[3 * row + 1] * a.res[row]);
+    o = w.dinv * y + w.dinv * (w.c1 * w.res);
   else
-    o = a.xin[row] + (a.dinv[row] * y + a.dinv[row] * (a.coef[3 * row] * a.res[row]));
+    o = w.xin + (w.dinv * y + w.dinv * (w.c0 * w.res));
   a.out[row] = o;
   if constexpr (ND == 1) {
-    acc[0] += (double)o * a.q64[row];
+    acc[0] += (double)o * w.q;
   } else if constexpr (ND >= 2) {
-    const double oy = (double)o, sv = a.dot_y ? oy : (double)a.x[row];
+    const double oy = (double)o, sv = a.dot_y ? oy : (double)w.s;
     acc[0] += sv * oy;
-    acc[1] += sv * (double)a.u1[row];
-    if constexpr (ND == 3) acc[2] += sv * (double)a.u2[row];
+    acc[1] += sv * (double)w.u1;
+    if constexpr (ND == 3) acc[2] += sv * (double)w.u2;
   }
 }
 
@@ -285,8 +323,9 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
   double acc[ND ? ND : 1] = {0.0};
   // U entries of a row per step: 6 with FP32 vectors (a 7-point row without its
   // split-off diagonal in one step, at 40 registers), 8 with FP64
-  constexpr int U = sizeof(VT) == 4 ? 6 : 8;
+  constexpr int U = sizeof(VT) == 4 ? 6 : (ND > 0 ? 10 : 8);
   bool first = true, run = true, live = true;
+  constexpr bool kOpsAhead = ops_ahead<VT, EPI, ND>();
   // FP32 vectors at 64 registers wait for the predecessor after the first slice's
   // matrix loads have gone out; at 40 registers, and with FP64 vectors, that spills
   constexpr bool kAhead = sizeof(VT) == 4 && ND > 0;
@@ -309,6 +348,7 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
     }
     const int32_t row = sl * 32 + lane;
     VT y = VT(0), dg = VT(0), xr = VT(0);
+    RowOps<VT> own;
     const bool diag = !std::is_same<MV, double>::value && a.sdiag != nullptr && row < a.n;
     const int64_t base = a.sptr[sl];
     const int32_t width = (int32_t)((a.sptr[sl + 1] - base) >> 5);
@@ -350,6 +390,7 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
           if (diag) dg = (VT)ld_stream(a.sdiag + row);
           enter(sl);
           if (diag) xr = a.x[row];
+          if (kOpsAhead) own = load_row_ops<VT, EPI, ND>(a, min(row, a.n - 1));
         }
         VT xv[S];
 #pragma unroll
@@ -383,7 +424,10 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
             v[q] = ld_stream(vp + 32 * (e + q));
           }
         }
-        if (e == 0) enter(sl);
+        if (e == 0) {
+          enter(sl);
+          if (kOpsAhead) own = load_row_ops<VT, EPI, ND>(a, min(row, a.n - 1));
+        }
         VT xv[U];
 #pragma unroll
         for (int q = 0; q < U; ++q)
@@ -396,6 +440,7 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
     enter(sl);  // a slice without entries has not waited yet
     if (!run) return;
     if (GATE && !live) continue;
+    if (!kOpsAhead || width == 0) own = load_row_ops<VT, EPI, ND>(a, min(row, a.n - 1));
     if (diag) {
       if (width == 0) {  // a row without off-diagonal entries
         dg = (VT)a.sdiag[row];
@@ -403,7 +448,7 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
       }
       y += dg * xr;
     }
-    if (row < a.n) sell_epilogue<VT, EPI, ND>(a, row, y, acc);
+    if (row < a.n) sell_epilogue<VT, EPI, ND>(a, row, y, own, acc);
   }
   enter(a.nslices);  // a warp without a slice
   if (!run) return;
@@ -485,11 +530,18 @@ __global__ void __launch_bounds__(kThreads) k_sell_small(SellArgs<VT> a, int wl)
         if (c[q] >= 0) y += v[q] * xv[q];
     };
     bool run = true;
+    RowOps<VT> own;
+    VT xr = VT(0);
     step(0, [&] {
-      if (!first) return;
-      first = false;
-      pdl_wait();
-      run = !(a.pred && *a.pred == 0);
+      if (first) {
+        first = false;
+        pdl_wait();
+        run = !(a.pred && *a.pred == 0);
+      }
+      if (mine) {
+        if (!std::is_same<MV, double>::value && a.sdiag) xr = a.x[row];
+        own = load_row_ops<VT, EPI, ND>(a, row);
+      }
     });
     if (!run) return;  // the same in every thread of the grid
     const bool live = !GATE || (in && a.live[sl]);  // of a batch: a dead slice is not stored
@@ -503,8 +555,8 @@ __global__ void __launch_bounds__(kThreads) k_sell_small(SellArgs<VT> a, int wl)
         for (int q = 1; q < wps; ++q) y += sh[wid + q][lane];
     }
     if (mine && live) {
-      if (!std::is_same<MV, double>::value && a.sdiag) y += dg * a.x[row];
-      sell_epilogue<VT, EPI, ND>(a, row, y, acc);
+      if (!std::is_same<MV, double>::value && a.sdiag) y += dg * xr;
+      sell_epilogue<VT, EPI, ND>(a, row, y, own, acc);
     }
   }
   if (first) {  // a block without a slice
@@ -695,6 +747,7 @@ __global__ void __launch_bounds__(kThreads, post_blocks<VT>()) k_post(PostArgs<V
     };
     bool live = true;
     VT xg = VT(0), ri = VT(0), xi = VT(0);
+    double qi = 0.0;
     auto enter = [&] {  // wait (first slice), then the row's own operands
       if (first) {
         first = false;
@@ -705,6 +758,7 @@ __global__ void __launch_bounds__(kThreads, post_blocks<VT>()) k_post(PostArgs<V
       xg = a.xc[g];
       ri = a.r[rr];
       xi = a.x[rr];
+      if constexpr (ND == 1) qi = a.q64[rr];
     };
     using S4 = std::integral_constant<int, 4>;
     using S6 = std::integral_constant<int, 6>;
@@ -720,7 +774,7 @@ __global__ void __launch_bounds__(kThreads, post_blocks<VT>()) k_post(PostArgs<V
     if (row < a.n) {
       const VT o = (xi + p * xg) + w * (ri - (own * xg + y));
       a.out[row] = o;
-      if constexpr (ND == 1) acc[0] += (double)o * a.q64[row];
+      if constexpr (ND == 1) acc[0] += (double)o * qi;
     }
   }
   if (first) {  // a warp without a slice
@@ -1688,9 +1742,10 @@ inline int default_sell_grid(const Level &L) {
   return grid_for((int64_t)L.nslices, kWarps, sell_min_blocks<VT>() * 152);
 }
 // launches with fused inner products: at most one wave of their kernel, which
-// runs kDotBlocks blocks per SM (a second, short wave and its reductions took the
+// runs dot_blocks per SM (a second, short wave and its reductions took the
 // 190k-row level of 128^3 from 10 to 17 us)
-inline int dot_grid(const Level &L) { return std::min(L.sell_blocks, kDotBlocks * 152); }
+template <class VT>
+inline int dot_grid(const Level &L) { return std::min(L.sell_blocks, dot_blocks<VT>() * 152); }
 // launches without inner products have no partial-sum buffer to fill, so the
 // autotuner may give them up to one warp per slice; by default they take the
 // same wave of resident blocks (one warp per slice measured slower on the 128^3
@@ -1775,7 +1830,7 @@ struct Engine {
     if (h.batched)
       klaunch(k_sell<MV, VT, EPI, 0, true>, plain_grid(L), kThreads, s, a);
     else
-      klaunch(k_sell<MV, VT, EPI, ND, false>, ND ? dot_grid(L) : plain_grid(L), kThreads, s, a);
+      klaunch(k_sell<MV, VT, EPI, ND, false>, ND ? dot_grid<VT>(L) : plain_grid(L), kThreads, s, a);
     check();
   }
 
@@ -2111,7 +2166,7 @@ struct Engine {
       a.u1 = h.r;
       a.fin = fin_args(0, FIN_ALPHA, L0.partials);
       a.pred = active;
-      klaunch(k_sell<double, double, E_Y, 2, false>, outer_grid(L0), kThreads, s, a);
+      klaunch(k_sell<double, double, E_Y, 2, false>, std::min(outer_grid(L0), dot_blocks<double>() * 152), kThreads, s, a);
       check();
     }
     // x, r update, the next preconditioner input, and the end of the iteration
