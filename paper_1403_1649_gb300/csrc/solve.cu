@@ -26,17 +26,6 @@ namespace amg {
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 
-// the scalar step that follows a kernel's inner products (run_fin)
-enum FinKind { FIN_K1 = 0, FIN_K3 = 1, FIN_ALPHA = 2, FIN_BETA = 3 };
-
-struct FinArgs {
-  int kind;
-  double *slots;
-  const int *restart;  // FIN_BETA
-  double *partials;    // ndot x kRedBlocks
-  unsigned *ticket;    // 0 between launches
-};
-
 template <class VT>
 struct SellArgs {
   int32_t n, nslices;
@@ -51,11 +40,12 @@ struct SellArgs {
   const VT *rhs;  // right-hand side (residual epilogues)
   const VT *xin;  // the iterate that the last Horner step updates
   // fused inner products with left operand s = x (dot_y: the output): ND = 2:
-  // {s.out, s.u1}, ND = 3: {s.out, s.u1, s.u2}, ND = 1: {out.q64}; then fin
+  // {s.out, s.u1}, ND = 3: {s.out, s.u1, s.u2}, ND = 5: {x.out, x.u1, out.out, out.u1,
+  // u1.u1}, ND = 1: {out.q64}; the blocks' sums to partials
   const VT *u1, *u2;
   const double *q64;
   int dot_y;
-  FinArgs fin;
+  double *partials;
   const int *pred;
   // polynomial smoother operands
   const VT *dinv;     // 1 / A_ii
@@ -83,55 +73,105 @@ template <class MV> __device__ __forceinline__ MV ld_stream(const MV *p) { retur
 template <class MV> constexpr bool kPairs = std::is_same<MV, float>::value;
 template <class MV> constexpr bool kHalfPairs = std::is_same<MV, __nv_bfloat16>::value;
 
-// ---- inner products and the scalars they lead to, in one launch
-// A kernel that ends with inner products also forms the scalars of Alg. 5 or of
-// the outer iteration: its blocks publish their partial sums, take a ticket, and
-// the block that finishes last sums all partials in block order (deterministic)
-// and runs the scalar step.  A separate one-block kernel for that costs 3-5 us of
-// dependent latency in the chain even with programmatic dependent launch; the
-// last block adds ~1.5 us (128^3, 27 outer iterations: 36 such kernels an
-// iteration removed).
-// GB300 issues an FP64 warp instruction every 16 cycles an SM, so the reduction
-// counts them: the block's values go through shared memory and one warp per
-// product adds 8 values a lane and 5 shuffles (12 warp instructions a product,
-// against 45 with a shuffle tree in each of the 8 warps).
-// the scalar step, by one thread, from the totals of the kernel's inner products
-__device__ __forceinline__ void run_fin(const FinArgs &f, const double *tot) {
-  double *slots = f.slots;
-  if (f.kind == FIN_K1) {
-    // Alg. 5 after v = A c: rho_1 and alpha_1 (CG: c^T v, c^T r; GMRES: ||v||^2, v^T r)
-    slots[S_RHO1] = tot[0];
-    slots[S_A1] = tot[1];
-    slots[S_S1] = tot[1] / tot[0];
-  } else if (f.kind == FIN_K3) {
-    // Alg. 5 after w = A d: gamma, beta, alpha_2 (CG: d^T v, d^T w, d^T r~; GMRES
-    // with w in place of d on the left), rho_2 = beta - gamma^2 / rho_1 and the
-    // combination weights; the products come as {beta, gamma, alpha_2}
-    const double bet = tot[0], gam = tot[1], a2 = tot[2];
-    const double g1 = gam / slots[S_RHO1];
-    const double cd = a2 / (bet - gam * g1);
-    slots[S_GAM] = gam;
-    slots[S_BET] = bet;
-    slots[S_A2] = a2;
-    slots[S_CC] = slots[S_S1] - g1 * cd;
-    slots[S_CD] = cd;
-  } else if (f.kind == FIN_ALPHA) {  // outer flexible CG: alpha = p^T r / p^T q
-    slots[S_PQ] = tot[0];
-    slots[S_PR] = tot[1];
-    slots[S_ALPHA] = tot[1] / tot[0];
-  } else {  // beta = -(z^T q_old) / (p_old^T q_old), 0 right after a restart
-    slots[S_ZQ] = tot[0];
-    slots[S_BETA] = *f.restart != 0 ? 0.0 : -tot[0] / slots[S_PQ];
+// ---- inner products
+// A kernel with inner products stores its blocks' sums, and every block of the kernel
+// that needs the totals adds them up itself, in the same fixed order (sum_partials_of):
+// the sums over the grid are no launch, no ticket and no trip of a last block through
+// fence, atomic, partials and scalars, which added ~3.5 us to each of 12 kernels of an
+// iteration (1.5-2 us now, in the kernel that reads them: 128^3 step 16.9 -> 16.5 ms,
+// FEM 1024^2 solve 28.3 -> 26.1, learned 501^2 8.0 -> 7.0, 700^2 re-setup + solve 35.4 ->
+// 32.3, 64^2 step 3.25 -> 3.07).  What the host or a predicate of later launches needs (the end of an
+// outer iteration) is still formed by the last block (grid_totals).
+// GB300 issues an FP64 warp instruction every 16 cycles an SM, so the reductions
+// count them: the block's values go through shared memory and one warp per product
+// adds 8 values a lane and 5 shuffles (12 warp instructions a product, against 45
+// with a shuffle tree in each of the 8 warps).
+
+// the block's sums of ND inner products to partials[k kRedBlocks + block].  `step`:
+// only the threads of every step-th warp hold a value.  Every thread calls it.
+template <int ND>
+__device__ __forceinline__ void store_dots(const double (&acc)[ND], int step, double *partials) {
+  __shared__ double sh[ND][kThreads];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < ND; ++k) sh[k][threadIdx.x] = acc[k];
+  __syncthreads();
+  if (wid < ND) {
+    double v = sh[wid][lane];
+    for (int q = step; q < kWarps; q += step) v += sh[wid][q * 32 + lane];
+    v = warp_sum(v);
+    if (lane == 0) partials[wid * kRedBlocks + blockIdx.x] = v;
   }
+}
+
+// kernels that add up a product's partials run at most two blocks of kSumThreads an SM:
+// fewer blocks read the same partials, and each row's loads overlap the sums once
+constexpr int kSumThreads = 512;
+constexpr int kSumWarps = kSumThreads / 32;
+inline int sum_grid(int64_t n) { return grid_for(n, kSumThreads, 304); }
+
+// tot[k] = sum of the nb partials of product k, the same bits in every block; valid in
+// warp 0 (all lanes).  Every thread of the block calls it.  An FP64 addition takes ~60
+// cycles to its result: up to 128 partials warp 0 sums alone (four loads a lane, all
+// products side by side), more are shared among the block's warps.
+template <int ND>
+__device__ __forceinline__ void sum_partials_of(const double *partials, int nb, double (&tot)[ND]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  constexpr int kAhead = 4;
+  auto four = [&](int k, int j0, int stride) {
+    double v[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      v[u] = j0 + u * stride < nb ? __ldcg(partials + k * kRedBlocks + j0 + u * stride) : 0.0;
+    return (v[0] + v[1]) + (v[2] + v[3]);
+  };
+  if (nb <= 32 * kAhead) {
+    if (wid == 0) {
+#pragma unroll
+      for (int k = 0; k < ND; ++k) tot[k] = four(k, lane, 32);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < ND; ++k) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], o);
+    }
+    return;
+  }
+  constexpr int kPer = ND == 1 ? 8 : (ND == 2 ? 8 : (ND == 3 ? 4 : 3));  // warps per product
+  static_assert(kPer * ND <= kSumWarps, "");
+  __shared__ double sh[ND][8];
+  const int k = wid / kPer, sub = wid % kPer;
+  if (k < ND) {
+    double t = 0.0;
+    for (int j0 = sub * 32 + lane; j0 < nb; j0 += kAhead * kPer * 32) t += four(k, j0, kPer * 32);
+    t = warp_sum(t);
+    if (lane == 0) sh[k][sub] = t;
+  }
+  __syncthreads();
+  if (wid == 0) {
+#pragma unroll
+    for (int q = 0; q < ND; ++q) tot[q] = lane < kPer ? sh[q][lane] : 0.0;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < ND; ++q) tot[q] += __shfl_xor_sync(0xffffffffu, tot[q], o);
+  }
+}
+
+// rows [r0, r1) of this block: equal contiguous shares, so that every SM has the same
+// number of load batches
+__device__ __forceinline__ void block_rows(int32_t n, int32_t &r0, int32_t &r1) {
+  const int32_t share = (n + gridDim.x - 1) / gridDim.x, up = (share + 31) & ~31;
+  r0 = (int32_t)min((int64_t)n, (int64_t)blockIdx.x * up);
+  r1 = (int32_t)min((int64_t)n, (int64_t)r0 + up);
 }
 
 // totals of ND inner products over the grid; true in thread 0 of the last block
 // only, with the totals in tot.  `step`: only the threads of every step-th warp
 // hold a value.  Every thread of the block calls it, all blocks of the grid.
-template <int ND>
+template <int ND, int T = kThreads>  // T threads a block
 __device__ __forceinline__ bool grid_totals(const double (&acc)[ND], int step, double *partials, unsigned *ticket,
                                             double (&tot)[ND]) {
-  __shared__ double sh[ND][kThreads];
+  __shared__ double sh[ND][T];
   __shared__ double tot_sh[ND];
   __shared__ bool last;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -140,7 +180,7 @@ __device__ __forceinline__ bool grid_totals(const double (&acc)[ND], int step, d
   __syncthreads();
   if (wid < ND) {
     double v = sh[wid][lane];
-    for (int q = step; q < kWarps; q += step) v += sh[wid][q * 32 + lane];
+    for (int q = step; q < T / 32; q += step) v += sh[wid][q * 32 + lane];
     v = warp_sum(v);
     if (lane == 0) {
       if (gridDim.x == 1) {
@@ -159,22 +199,22 @@ __device__ __forceinline__ bool grid_totals(const double (&acc)[ND], int step, d
     __threadfence();
 #pragma unroll
     for (int k = 0; k < ND; ++k) {
-      double v[kRedBlocks / kThreads + 1];
+      double v[kRedBlocks / T + 1];
 #pragma unroll
-      for (int u = 0; u <= kRedBlocks / kThreads; ++u) {
-        const int j = threadIdx.x + u * kThreads;
+      for (int u = 0; u <= kRedBlocks / T; ++u) {
+        const int j = threadIdx.x + u * T;
         v[u] = j < (int)gridDim.x ? __ldcg(partials + k * kRedBlocks + j) : 0.0;
       }
       double t = v[0];
 #pragma unroll
-      for (int u = 1; u <= kRedBlocks / kThreads; ++u)
-        if (u * kThreads < (int)gridDim.x) t += v[u];
+      for (int u = 1; u <= kRedBlocks / T; ++u)
+        if (u * T < (int)gridDim.x) t += v[u];
       sh[k][threadIdx.x] = t;
     }
     __syncthreads();
     if (wid < ND) {
       double v = sh[wid][lane];
-      for (int q = 1; q < kWarps && q * 32 < (int)gridDim.x; ++q) v += sh[wid][q * 32 + lane];
+      for (int q = 1; q < T / 32 && q * 32 < (int)gridDim.x; ++q) v += sh[wid][q * 32 + lane];
       v = warp_sum(v);
       if (lane == 0) tot_sh[wid] = v;
     }
@@ -185,12 +225,6 @@ __device__ __forceinline__ bool grid_totals(const double (&acc)[ND], int step, d
 #pragma unroll
   for (int k = 0; k < ND; ++k) tot[k] = tot_sh[k];
   return true;
-}
-
-template <int ND>
-__device__ __forceinline__ void grid_dots(const double (&acc)[ND], int step, const FinArgs &f) {
-  double tot[ND];
-  if (grid_totals<ND>(acc, step, f.partials, f.ticket, tot)) run_fin(f, tot);
 }
 
 // per-block partial sums of one inner product -> partials[block] (no finish)
@@ -246,8 +280,7 @@ constexpr int sell_min_blocks() { return sizeof(VT) == 4 ? 6 : 4; }
 // With fused inner products: FP32 vectors need more than the 40 registers of six
 // resident blocks (they spilled there), four blocks of 64; FP64 vectors hold ten
 // entries and the row's operands in 80 registers, three blocks.  Ten entries: an FEM
-// slice has nine with the diagonal, which took two steps of eight (q = A p on 1024^2
-// rows; with the operands ahead the FEM solve went from 28.4 to 27.5 ms).
+// slice has nine with the diagonal, which took two steps of eight.
 template <class VT>
 constexpr int dot_blocks() { return sizeof(VT) == 4 ? 4 : 3; }
 template <class VT, int ND>
@@ -307,10 +340,15 @@ __device__ __forceinline__ void sell_epilogue(const SellArgs<VT> &a, int32_t row
   if constexpr (ND == 1) {
     acc[0] += (double)o * w.q;
   } else if constexpr (ND >= 2) {
-    const double oy = (double)o, sv = a.dot_y ? oy : (double)w.s;
+    const double oy = (double)o, sv = ND != 5 && a.dot_y ? oy : (double)w.s, u1 = (double)w.u1;
     acc[0] += sv * oy;
-    acc[1] += sv * (double)w.u1;
+    acc[1] += sv * u1;
     if constexpr (ND == 3) acc[2] += sv * (double)w.u2;
+    if constexpr (ND == 5) {
+      acc[2] += oy * oy;
+      acc[3] += oy * u1;
+      acc[4] += u1 * u1;
+    }
   }
 }
 
@@ -323,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
   double acc[ND ? ND : 1] = {0.0};
   // U entries of a row per step: 6 with FP32 vectors (a 7-point row without its
   // split-off diagonal in one step, at 40 registers), 8 with FP64
-  constexpr int U = sizeof(VT) == 4 ? 6 : (ND > 0 ? 10 : 8);
+  constexpr int U = sizeof(VT) == 4 ? 6 : (ND == 2 ? 10 : 8);
   bool first = true, run = true, live = true;
   constexpr bool kOpsAhead = ops_ahead<VT, EPI, ND>();
   // FP32 vectors at 64 registers wait for the predecessor after the first slice's
@@ -452,7 +490,7 @@ __global__ void __launch_bounds__(kThreads, sell_launch_blocks<VT, ND>()) k_sell
   }
   enter(a.nslices);  // a warp without a slice
   if (!run) return;
-  if constexpr (ND > 0) grid_dots<ND>(acc, 1, a.fin);
+  if constexpr (ND > 0) store_dots<ND>(acc, 1, a.partials);
 }
 
 // The product on a small level (at most kSmallSlices slices): 2^wl warps share a
@@ -563,7 +601,7 @@ __global__ void __launch_bounds__(kThreads) k_sell_small(SellArgs<VT> a, int wl)
     pdl_wait();
     if (a.pred && *a.pred == 0) return;
   }
-  if constexpr (ND > 0) grid_dots<ND>(acc, wps, a.fin);
+  if constexpr (ND > 0) store_dots<ND>(acc, wps, a.partials);
 }
 
 // out = wd * rhs: damped Jacobi from a zero initial guess
@@ -688,8 +726,8 @@ struct PostArgs {
   const unsigned char *live;  // batch
   const VT *x, *r, *xc;
   VT *out;
-  const double *q64;  // ND = 1: out . q64
-  FinArgs fin;
+  const double *q64;  // ND = 1: out . q64, the blocks' sums to partials
+  double *partials;
   const int *pred;
 };
 
@@ -781,7 +819,7 @@ __global__ void __launch_bounds__(kThreads, post_blocks<VT>()) k_post(PostArgs<V
     pdl_wait();
     if (a.pred && *a.pred == 0) return;
   }
-  if constexpr (ND > 0) grid_dots<ND>(acc, 1, a.fin);
+  if constexpr (ND > 0) store_dots<ND>(acc, 1, a.partials);
 }
 
 // exact coarsest solve x = A_L^-1 b (one warp per row, FP64 accumulation)
@@ -899,46 +937,138 @@ __device__ __forceinline__ void axpy_rt_rows(int32_t i, int32_t step, int32_t en
   }
 }
 
-// r~ = r - (alpha_1/rho_1) v, the next smoothing start x0 = wd * r~, and the
-// test of Alg. 5 in the last block: the second inner step runs iff the enclosing
-// step runs and ||r~|| > t ||r||.  A skipped enclosing step clears the flag.
+// r~ = r - (alpha_1/rho_1) v and the next smoothing start x0 = wd * r~, from the sums
+// {c.v, c.r, v.v, v.r, r.r} of the product before (rho_1 and alpha_1: c.v and c.r, or
+// v.v and v.r in the GMRES variant), and the test of Alg. 5: the second inner step runs
+// iff the enclosing step runs and ||r~|| > t ||r||, with ||r~||^2 = r.r - 2 s v.r +
+// s^2 v.v.  The subtraction keeps about 2^-50 of r.r, far below t^2 r.r for any
+// threshold above kTestBySums; smaller ones take k_test on r~ itself.  A skipped
+// enclosing step clears the flag.
+constexpr double kTestBySums = 1e-4;
 template <class VT>
-__global__ void __launch_bounds__(kThreads) k_axpy_rt(int32_t n, const VT *r, const VT *v, VT *rt,
-                                                      const VT *__restrict__ wd, VT *x0, double t, double *slots,
-                                                      int *flag, double *part, unsigned *ticket, const int *pred) {
+__global__ void __launch_bounds__(kSumThreads) k_axpy_rt(int32_t n, const VT *r, const VT *v, VT *rt,
+                                                         const VT *__restrict__ wd, VT *x0, double t, int gmres,
+                                                         double *slots, int *flag, const double *part, int nb,
+                                                         const int *pred) {
+  __shared__ double s1_sh;
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *flag = 0;
     return;
   }
-  const VT s1 = (VT)slots[S_S1];
-  double acc[2] = {0.0, 0.0};
-  const int32_t step = gridDim.x * blockDim.x;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kRows * step)
-    axpy_rt_rows<VT>(i, step, n, s1, r, v, rt, wd, x0, acc);
-  double tot[2];
-  if (grid_totals<2>(acc, 1, part, ticket, tot)) {
-    slots[S_NRT2] = tot[0];
-    slots[S_NR2] = tot[1];
-    const bool second = !(sqrt(tot[0]) <= t * sqrt(tot[1]));
-    *flag = second ? 1 : 0;
-    if (second) slots[S_TAKEN] += 1.0;  // cycle trace (one thread)
+  int32_t r0, end;
+  block_rows(n, r0, end);
+  constexpr int32_t step = kSumThreads;
+  const int32_t i0 = r0 + threadIdx.x;
+  VT rv[kRows], vv[kRows], wv[kRows];
+  auto load = [&](int32_t i) {
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (i + u * step < end) {
+        rv[u] = r[i + u * step];
+        vv[u] = v[i + u * step];
+        wv[u] = wd[i + u * step];
+      }
+  };
+  load(i0);  // the first rows come with the partials
+  double tot[5];
+  sum_partials_of<5>(part, nb, tot);
+  if (threadIdx.x == 0) {
+    const double rho1 = gmres ? tot[2] : tot[0], a1 = gmres ? tot[3] : tot[1], s1 = a1 / rho1;
+    s1_sh = s1;
+    if (blockIdx.x == 0) {
+      slots[S_RHO1] = rho1;
+      slots[S_A1] = a1;
+      slots[S_S1] = s1;
+      if (t >= kTestBySums) {
+        const double rt2 = (tot[4] - s1 * tot[3]) - s1 * (tot[3] - s1 * tot[2]);
+        const bool second = !(rt2 <= t * t * tot[4]);
+        *flag = second ? 1 : 0;
+        if (second) slots[S_TAKEN] += 1.0;  // cycle trace
+      }
+    }
+  }
+  __syncthreads();
+  const VT s1 = (VT)s1_sh;
+  for (int32_t i = i0; i < end; i += kRows * step) {
+    if (i != i0) load(i);
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (i + u * step < end) {
+        const VT ti = rv[u] - s1 * vv[u];
+        rt[i + u * step] = ti;
+        x0[i + u * step] = wv[u] * ti;
+      }
   }
 }
 
-// x_{k+1} = (alpha1/rho1) c, or the two-step combination when it was taken
+// the test of Alg. 5 on ||r~|| and ||r|| themselves (thresholds below kTestBySums)
 template <class VT>
-__global__ void k_combine(int32_t n, const VT *__restrict__ c, const VT *__restrict__ d, VT *__restrict__ x,
-                          const double *__restrict__ slots, const int *__restrict__ flag, const int *pred) {
+__global__ void __launch_bounds__(kThreads) k_test(int32_t n, const VT *r, const VT *rt, double t, double *slots,
+                                                   int *flag, double *part, unsigned *ticket, const int *pred) {
+  pdl_trigger();
+  pdl_wait();
+  if (pred && *pred == 0) return;
+  double acc[2] = {0.0, 0.0}, tot[2];
+  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    acc[0] += (double)rt[i] * (double)rt[i];
+    acc[1] += (double)r[i] * (double)r[i];
+  }
+  if (grid_totals<2>(acc, 1, part, ticket, tot)) {
+    const bool second = !(sqrt(tot[0]) <= t * sqrt(tot[1]));
+    *flag = second ? 1 : 0;
+    if (second) slots[S_TAKEN] += 1.0;
+  }
+}
+
+// x_{k+1} = (alpha1/rho1) c, or the two-step combination when it was taken: from the
+// sums {beta, gamma, alpha_2} of the product w = A d (CG: d.w, d.v, d.r~; GMRES with w
+// in place of d on the left), rho_2 = beta - gamma^2 / rho_1
+template <class VT>
+__global__ void __launch_bounds__(kSumThreads) k_combine(int32_t n, const VT *c, const VT *d, VT *x,
+                                                         const double *slots, const int *flag, const double *part,
+                                                         int nb, const int *pred) {
+  __shared__ double w_sh[2];
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
   const bool two = *flag != 0;
-  const VT cc = (VT)(two ? slots[S_CC] : slots[S_S1]);
-  const VT cd = (VT)(two ? slots[S_CD] : 0.0);
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    x[i] = two ? cc * c[i] + cd * d[i] : cc * c[i];
+  int32_t r0, end;
+  block_rows(n, r0, end);
+  constexpr int32_t step = kSumThreads;
+  const int32_t i0 = r0 + threadIdx.x;
+  VT cv[kRows], dv[kRows];
+  auto load = [&](int32_t i) {
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (i + u * step < end) {
+        cv[u] = c[i + u * step];
+        dv[u] = two ? d[i + u * step] : VT(0);
+      }
+  };
+  load(i0);
+  if (two) {
+    const double rho1 = slots[S_RHO1], s1 = slots[S_S1];
+    double tot[3];
+    sum_partials_of<3>(part, nb, tot);
+    if (threadIdx.x == 0) {
+      const double g1 = tot[1] / rho1, cd = tot[2] / (tot[0] - tot[1] * g1);
+      w_sh[0] = s1 - g1 * cd;
+      w_sh[1] = cd;
+    }
+  } else if (threadIdx.x == 0) {
+    w_sh[0] = slots[S_S1];
+    w_sh[1] = 0.0;
+  }
+  __syncthreads();
+  const VT cc = (VT)w_sh[0], cd = (VT)w_sh[1];
+  for (int32_t i = i0; i < end; i += kRows * step) {
+    if (i != i0) load(i);
+#pragma unroll
+    for (int u = 0; u < kRows; ++u)
+      if (i + u * step < end) x[i + u * step] = two ? cc * cv[u] + cd * dv[u] : cc * cv[u];
+  }
 }
 
 // ---------------------------------------------------------------- outer FCG (FP64)
@@ -964,42 +1094,59 @@ __global__ void k_from_vt(int32_t n, const VT *__restrict__ zin, double *__restr
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) z[i] = (double)zin[i];
 }
 
-// z^T q and beta of the outer flexible CG where the cycle has no product to fuse
-// them into (a hierarchy of one level)
+// z^T q of the outer flexible CG where the cycle has no product to fuse it into (a
+// hierarchy of one level)
 template <class VT>
 __global__ void __launch_bounds__(kThreads) k_dot_zq(int32_t n, const VT *__restrict__ z, const double *__restrict__ q,
-                                                     FinArgs fin, const int *pred) {
+                                                     double *part, const int *pred) {
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
   double acc[1] = {0.0};
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     acc[0] += (double)z[i] * q[i];
-  grid_dots<1>(acc, 1, fin);
+  store_dots<1>(acc, 1, part);
 }
 
-// p = z + beta p (beta = 0 right after a restart); z in the cycle's vector type
+// p = z + beta p, beta = -(z^T q_old) / (p_old^T q_old) from z^T q's partials (0 right
+// after a restart); z in the cycle's vector type
 template <class VT>
-__global__ void k_fcg_p(int32_t n, const VT *z, double *p, const double *slots, const int *restart,
-                        const int *pred) {
+__global__ void __launch_bounds__(kSumThreads) k_fcg_p(int32_t n, const VT *z, double *p, double *slots,
+                                                       const int *restart, const double *part, int nb,
+                                                       const int *pred) {
+  __shared__ double beta_sh;
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
   const bool rs = *restart != 0;
-  const double beta = slots[S_BETA];
-  const int32_t step = gridDim.x * blockDim.x;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kRows * step) {
-    VT zv[kRows];
-    double pv[kRows];
+  const double pq = slots[S_PQ];
+  int32_t r0, end;
+  block_rows(n, r0, end);
+  const int32_t i0 = r0 + threadIdx.x;
+  VT zv[kRows];
+  double pv[kRows];
+  auto load = [&](int32_t i) {
 #pragma unroll
     for (int u = 0; u < kRows; ++u)
-      if (i + u * step < n) {
-        zv[u] = z[i + u * step];
-        pv[u] = p[i + u * step];
+      if (i + u * kSumThreads < end) {
+        zv[u] = z[i + u * kSumThreads];
+        pv[u] = p[i + u * kSumThreads];
       }
+  };
+  load(i0);  // the first rows come with the partials
+  double tot[1];
+  sum_partials_of<1>(part, nb, tot);
+  if (threadIdx.x == 0) {
+    beta_sh = rs ? 0.0 : -tot[0] / pq;
+    if (blockIdx.x == 0) slots[S_ZQ] = tot[0];
+  }
+  __syncthreads();
+  const double beta = beta_sh;
+  for (int32_t i = i0; i < end; i += kRows * kSumThreads) {
+    if (i != i0) load(i);
 #pragma unroll
     for (int u = 0; u < kRows; ++u)
-      if (i + u * step < n) p[i + u * step] = rs ? (double)zv[u] : (double)zv[u] + beta * pv[u];
+      if (i + u * kSumThreads < end) p[i + u * kSumThreads] = rs ? (double)zv[u] : (double)zv[u] + beta * pv[u];
   }
 }
 
@@ -1012,57 +1159,80 @@ struct FcgState {
 // kRows rows i, i + step, ... < end of the update of x and r, of the next
 // preconditioner input rvt (nullable) and its smoothing start x0, and of ||r||^2
 template <class VT>
-__device__ __forceinline__ void fcg_update_rows(int32_t i, int32_t step, int32_t end, double alpha, double *x,
-                                                double *r, const double *p, const double *q, VT *rvt,
-                                                const VT *__restrict__ wd, VT *x0, double &acc) {
+struct FcgRows {
   double xv[kRows], rv[kRows], pv[kRows], qv[kRows];
   VT wv[kRows];
+  __device__ __forceinline__ void load(int32_t i, int32_t step, int32_t end, const double *x, const double *r,
+                                       const double *p, const double *q, const VT *__restrict__ wd) {
 #pragma unroll
-  for (int u = 0; u < kRows; ++u) {
-    const int32_t k = i + u * step;
-    if (k < end) {
-      xv[u] = x[k];
-      pv[u] = p[k];
-      rv[u] = r[k];
-      qv[u] = q[k];
-      wv[u] = wd[k];
+    for (int u = 0; u < kRows; ++u) {
+      const int32_t k = i + u * step;
+      if (k < end) {
+        xv[u] = x[k];
+        pv[u] = p[k];
+        rv[u] = r[k];
+        qv[u] = q[k];
+        wv[u] = wd[k];
+      }
     }
   }
+  __device__ __forceinline__ void apply(int32_t i, int32_t step, int32_t end, double alpha, double *x, double *r,
+                                        VT *rvt, VT *x0, double &acc) {
 #pragma unroll
-  for (int u = 0; u < kRows; ++u) {
-    const int32_t k = i + u * step;
-    if (k < end) {
-      x[k] = xv[u] + alpha * pv[u];
-      const double ri = rv[u] - alpha * qv[u];
-      r[k] = ri;
-      acc += ri * ri;
-      const VT v = (VT)ri;
-      if (rvt) rvt[k] = v;
-      x0[k] = wv[u] * v;
+    for (int u = 0; u < kRows; ++u) {
+      const int32_t k = i + u * step;
+      if (k < end) {
+        x[k] = xv[u] + alpha * pv[u];
+        const double ri = rv[u] - alpha * qv[u];
+        r[k] = ri;
+        acc += ri * ri;
+        const VT v = (VT)ri;
+        if (rvt) rvt[k] = v;
+        x0[k] = wv[u] * v;
+      }
     }
   }
-}
+};
 
+// alpha = p^T r / p^T q from the partials of the product q = A p;
 // x += alpha p;  r -= alpha q;  the preconditioner input (in reduced precision
 // also rounded to VT) and its smoothing start x0 = wd r.  The last block ends the
 // outer iteration: relative residual into the history, iteration count,
 // convergence / breakdown status (deactivates the following launches).
 template <class VT>
-__global__ void __launch_bounds__(kThreads) k_fcg_update(int32_t n, double *x, double *r, const double *p,
-                                                         const double *q, double *slots, double *part,
-                                                         unsigned *ticket, VT *rvt, const VT *__restrict__ wd,
-                                                         VT *x0, FcgState st, const int *pred) {
+__global__ void __launch_bounds__(kSumThreads, 2) k_fcg_update(int32_t n, double *x, double *r, const double *p,
+                                                            const double *q, double *slots, const double *pq_part,
+                                                            int nb, double *part, unsigned *ticket, VT *rvt,
+                                                            const VT *__restrict__ wd, VT *x0, FcgState st,
+                                                            const int *pred) {
+  __shared__ double alpha_sh, pq_sh;
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
-  const double alpha = slots[S_ALPHA];
+  int32_t r0, end;
+  block_rows(n, r0, end);
+  const int32_t i0 = r0 + threadIdx.x;
+  FcgRows<VT> rows;
+  rows.load(i0, kSumThreads, end, x, r, p, q, wd);  // the first rows come with the partials
+  {
+    double tot[2];
+    sum_partials_of<2>(pq_part, nb, tot);
+    if (threadIdx.x == 0) {
+      pq_sh = tot[0];
+      alpha_sh = tot[1] / tot[0];
+    }
+    __syncthreads();
+  }
+  const double alpha = alpha_sh;
   double acc[1] = {0.0};
-  const int32_t step = gridDim.x * blockDim.x;
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += kRows * step)
-    fcg_update_rows<VT>(i, step, n, alpha, x, r, p, q, rvt, wd, x0, acc[0]);
+  for (int32_t i = i0; i < end; i += kRows * kSumThreads) {
+    if (i != i0) rows.load(i, kSumThreads, end, x, r, p, q, wd);
+    rows.apply(i, kSumThreads, end, alpha, x, r, rvt, x0, acc[0]);
+  }
   double tot[1];
-  if (grid_totals<1>(acc, 1, part, ticket, tot)) {
+  if (grid_totals<1, kSumThreads>(acc, 1, part, ticket, tot)) {
     const double rel = sqrt(tot[0]) / sqrt(slots[S_NB2]);
+    slots[S_PQ] = pq_sh;
     const int k = *st.it + 1;
     *st.it = k;
     st.hist[k] = rel;
@@ -1070,7 +1240,7 @@ __global__ void __launch_bounds__(kThreads) k_fcg_update(int32_t n, double *x, d
     slots[S_REL] = rel;
     *st.restart = 0;
     int status = 0;
-    if (!(slots[S_PQ] > 0.0)) status = AMG_ERR_BREAKDOWN;
+    if (!(pq_sh > 0.0)) status = AMG_ERR_BREAKDOWN;
     else if (!isfinite(rel)) status = AMG_ERR_NAN;
     else if (rel <= slots[S_TOL]) status = 1;  // updated residual converged: the host checks the true residual
     else if (k >= (int)slots[S_MAXIT]) status = AMG_ERR_NOT_CONVERGED;
@@ -1645,8 +1815,11 @@ __global__ void __launch_bounds__(kSegThreads) k_bfcg_update(SegArgs g, double *
     const double a = g.bslots[(int64_t)S_ALPHA * g.nsys + s];
     double acc[1] = {0.0};
     const int32_t i1 = g.tile_row[t + 1];
-    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kRows * kSegThreads)
-      fcg_update_rows<VT>(i, kSegThreads, i1, a, x, r, p, q, rvt, wd, x0, acc[0]);
+    for (int32_t i = g.tile_row[t] + threadIdx.x; i < i1; i += kRows * kSegThreads) {
+      FcgRows<VT> rows;
+      rows.load(i, kSegThreads, i1, x, r, p, q, wd);
+      rows.apply(i, kSegThreads, i1, a, x, r, rvt, x0, acc[0]);
+    }
     seg_finish<1>(acc, g, t, s);
     __syncthreads();
   }
@@ -1804,16 +1977,13 @@ struct Engine {
     return a;
   }
 
-  // where level k's inner products end: their scalar step and its scratch
-  FinArgs fin_args(int k, FinKind kind, double *partials) {
-    return {kind, h.lev[k].slots, h.it_dev + 2, partials, ticket(h.lev[k])};
-  }
   unsigned *ticket(const Level &L) const { return reinterpret_cast<unsigned *>(L.flag + 1); }
 
   // ND fused inner products: after the plain product (Alg. 5) and on the last
   // post-smoothing step of level 0 (z^T q of the outer flexible CG)
+  // (returns the launch's blocks: the partial sums of each product)
   template <int EPI, int ND = 0>
-  void sell(const SellArgs<VT> &a, int k) {
+  int sell(const SellArgs<VT> &a, int k) {
     const Level &L = h.lev[k];
     if (h.batched && ND)  // inner products of a batch are per system (segdot)
       throw Error{AMG_ERR_UNSUPPORTED, "batched SpMV was given fused inner products"};
@@ -1825,13 +1995,15 @@ struct Engine {
         else
           klaunch(k_sell_small<MV, VT, EPI, ND, false>, grid, kThreads, s, a, (int)L.split_log);
         check();
-        return;
+        return grid;
       }
+    const int grid = ND ? dot_grid<VT>(L) : plain_grid(L);
     if (h.batched)
-      klaunch(k_sell<MV, VT, EPI, 0, true>, plain_grid(L), kThreads, s, a);
+      klaunch(k_sell<MV, VT, EPI, 0, true>, grid, kThreads, s, a);
     else
-      klaunch(k_sell<MV, VT, EPI, ND, false>, ND ? dot_grid<VT>(L) : plain_grid(L), kThreads, s, a);
+      klaunch(k_sell<MV, VT, EPI, ND, false>, grid, kThreads, s, a);
     check();
+    return grid;
   }
 
   // out = approximately A_k^-1 rhs with a zero initial guess (Alg. 4/5).
@@ -1928,9 +2100,10 @@ struct Engine {
       if (h.batched) {
         a.live = L.slive;
         klaunch(k_post<VT, 0, true>, grid, kThreads, s, a);
-      } else if (k == 0 && zq_fuse) {  // z^T q and beta of the outer flexible CG
+      } else if (k == 0 && zq_fuse) {  // z^T q of the outer flexible CG
         a.q64 = h.q;
-        a.fin = fin_args(0, FIN_BETA, L.partials);
+        a.partials = L.partials;
+        zq_blocks = grid;
         klaunch(k_post<VT, 1, false>, grid, kThreads, s, a);
       } else {
         klaunch(k_post<VT, 0, false>, grid, kThreads, s, a);
@@ -1960,13 +2133,14 @@ struct Engine {
     a.res = V(L.r);
     if (k == 0 && zq_fuse) {
       a.q64 = h.q;
-      a.fin = fin_args(0, FIN_BETA, L.partials);
-      sell<E_HORNER_LAST, 1>(a, k);
+      a.partials = L.partials;
+      zq_blocks = sell<E_HORNER_LAST, 1>(a, k);
     } else {
       sell<E_HORNER_LAST>(a, k);
     }
   }
   bool zq_fuse = false;
+  int zq_blocks = 0;  // partial sums of z^T q
 
   // tiles of level k and the scalar step that ends its per-system inner products;
   // gate: systems still iterating only
@@ -2028,17 +2202,23 @@ struct Engine {
     Level &L = h.lev[m];
     // c = cycle(m, r)
     cycle(m, V(L.bc), V(L.c), true, pred);
-    {  // v = A c; rho_1, alpha_1
+    int nb;
+    {  // v = A c with the sums that rho_1, alpha_1 and the test need
       SellArgs<VT> a = sell_args(m, V(L.c), V(L.v), pred);
       a.u1 = V(L.bc);
-      a.dot_y = gmres_variant;  // GMRES: v^T v, v^T r; CG: c^T v, c^T r
-      a.fin = fin_args(m, FIN_K1, L.partials);
-      sell<E_Y, 2>(a, m);
+      a.partials = L.partials;
+      nb = sell<E_Y, 5>(a, m);
     }
-    const int ng = ew_grid(L.n);
-    klaunch(k_axpy_rt<VT>, ng, kThreads, s, L.n, (const VT *)V(L.bc), (const VT *)V(L.v), V(L.rt), (const VT *)V(L.wd),
-            V(L.tmp), h.p.kcycle_t, L.slots, L.flag, L.partials, ticket(L), pred);
+    const int ng = sum_grid(L.n);
+    klaunch(k_axpy_rt<VT>, ng, kSumThreads, s, L.n, (const VT *)V(L.bc), (const VT *)V(L.v), V(L.rt),
+            (const VT *)V(L.wd), V(L.tmp), h.p.kcycle_t, gmres_variant ? 1 : 0, L.slots, L.flag,
+            (const double *)L.partials, nb, pred);
     check();
+    if (!(h.p.kcycle_t >= kTestBySums)) {
+      klaunch(k_test<VT>, ew_grid(L.n), kThreads, s, L.n, (const VT *)V(L.bc), (const VT *)V(L.rt), h.p.kcycle_t,
+              L.slots, L.flag, L.partials, ticket(L), pred);
+      check();
+    }
     // second inner step, predicated on the decision
     cycle(m, V(L.rt), V(L.d), true, L.flag);
     {
@@ -2046,15 +2226,16 @@ struct Engine {
       a.u1 = V(L.v);
       a.u2 = V(L.rt);
       a.dot_y = gmres_variant;  // GMRES: w^T w, w^T v, w^T r~; CG: d^T w, d^T v, d^T r~
-      a.fin = fin_args(m, FIN_K3, L.partials);
-      sell<E_Y, 3>(a, m);
+      a.partials = L.partials;
+      nb = sell<E_Y, 3>(a, m);
     }
-    klaunch(k_combine<VT>, ng, kThreads, s, L.n, V(L.c), V(L.d), V(L.xc), L.slots, L.flag, pred);
+    klaunch(k_combine<VT>, ng, kSumThreads, s, L.n, (const VT *)V(L.c), (const VT *)V(L.d), V(L.xc),
+            (const double *)L.slots, (const int *)L.flag, (const double *)L.partials, nb, pred);
     check();
   }
 
   // flexible CG: out = M r with the smoothing start x0 of level 0 already formed
-  // (by k_to_vt or k_fcg_update), then z^T q and beta.  The result stays in VT.
+  // (by k_to_vt or k_fcg_update), with the sums of z^T q.  The result stays in VT.
   const VT *precond_fcg(const int *pred) {
     Level &L0 = h.lev[0];
     constexpr bool f64 = std::is_same<VT, double>::value;
@@ -2064,8 +2245,8 @@ struct Engine {
     cycle(0, in, out, true, pred);
     zq_fuse = false;
     if (h.L == 1) {
-      klaunch(k_dot_zq<VT>, ew_grid(L0.n), kThreads, s, L0.n, (const VT *)out, (const double *)h.q,
-              fin_args(0, FIN_BETA, L0.partials), pred);
+      zq_blocks = ew_grid(L0.n);
+      klaunch(k_dot_zq<VT>, zq_blocks, kThreads, s, L0.n, (const VT *)out, (const double *)h.q, L0.partials, pred);
       check();
     }
     return out;
@@ -2148,13 +2329,15 @@ struct Engine {
   // one flexible-CG iteration, all on the device (graph-capturable)
   void fcg_iteration(int *active, int *restart, volatile int *host_state) {
     Level &L0 = h.lev[0];
-    const int ng = ew_grid(L0.n);
-    // z = M r, z^T q and beta
+    const int ng = sum_grid(L0.n);
+    // z = M r, z^T q
     const VT *z = precond_fcg(active);
     // p = z + beta p
-    klaunch(k_fcg_p<VT>, ng, kThreads, s, L0.n, z, h.pdir, (const double *)L0.slots, (const int *)restart, active);
+    klaunch(k_fcg_p<VT>, ng, kSumThreads, s, L0.n, z, h.pdir, L0.slots, (const int *)restart,
+            (const double *)L0.partials, zq_blocks, active);
     check();
-    {  // q = A p (FP64), p^T q, p^T r, alpha
+    const int nb = std::min(outer_grid(L0), dot_blocks<double>() * 152);
+    {  // q = A p (FP64), p^T q, p^T r
       SellArgs<double> a{};
       a.n = L0.n;
       a.nslices = L0.nslices;
@@ -2164,15 +2347,15 @@ struct Engine {
       a.x = h.pdir;
       a.out = h.q;
       a.u1 = h.r;
-      a.fin = fin_args(0, FIN_ALPHA, L0.partials);
+      a.partials = L0.partials;
       a.pred = active;
-      klaunch(k_sell<double, double, E_Y, 2, false>, std::min(outer_grid(L0), dot_blocks<double>() * 152), kThreads, s, a);
+      klaunch(k_sell<double, double, E_Y, 2, false>, nb, kThreads, s, a);
       check();
     }
     // x, r update, the next preconditioner input, and the end of the iteration
     const FcgState st{h.hist, h.it_dev, active, restart, h.status_dev, host_state};
-    klaunch(k_fcg_update<VT>, ng, kThreads, s, L0.n, h.x, h.r, (const double *)h.pdir, (const double *)h.q, L0.slots,
-            L0.partials, ticket(L0), std::is_same<VT, double>::value ? (VT *)nullptr : V(h.pre_in),
+    klaunch(k_fcg_update<VT>, ng, kSumThreads, s, L0.n, h.x, h.r, (const double *)h.pdir, (const double *)h.q, L0.slots,
+            (const double *)L0.partials, nb, L0.partials + 2 * kRedBlocks, ticket(L0), std::is_same<VT, double>::value ? (VT *)nullptr : V(h.pre_in),
             (const VT *)V(L0.wd), V(L0.tmp), st, active);
     check();
   }

@@ -109,3 +109,17 @@ def test_cycle_over_large_aggregates(gpu, orc, hubs, leaves):
     for prec in (1, 2):
         _, info = gpu.Hierarchy(A, alpha=0.25, seed=2, coarse_max=8, precision=prec).solve(b, tol=1e-8)
         assert info["final_relres"] <= 1e-8
+
+
+@pytest.mark.parametrize("t", [0.0, 5e-5, 2e-4, 0.25, 50.0])
+@pytest.mark.parametrize("outer", [0, 1])
+@pytest.mark.parametrize("m", [6, 61])
+def test_inner_step_threshold(gpu, orc, t, outer, m):
+    """The test of Alg. 5 from the product's sums and, for thresholds below 1e-4, from
+    r~ itself: always, never and by the data, in the CG and GMRES variants, on levels
+    of one and of several blocks; the cycle to 1e-10 of the oracle's."""
+    A = P.varcoef2d(m, 4)
+    b = P.rhs_uniform(A.n, 29)
+    kw = dict(alpha=0.25, seed=2, coarse_max=4, kcycle_t=t, outer=outer)
+    zg, zo = gpu.Hierarchy(A, **kw).precond(b), orc.Hierarchy(A, **kw).precond(b)
+    assert np.linalg.norm(zg - zo) <= 1e-10 * np.linalg.norm(zo)
