@@ -8,8 +8,8 @@
 // setup.  Outer iteration: flexible CG (Sec. 2.2) in FP64.
 //
 // Data-dependent control stays on the device.  The branch of Alg. 5
-// (||r~|| <= t ||r||) is written to a per-level predicate by a one-block
-// kernel; every kernel of the second inner step reads the predicate and returns
+// (||r~|| <= t ||r||) is written to a per-level predicate by the kernel that forms
+// r~; every kernel of the second inner step reads the predicate and returns
 // at once when the step is not taken.  The Krylov scalars live in device
 // memory, so an outer iteration is a fixed sequence of launches that can be
 // captured once as a CUDA graph and replayed.
