@@ -1947,8 +1947,11 @@ struct Engine {
   cudaStream_t s;
   int64_t launches = 0;
   bool gmres_variant;
+  // products skip the slices whose systems have all stopped (a batch's cycle); a
+  // product of its own (amg_spmv) computes every row whatever the last solve stopped
+  bool gate;
 
-  Engine(Hierarchy &hh, cudaStream_t ss) : h(hh), s(ss) { gmres_variant = h.p.outer == 1; }
+  Engine(Hierarchy &hh, cudaStream_t ss) : h(hh), s(ss) { gmres_variant = h.p.outer == 1, gate = h.batched; }
 
   VT *V(void *p) { return static_cast<VT *>(p); }
   // batch: the system map of a level and the systems still iterating (null otherwise)
@@ -1970,7 +1973,7 @@ struct Engine {
     a.sval = L.sval;
     a.spair = L.spair;
     a.sdiag = L.sdiag;
-    if (h.batched) a.live = L.slive;
+    if (gate) a.live = L.slive;
     a.x = x;
     a.out = out;
     a.pred = pred;
@@ -1990,7 +1993,7 @@ struct Engine {
     if constexpr (EPI == E_Y || EPI == E_RESID)
       if (L.split_log >= 0) {
         const int grid = grid_for(L.nslices, kWarps >> L.split_log, kRedBlocks);
-        if (h.batched)
+        if (gate)
           klaunch(k_sell_small<MV, VT, EPI, 0, true>, grid, kThreads, s, a, (int)L.split_log);
         else
           klaunch(k_sell_small<MV, VT, EPI, ND, false>, grid, kThreads, s, a, (int)L.split_log);
@@ -1998,7 +2001,7 @@ struct Engine {
         return grid;
       }
     const int grid = ND ? dot_grid<VT>(L) : plain_grid(L);
-    if (h.batched)
+    if (gate)
       klaunch(k_sell<MV, VT, EPI, 0, true>, grid, kThreads, s, a);
     else
       klaunch(k_sell<MV, VT, EPI, ND, false>, grid, kThreads, s, a);
@@ -3191,6 +3194,7 @@ void run_precond_t(Hierarchy &h, const double *b, double *x, cudaStream_t s) {
 template <class MV, class VT>
 void run_spmv_t(Hierarchy &h, int k, const void *x, void *y, cudaStream_t s) {
   Engine<MV, VT> eng(h, s);
+  eng.gate = false;
   SellArgs<VT> a = eng.sell_args(k, static_cast<const VT *>(x), static_cast<VT *>(y), nullptr);
   eng.template sell<E_Y>(a, k);
 }
