@@ -147,7 +147,6 @@ struct MlpShared {
   float w1[NH * FS], w2[NH * HS], w3[NO * NH], b1[NH], b2[NH], b3[4];
   float feat[kTile * FS], dout[kTile * 4];
   float h1[kTile * HS], h2[kTile * HS], dz2[kTile * HS];
-  int wild;  // a tile whose products leave the safe range of FP32
 };
 
 __device__ __forceinline__ void mlp_load_weights(MlpShared &m, const float *__restrict__ w) {
@@ -235,8 +234,12 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_coef(int32_t n, const float
 // below 1e-13 of the sum of their magnitudes; the terms themselves carry FP32
 // roundings, so that the gradient's error against a 64-bit network (1.0e-7 to
 // 2.5e-7 for 1,024 to 40,000 FEM rows) is the same to seven digits as with FP64 sums.
-// Ten training steps on four problems (22,016 rows, two error vectors): 33.8 ms with
-// a thread per row and FP64 sums of 64 row chunks, 2.6 ms now.
+//
+// The error terms are exact while nothing overflows (an infinity or NaN stays in the
+// pair to its end) and no product's error is subnormal: what a tile's 64 products can
+// lose there is at most 64 x 2^-150, below 2^-48 of a sum of at least 2^-96.  A sum
+// that is not finite or smaller than that, a parameter's own, is taken again in FP64
+// (wide_sum); a zero column, the usual case, stops there at its first pass.
 struct Pair {
   float hi = 0.0f, lo = 0.0f;
   __device__ __forceinline__ void add_err(float p, float e) {
@@ -250,22 +253,26 @@ struct Pair {
     add_err(p, __fmaf_rn(a, b, -p));
   }
   __device__ __forceinline__ void add(float a) { add_err(a, 0.0f); }
+  __device__ __forceinline__ bool sound() const { return fabsf(hi) >= 0x1p-96f && isfinite(hi) && isfinite(lo); }
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
-struct Wide {  // the same sum in FP64, for tiles out of the range where a Pair is exact enough
+
+// sum over the tile's rows of x y (y null: of x) in FP64; row strides sx, sy
+__device__ __noinline__ double wide_sum(const float *x, int sx, const float *y, int sy) {
+  bool any = false;
+  for (int r = 0; r < kTile; ++r) any |= x[r * sx] != 0.0f && (!y || y[r * sy] != 0.0f);
   double s = 0.0;
-  __device__ __forceinline__ void mac(float a, float b) { s = fma((double)a, (double)b, s); }
-  __device__ __forceinline__ void add(float a) { s += (double)a; }
-  __device__ __forceinline__ double value() const { return s; }
-};
+  if (any)
+    for (int r = 0; r < kTile; ++r) s = fma((double)x[r * sx], y ? (double)y[r * sy] : 1.0, s);
+  return s;
+}
 
 // the tile's weight gradients, added to the thread's sums: W2 (4 x 4 a thread), W1
 // (4 a thread), then b1, b2, W3, b3 (one or two a thread)
 constexpr int kMisc = 2 * NH + NO * NH + NO;  // 323
-template <class S>
 __device__ __forceinline__ void mlp_w2_sums(const MlpShared &m, double (&g2)[16]) {
   const int v0 = 4 * (threadIdx.x / 16), u0 = 4 * (threadIdx.x % 16);
-  S a[16];
+  Pair a[16];
   for (int r = 0; r < kTile; ++r) {
     const float4 d = *reinterpret_cast<const float4 *>(m.dz2 + r * HS + v0);
     const float4 h = *reinterpret_cast<const float4 *>(m.h1 + r * HS + u0);
@@ -276,13 +283,13 @@ __device__ __forceinline__ void mlp_w2_sums(const MlpShared &m, double (&g2)[16]
       for (int j = 0; j < 4; ++j) a[4 * i + j].mac(dv[i], hv[j]);
   }
 #pragma unroll
-  for (int q = 0; q < 16; ++q) g2[q] += a[q].value();
+  for (int q = 0; q < 16; ++q)
+    g2[q] += a[q].sound() ? a[q].value() : wide_sum(m.dz2 + v0 + q / 4, HS, m.h1 + u0 + q % 4, HS);
 }
 // dz1 is in m.h2's place by then; W3 and b3 come from m.h2 before (pass 0)
-template <class S>
 __device__ __forceinline__ void mlp_w1_sums(const MlpShared &m, double (&g1)[4]) {
   const int u = threadIdx.x / 4, k0 = 4 * (threadIdx.x % 4);
-  S a[4];
+  Pair a[4];
   for (int r = 0; r < kTile; ++r) {
     const float d = m.h2[r * HS + u];
     const float4 f = *reinterpret_cast<const float4 *>(m.feat + r * FS + k0);
@@ -292,22 +299,23 @@ __device__ __forceinline__ void mlp_w1_sums(const MlpShared &m, double (&g1)[4])
     a[3].mac(d, f.w);
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) g1[q] += a[q].value();
+  for (int q = 0; q < 4; ++q) g1[q] += a[q].sound() ? a[q].value() : wide_sum(m.h2 + u, HS, m.feat + k0 + q, FS);
 }
-template <class S>
 __device__ __forceinline__ void mlp_misc_sums(const MlpShared &m, int pass, double (&g)[2]) {
 #pragma unroll
   for (int q = 0; q < 2; ++q) {
     const int o = threadIdx.x + q * kMlpThreads;
     if (o >= kMisc || (o < NH) != (pass == 1)) continue;  // b1 needs dz1: the second pass
-    S a;
+    const int w3 = o - 2 * NH;  // index into W3, then b3
+    const float *x = o < NH ? m.h2 + o : (o < 2 * NH ? m.dz2 + o - NH : m.dout + (w3 < NO * NH ? w3 / NH : w3 - NO * NH));
+    const float *y = o >= 2 * NH && w3 < NO * NH ? m.h2 + w3 % NH : nullptr;
+    const int sx = o < 2 * NH ? HS : 4;
+    Pair a;
     for (int r = 0; r < kTile; ++r) {
-      if (o < NH) a.add(m.h2[r * HS + o]);
-      else if (o < 2 * NH) a.add(m.dz2[r * HS + o - NH]);
-      else if (o < 2 * NH + NO * NH) a.mac(m.dout[4 * r + (o - 2 * NH) / NH], m.h2[r * HS + (o - 2 * NH) % NH]);
-      else a.add(m.dout[4 * r + o - 2 * NH - NO * NH]);
+      if (y) a.mac(x[r * sx], y[r * HS]);
+      else a.add(x[r * sx]);
     }
-    g[q] += a.value();
+    g[q] += a.sound() ? a.value() : wide_sum(x, sx, y, HS);
   }
 }
 __device__ __forceinline__ int misc_param(int o) {
@@ -326,22 +334,16 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_grad(int32_t n, const float
   mlp_load_weights(m, wg);
   double g2[16] = {0.0}, g1[4] = {0.0}, gm[2] = {0.0};
   for (int32_t base = blockIdx.x * kTile; base < n; base += gridDim.x * kTile) {
-    if (threadIdx.x == 0) m.wild = 0;
     {
       const int r = threadIdx.x / 4, q = threadIdx.x % 4;
       m.dout[threadIdx.x] = q < NO && base + r < n ? dout[(size_t)(base + r) * NO + q] : 0.0f;
     }
     mlp_hidden(m, n, base, feat);
-    float big = 0.0f;  // largest factor of the tile's products
-    for (int q = threadIdx.x; q < kTile * NF; q += kMlpThreads) big = fmaxf(big, fabsf(m.feat[(q / NF) * FS + q % NF]));
-    float top = fmaxf(fabsf(m.dout[threadIdx.x]), 0.0f);
     for (int q = threadIdx.x; q < kTile * NH; q += kMlpThreads) {
       const int r = q / NH, v = q % NH;
       const float h2 = m.h2[r * HS + v];
       const float dh = m.w3[v] * m.dout[4 * r] + m.w3[NH + v] * m.dout[4 * r + 1] + m.w3[2 * NH + v] * m.dout[4 * r + 2];
-      const float d = dh * (1.0f - h2 * h2);
-      m.dz2[r * HS + v] = d;
-      top = fmaxf(top, fabsf(d));
+      m.dz2[r * HS + v] = dh * (1.0f - h2 * h2);
     }
     __syncthreads();
     float dz1[4][4];
@@ -368,33 +370,17 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_grad(int32_t n, const float
       for (int j = 0; j < 4; ++j) {
         const float h1 = m.h1[(r0 + i) * HS + u0 + j];
         dz1[i][j] *= 1.0f - h1 * h1;
-        top = fmaxf(top, fabsf(dz1[i][j]));
       }
-    // a product within 1e30 and the largest factor above 1e-25 leave the pair's error
-    // terms normal; otherwise (also for NaN) the tile is summed in FP64
-    if (!(top * fmaxf(big, 1.0f) < 1e30f)) m.wild = 1;
-    const bool small = __syncthreads_or(top > 1e-25f) == 0;
-    const bool wild = m.wild != 0 || small;
-    if (wild) {
-      mlp_w2_sums<Wide>(m, g2);
-      mlp_misc_sums<Wide>(m, 0, gm);
-    } else {
-      mlp_w2_sums<Pair>(m, g2);
-      mlp_misc_sums<Pair>(m, 0, gm);
-    }
+    mlp_w2_sums(m, g2);
+    mlp_misc_sums(m, 0, gm);
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) m.h2[(r0 + i) * HS + u0 + j] = dz1[i][j];
     __syncthreads();
-    if (wild) {
-      mlp_w1_sums<Wide>(m, g1);
-      mlp_misc_sums<Wide>(m, 1, gm);
-    } else {
-      mlp_w1_sums<Pair>(m, g1);
-      mlp_misc_sums<Pair>(m, 1, gm);
-    }
+    mlp_w1_sums(m, g1);
+    mlp_misc_sums(m, 1, gm);
     __syncthreads();
   }
   double *out = partial + (size_t)blockIdx.x * NP;
