@@ -1773,10 +1773,11 @@ __global__ void k_bcoarse(int32_t nL, const int32_t *__restrict__ sys, const int
   }
 }
 
-// flexible CG per system.  bact[s]: still iterating
+// flexible CG per system: p = z + beta p, p = z right after a restart (brs), whatever an
+// earlier solve left in p.  bact[s]: still iterating
 template <class VT>
 __global__ void k_bfcg_p(int32_t n, const int32_t *__restrict__ sys, int32_t nsys, const VT *z, double *p,
-                         const double *bslots, const int *bact) {
+                         const double *bslots, const int *bact, const int *brs) {
   pdl_trigger();
   pdl_wait();
   const int32_t step = gridDim.x * blockDim.x;
@@ -1797,7 +1798,7 @@ __global__ void k_bfcg_p(int32_t n, const int32_t *__restrict__ sys, int32_t nsy
       }
 #pragma unroll
     for (int u = 0; u < kRows; ++u)
-      if (sv[u] >= 0) p[i + u * step] = (double)zv[u] + BS(S_BETA, sv[u]) * pv[u];
+      if (sv[u] >= 0) p[i + u * step] = brs[sv[u]] ? (double)zv[u] : (double)zv[u] + BS(S_BETA, sv[u]) * pv[u];
   }
 }
 
@@ -2303,7 +2304,7 @@ struct Engine {
     const double *nil = nullptr;
     segdot<1>(seg_args(0, BF_BETA, true), (const VT *)z, (const double *)h.q, nil, nil, nullptr);
     klaunch(k_bfcg_p<VT>, ng, kThreads, s, n, (const int32_t *)L0.sys_of, ns, (const VT *)z, h.pdir,
-            (const double *)L0.bslots, (const int *)bact);
+            (const double *)L0.bslots, (const int *)bact, (const int *)brs);
     check();
     {  // q = A p in FP64
       SellArgs<double> a{};

@@ -72,3 +72,24 @@ def test_product_and_preconditioner_after_a_solve(env, prec, sides):
             w = np.diff(Ak.rowptr) + 4.0
             assert (np.abs(y[0] - Ak.matvec(x)) <= 2 * w * 2.0 ** -53 * mag).all(), k
     assert np.array_equal(solved.precond(b), fresh.precond(b))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_solve_after_a_system_ran_into_infinities(env, prec):
+    """A right-hand side outside the preconditioner's range ends one system of a batch
+    with a failure code; the next solve on the same hierarchy, with ordinary data, is
+    that of a fresh one."""
+    _, amg = env
+    mats, b = batch(UNEVEN)
+    used, fresh = Batch(amg, mats, precision=prec), Batch(amg, mats, precision=prec)
+    n0, n1 = mats[0].n, mats[0].n + mats[1].n
+    bad = b.copy()
+    bad[n0:n1] *= 1e60 if prec else 1e152  # squares overflow on the way, the norm does not
+    rc, it, rel = amg.amg_solve_batch(used.h, bad, np.zeros_like(b), 1e-8, len(mats),
+                                      allow=(amg.AMG_OK, amg.AMG_ERR_BREAKDOWN, amg.AMG_ERR_NAN))
+    x = [np.zeros_like(b), np.zeros_like(b)]
+    for g, xs in ((used, x[0]), (fresh, x[1])):
+        rc, it, rel = amg.amg_solve_batch(g.h, b, xs, 1e-8, len(mats), allow=(amg.AMG_OK, amg.AMG_ERR_BREAKDOWN,
+                                                                             amg.AMG_ERR_NAN))
+        assert rc == amg.AMG_OK and (rel <= 1e-8).all()
+    assert np.array_equal(*x)
