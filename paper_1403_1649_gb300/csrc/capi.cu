@@ -1,6 +1,8 @@
 // capi.cu -- the C ABI of include/amg.h: argument checks, stream handoff,
 // error translation (no exception crosses the boundary).
+#include <cmath>
 #include <cstring>
+#include <map>
 #include <mutex>
 
 #include "amg_internal.cuh"
@@ -182,6 +184,82 @@ std::vector<T> fetch(const T *dev, size_t n) {
 }
 void expect(bool ok, int k, const char *what) {
   if (!ok) throw amg::Error{AMG_ERR_SETUP, "level " + std::to_string(k) + ": " + what};
+}
+
+// entries of a SELL matrix in storage order: {column, value}; pairs (FP32) hold both
+// words, FP64 and BF16 separate arrays (BF16: a lane's entries 2j and 2j + 1 adjacent)
+struct SellEntries {
+  std::vector<int32_t> pair, col;
+  std::vector<double> val;
+  std::vector<__nv_bfloat16> half;
+  // entry e of lane `lane` in the slice that starts at `base`
+  std::pair<int32_t, double> at(int64_t base, int32_t e, int lane) const {
+    const int64_t two = base + (int64_t)(e >> 1) * 64 + 2 * lane + (e & 1), one = base + (int64_t)e * 32 + lane;
+    if (!pair.empty()) {
+      float v;
+      std::memcpy(&v, &pair[2 * two + 1], sizeof v);
+      return {pair[2 * two], v};
+    }
+    if (!half.empty()) return {col[two], __bfloat162float(half[two])};
+    return {col[one], val[one]};
+  }
+};
+
+// A P of level k against the products of the solve-phase matrix and P: columns in
+// range, and every (row, aggregate) sum within its roundings
+void check_ap(const amg::Hierarchy &h, int k, const std::vector<int32_t> &agg) {
+  const amg::Level &L = h.lev[k];
+  const bool f64 = h.p.precision == AMG_PREC_F64;
+  auto vec = [&](const void *p) {
+    if (f64) return fetch(static_cast<const double *>(p), (size_t)L.n);
+    auto f = fetch(static_cast<const float *>(p), (size_t)L.n);
+    return std::vector<double>(f.begin(), f.end());
+  };
+  auto sp = fetch(L.sptr, (size_t)L.nslices + 1), pp = fetch(L.ap_ptr, (size_t)L.nslices + 1);
+  const auto pw = vec(L.pw), own = vec(L.ap_own);
+  const auto sd = fetch(L.sdiag, L.sdiag ? (size_t)L.n : 0);
+  SellEntries a, q;
+  if (L.spair) {
+    a.pair = fetch(reinterpret_cast<const int32_t *>(L.spair), 2 * (size_t)L.sell_entries);
+  } else {
+    a.col = fetch(L.scol, (size_t)L.sell_entries);
+    if (f64) a.val = fetch(static_cast<const double *>(L.sval), (size_t)L.sell_entries);
+    else a.half = fetch(static_cast<const __nv_bfloat16 *>(L.sval), (size_t)L.sell_entries);
+  }
+  if (L.ap_pair) {
+    q.pair = fetch(reinterpret_cast<const int32_t *>(L.ap_pair), 2 * (size_t)L.ap_entries);
+  } else {
+    q.col = fetch(L.ap_col, (size_t)L.ap_entries);
+    q.val = fetch(L.ap_val, (size_t)L.ap_entries);
+  }
+  std::map<int32_t, std::pair<double, double>> sum;  // aggregate: difference, sum of magnitudes
+  for (int32_t i = 0; i < L.nslices * 32; ++i) {
+    const int32_t sl = i / 32, lane = i % 32;
+    sum.clear();
+    auto add = [&](int32_t J, double v, double mag) {
+      auto &s = sum[J];
+      s.first += v;
+      s.second += mag;
+    };
+    const int32_t width = (int32_t)((sp[sl + 1] - sp[sl]) / 32), apw = (int32_t)((pp[sl + 1] - pp[sl]) / 32);
+    for (int32_t e = 0; i < L.n && e < width; ++e) {
+      const auto [c, v] = a.at(sp[sl], e, lane);
+      add(agg[c], v * pw[c], std::fabs(v * pw[c]));
+    }
+    if (i < L.n) {
+      if (!sd.empty()) add(agg[i], sd[i] * pw[i], std::fabs(sd[i] * pw[i]));
+      add(agg[i], -own[i], 0.0);
+    }
+    for (int32_t e = 0; e < apw; ++e) {
+      const auto [J, v] = q.at(pp[sl], e, lane);
+      expect(J >= 0 && J < L.nc, k, "A P column out of range");
+      add(J, -v, 0.0);
+    }
+    // a product and an addition rounded per term, in the vectors' type
+    const double eps = (width + 2) * (f64 ? 0x1p-52 : 0x1p-23);
+    for (const auto &s : sum)
+      expect(!(std::fabs(s.second.first) > eps * s.second.second), k, "A P value");
+  }
 }
 
 }  // namespace
@@ -586,13 +664,7 @@ int amg_validate_hierarchy(const amg_hierarchy *H) {
         expect(pp[0] == 0 && pp[L.nslices] == L.ap_entries, k, "A P pointer ends");
         for (int32_t q = 0; q < L.nslices; ++q)
           expect(pp[q] <= pp[q + 1] && (pp[q + 1] - pp[q]) % unit == 0, k, "A P slice");
-        if (L.ap_pair) {
-          auto pw = fetch(reinterpret_cast<const int32_t *>(L.ap_pair), 2 * (size_t)L.ap_entries);
-          for (size_t q = 0; q < pw.size(); q += 2) expect(pw[q] >= 0 && pw[q] < L.nc, k, "A P column out of range");
-        } else {
-          for (int32_t c : fetch(L.ap_col, (size_t)L.ap_entries))
-            expect(c >= 0 && c < L.nc, k, "A P column out of range");
-        }
+        check_ap(h, k, agg);
         std::vector<char> seen(L.n, 0);
         for (int32_t I = 0; I < L.nc; ++I)
           for (int32_t m = ap[I]; m < ap[I + 1]; ++m) {

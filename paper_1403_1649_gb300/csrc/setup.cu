@@ -984,8 +984,8 @@ struct SellRow {
 };
 
 // The aggregates J != own of the row's neighbours, once each in order of first
-// occurrence: f(e, same) for the first entry e of each, same(q) telling whether
-// entry q > e belongs to it.  Up to K entries with their aggregates in registers.
+// occurrence: f(J, mask) with the row's entries of J as bits.  Up to K entries with
+// their aggregates in registers.
 template <int K, class Row, class F>
 __device__ __forceinline__ void ap_row_regs(const Row &r, int32_t width, int32_t own, const int32_t *__restrict__ agg,
                                             F &&f) {
@@ -1005,6 +1005,12 @@ __device__ __forceinline__ void ap_row_regs(const Row &r, int32_t width, int32_t
     }
   }
 }
+
+// Longer rows compare an entry's aggregate with those before it, a thread per row: the
+// square of the width in steps.  Beyond this width (a hub's row: 3,000 entries took the
+// setup 2.2 s) an entry of A stays an entry of A P of its own, which costs the cycle
+// what the row costs in A.
+constexpr int32_t kApMergeWidth = 128;
 
 // entries of A P per row without the row's own aggregate; slice width = the longest
 // row's, rounded up to even for the pair layout
@@ -1028,10 +1034,11 @@ __global__ void k_ap_width(int32_t n, int32_t nslices, const int64_t *__restrict
     } else if (width <= 24) {
       ap_row_regs<24>(r, width, own, agg, count);
     } else {
+      const bool merge = width <= kApMergeWidth;
       for (int32_t e = 0; e < width; ++e) {
         const int32_t J = agg[r.col(e)];
         bool first = J != own;
-        for (int32_t q = 0; first && q < e; ++q) first = agg[r.col(q)] != J;
+        for (int32_t q = 0; merge && first && q < e; ++q) first = agg[r.col(q)] != J;
         cnt += first ? 1 : 0;
       }
     }
@@ -1093,13 +1100,15 @@ __global__ void k_ap_fill(int32_t n, int32_t nslices, const int64_t *__restrict_
     } else if (width <= 24) {
       ap_row_regs<24>(r, width, own, agg, add);
     } else {
+      const bool merge = width <= kApMergeWidth;
       for (int32_t e = 0; e < width; ++e) {
         const int32_t J = agg[r.col(e)];
         bool first = J != own;
-        for (int32_t q = 0; first && q < e; ++q) first = agg[r.col(q)] != J;
+        for (int32_t q = 0; merge && first && q < e; ++q) first = agg[r.col(q)] != J;
         if (!first) continue;
         VT s = VT(0);
-        for (int32_t q = e; q < width; ++q) {
+        const int32_t end = merge ? width : e + 1;
+        for (int32_t q = e; q < end; ++q) {
           const int32_t c = r.col(q);
           if (agg[c] == J) s += (VT)r.val(q) * pw[c];
         }
