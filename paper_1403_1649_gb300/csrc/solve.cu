@@ -982,8 +982,10 @@ __global__ void __launch_bounds__(kSumThreads) k_axpy_rt(int32_t n, const VT *r,
       slots[S_A1] = a1;
       slots[S_S1] = s1;
       if (t >= kTestBySums) {
+        // an infinite ||r|| takes the first step of a finite length, as the comparison of
+        // the norms does (rt2 is then no number)
         const double rt2 = (tot[4] - s1 * tot[3]) - s1 * (tot[3] - s1 * tot[2]);
-        const bool second = !(rt2 <= t * t * tot[4]);
+        const bool second = isinf(tot[4]) ? !isfinite(s1) : !(rt2 <= t * t * tot[4]);
         *flag = second ? 1 : 0;
         if (second) slots[S_TAKEN] += 1.0;  // cycle trace
       }

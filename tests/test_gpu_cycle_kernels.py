@@ -123,3 +123,17 @@ def test_inner_step_threshold(gpu, orc, t, outer, m):
     kw = dict(alpha=0.25, seed=2, coarse_max=4, kcycle_t=t, outer=outer)
     zg, zo = gpu.Hierarchy(A, **kw).precond(b), orc.Hierarchy(A, **kw).precond(b)
     assert np.linalg.norm(zg - zo) <= 1e-10 * np.linalg.norm(zo)
+
+
+def test_second_step_test_with_sums_that_overflow(gpu, orc):
+    """Matrix and right-hand side scaled by powers of two until r.r overflows in FP64
+    while the step length stays finite: the test of Alg. 5 compares infinities and takes
+    the first step, as the oracle does."""
+    A = P.varcoef2d(60, 3)
+    big = P.CSR(A.n, A.rowptr, A.col, np.ldexp(A.val, 600))
+    b = np.ldexp(P.rhs_uniform(A.n, 4), 530)
+    z = gpu.Hierarchy(big, alpha=0.25, seed=1).precond(b)
+    zo = orc.Hierarchy(big, alpha=0.25, seed=1).precond(b)
+    assert np.isfinite(zo).all() and np.isfinite(z).all()
+    s = np.ldexp(1.0, 70)
+    assert np.linalg.norm(s * z - s * zo) <= 1e-10 * np.linalg.norm(s * zo)
