@@ -386,8 +386,9 @@ __device__ __forceinline__ void pdl_wait_and_trigger() {
 // The order stays complete: every block of every kernel waits before it reads or
 // writes anything that changes, so a grid ends only after its predecessor has.
 // What is read before the wait is complete before any solve is queued: setup,
-// re-setup and amg_set_poly synchronise before they return.  Vectors are read
-// with plain loads (no ld.global.nc), which the compiler keeps behind the wait.
+// re-setup and amg_set_poly synchronise before they return.  What a solve's
+// kernels write is never a const __restrict__ parameter of one: that would allow
+// ld.global.nc, which the compiler may move above the wait.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

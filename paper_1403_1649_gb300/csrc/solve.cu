@@ -886,7 +886,7 @@ __global__ void __launch_bounds__(kCoarseThreads, 1) k_restrict_coarse(
 }
 
 // sum of the first nb partials of dot k, identical in every block
-__device__ __forceinline__ double sum_partials(const double *__restrict__ part, int k, int nb) {
+__device__ __forceinline__ double sum_partials(const double *part, int k, int nb) {
   __shared__ double sh[kWarps];
   __shared__ double result;
   double acc = 0.0;
@@ -1075,7 +1075,7 @@ __global__ void __launch_bounds__(kSumThreads) k_combine(int32_t n, const VT *c,
 
 // ---------------------------------------------------------------- outer FCG (FP64)
 template <class VT>
-__global__ void k_to_vt(int32_t n, const double *__restrict__ in, VT *__restrict__ out, const VT *__restrict__ wd,
+__global__ void k_to_vt(int32_t n, const double *in, VT *__restrict__ out, const VT *__restrict__ wd,
                         VT *__restrict__ x0, const int *pred) {
   pdl_trigger();
   pdl_wait();
@@ -1089,7 +1089,7 @@ __global__ void k_to_vt(int32_t n, const double *__restrict__ in, VT *__restrict
 
 // z = (double) zin
 template <class VT>
-__global__ void k_from_vt(int32_t n, const VT *__restrict__ zin, double *__restrict__ z, const int *pred) {
+__global__ void k_from_vt(int32_t n, const VT *zin, double *__restrict__ z, const int *pred) {
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
@@ -1099,8 +1099,8 @@ __global__ void k_from_vt(int32_t n, const VT *__restrict__ zin, double *__restr
 // z^T q of the outer flexible CG where the cycle has no product to fuse it into (a
 // hierarchy of one level)
 template <class VT>
-__global__ void __launch_bounds__(kThreads) k_dot_zq(int32_t n, const VT *__restrict__ z, const double *__restrict__ q,
-                                                     double *part, const int *pred) {
+__global__ void __launch_bounds__(kThreads) k_dot_zq(int32_t n, const VT *z, const double *q, double *part,
+                                                     const int *pred) {
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
@@ -1258,8 +1258,7 @@ __global__ void __launch_bounds__(kSumThreads, 2) k_fcg_update(int32_t n, double
 }
 
 // block partial dot (generic)
-__global__ void k_dot64(int32_t n, const double *__restrict__ a, const double *__restrict__ b,
-                        double *__restrict__ part, const int *pred) {
+__global__ void k_dot64(int32_t n, const double *a, const double *b, double *__restrict__ part, const int *pred) {
   pdl_wait_and_trigger();
   if (pred && *pred == 0) return;
   double acc = 0.0;
@@ -1267,7 +1266,7 @@ __global__ void k_dot64(int32_t n, const double *__restrict__ a, const double *_
   block_store_dot(acc, part);
 }
 
-__global__ void k_store_sum(const double *__restrict__ part, int nb, double *__restrict__ dst) {
+__global__ void k_store_sum(const double *part, int nb, double *__restrict__ dst) {
   pdl_wait_and_trigger();
   const double v = sum_partials(part, 0, nb);
   if (threadIdx.x == 0) *dst = v;
@@ -1276,8 +1275,7 @@ __global__ void k_store_sum(const double *__restrict__ part, int nb, double *__r
 // r = b - A x in FP64 (level-0 SELL with FP64 values), with ||r||^2 partials
 __global__ void k_residual64(int32_t n, int32_t nslices, const int64_t *__restrict__ sptr,
                              const int32_t *__restrict__ scol, const double *__restrict__ sval,
-                             const double *__restrict__ x, const double *__restrict__ b, double *__restrict__ r,
-                             double *__restrict__ part) {
+                             const double *x, const double *b, double *__restrict__ r, double *__restrict__ part) {
   pdl_wait_and_trigger();
   const int lane = threadIdx.x & 31;
   double acc = 0.0;
@@ -1757,8 +1755,8 @@ __global__ void k_bcombine(int32_t n, const int32_t *__restrict__ sys, int32_t n
 // exact coarsest solve, one dense inverse per system; one warp per row
 template <class VT>
 __global__ void k_bcoarse(int32_t nL, const int32_t *__restrict__ sys, const int32_t *__restrict__ off,
-                          const double *__restrict__ binv, const int64_t *__restrict__ boff, const VT *__restrict__ b,
-                          VT *__restrict__ x, const int *bact, const int *pred) {
+                          const double *__restrict__ binv, const int64_t *__restrict__ boff, const VT *b, VT *__restrict__ x,
+                          const int *bact, const int *pred) {
   pdl_trigger();
   pdl_wait();
   if (pred && *pred == 0) return;
@@ -1880,8 +1878,8 @@ __global__ void k_bfcg_fin(int32_t nsys, double *__restrict__ bslots, int *__res
 #undef BS
 
 template <class VT>
-__global__ void k_convert_row_data(int32_t n, const double *__restrict__ diag, double omega_host,
-                                   const double *__restrict__ omega_dev, const double *__restrict__ pw64,
+__global__ void k_convert_row_data(int32_t n, const double *diag, double omega_host, const double *omega_dev,
+                                   const double *__restrict__ pw64,
                                    VT *__restrict__ wd, VT *__restrict__ dinv, VT *__restrict__ pw,
                                    const int32_t *__restrict__ amem, VT *__restrict__ pwm) {
   pdl_wait_and_trigger();
@@ -1897,7 +1895,7 @@ __global__ void k_convert_row_data(int32_t n, const double *__restrict__ diag, d
 }
 
 template <class VT>
-__global__ void k_copy_cast(int32_t n, const double *__restrict__ in, VT *__restrict__ out) {
+__global__ void k_copy_cast(int32_t n, const double *in, VT *__restrict__ out) {
   pdl_wait_and_trigger();
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = (VT)in[i];
 }
@@ -2890,8 +2888,7 @@ int run_fgmres_t(Hierarchy &h, const double *b, double *x, double tol, int32_t *
   return status;
 }
 
-__global__ void k_bset(int32_t nsys, const double *__restrict__ bslots, double tol, int *__restrict__ bact,
-                       int *__restrict__ bit) {
+__global__ void k_bset(int32_t nsys, const double *bslots, double tol, int *__restrict__ bact, int *__restrict__ bit) {
   pdl_wait_and_trigger();
   // bact[0..nsys) active, bact[nsys] count, bact[nsys+1 ..] restart flags; bit: iters, status
   __shared__ int nact;
@@ -2911,8 +2908,8 @@ __global__ void k_bset(int32_t nsys, const double *__restrict__ bslots, double t
 }
 
 // restart the systems whose updated residual met tol but whose true residual did not
-__global__ void k_brestart(int32_t nsys, const double *__restrict__ bslots, double tol, int max_iter,
-                           int *__restrict__ bact, int *__restrict__ bit) {
+__global__ void k_brestart(int32_t nsys, const double *bslots, double tol, int max_iter, int *__restrict__ bact,
+                           int *__restrict__ bit) {
   pdl_wait_and_trigger();
   __shared__ int nact;
   if (threadIdx.x == 0) nact = 0;
