@@ -27,8 +27,8 @@ static_assert(NP == AMG_MLP_NPARAM, "parameter layout");
 // Row i, d = |A_ii|, t_j = -A_ij / d (j != i):
 //  0: 1   1: #off/8   2..9: eight largest |A_ij|/d descending   10: fraction of
 //  off-diagonals with the sign of A_ii   11: (sum_j A_ij)/A_ii   12: level/4
-//  13: min t_j   14: max t_j   15: sum |A_ij|/d.  Sums in CSR order, IEEE
-//  division and addition only: identical to a sequential evaluation.
+//  13: min t_j   14: max t_j   15: sum |A_ij|/d.  Sums in CSR order by IEEE
+//  additions, quotients as below: the FP32 features of a sequential evaluation.
 //
 // The FP64 pipe bounds it (a warp instruction takes 16 cycles of an SM), so an
 // entry takes one quotient (|A_ij|/d = |t_j|) and two additions in FP64; what the
@@ -42,9 +42,10 @@ static_assert(NP == AMG_MLP_NPARAM, "parameter layout");
 // v / d for d > 0 with r = RN(1/d): q = v r, then one residual correction
 // q + (v - q d) r (Markstein, "Computation of elementary functions on the IBM RISC
 // System/6000 processor", 1990).  With q within an ulp the result is the correctly
-// rounded quotient; q = RN(v r) can be 1.5 ulp off, and then only a quotient within
-// 2^-106 of a rounding boundary could come out as its neighbour, which no FP32
-// feature sees.  Outside a safe range of exponents the division is taken as is.
+// rounded quotient.  q = RN(v r) can be 1.5 ulp off; then a quotient within 2^-51 of an
+// ulp of a rounding boundary can come out as its FP64 neighbour, a difference of 2^-53
+// in an FP32 feature's sums or before its rounding.  Outside a safe range of exponents
+// the division is taken as is.
 __device__ __forceinline__ bool quotient_safe(double d) { return d > 0x1p-400 && d < 0x1p400; }
 __device__ __forceinline__ double quotient(double v, double d, double r, bool safe) {
   const int ev = (__double2hiint(v) >> 20) & 0x7ff;  // biased exponent
@@ -78,8 +79,8 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(int32_t n, const int3
     __syncthreads();
     const int32_t i = i0 + threadIdx.x;
     if (threadIdx.x < rows) {
-      const int32_t p0 = rp[i], p1 = rp[i + 1];
-      auto row = [&](const double *__restrict__ v_, const int32_t *__restrict__ c_) {  // entries p0 .. p1 - 1
+      // entries p0 .. p1 - 1 of v_ and c_
+      auto row = [&](const double *__restrict__ v_, const int32_t *__restrict__ c_, int32_t p0, int32_t p1) {
         double aii = 0.0;
         for (int32_t p = p0; p < p1; ++p)
           if (c_[p] == i) aii = v_[p];
@@ -124,8 +125,8 @@ __global__ void __launch_bounds__(kFeatThreads) k_features(int32_t n, const int3
         f[14] = tmax;
         f[15] = (float)abssum;
       };
-      if (staged) row(sv - b0, sc - b0);
-      else row(val, ci);
+      if (staged) row(sv, sc, rp[i] - b0, rp[i + 1] - b0);
+      else row(val, ci, rp[i], rp[i + 1]);
     }
     __syncthreads();
     for (int32_t q = threadIdx.x; q < rows * NF; q += kFeatThreads)
