@@ -108,9 +108,12 @@ typedef struct amg_level_info {
   int32_t n_coarse;   /* n_{k+1} (0 on the coarsest level)                  */
   int32_t mis_rounds; /* PMIS iterations (k max rounds each) of this level  */
   double omega;       /* damped-Jacobi weight of this level                 */
-  int32_t spmv_blocks; /* thread blocks of the level's SpMV launches that fuse inner products */
-  int32_t seg_tile;    /* rows per tile of the per-system inner products of a
-                          batch (0: not a batch)                              */
+  int32_t spmv_blocks; /* thread blocks of the level's SpMV launches that fuse inner products
+                          (with a warp per 32 rows; levels of at most 2048 x 32 rows share
+                          rows among warps and size those launches by themselves) */
+  int32_t seg_tile;    /* batch: rows per tile of the per-system inner products on a level
+                          of 608 x 2048 rows; a level's tiles scale with its rows,
+                          between 512 and 4 seg_tile (0: not a batch)         */
 } amg_level_info;
 
 typedef struct amg_solve_info {

@@ -162,12 +162,12 @@ struct Level {
   // stay exact and the rounded matrix stays spectrally equivalent to A.
   int32_t nslices = 0;
   int32_t sell_blocks = 0;    // grid of this level's SpMV launches with fused inner products
-                              // (set at prepare, autotuned; at most kRedBlocks)
-  int32_t sell_plain_blocks = 0;  // grid of the launches without inner products (default: a
-                                  // warp per slice)
+                              // (set at prepare, autotuned; at most one wave of their kernel)
+  int32_t sell_plain_blocks = 0;  // grid of the launches without inner products (default: one
+                                  // wave of theirs)
   int32_t split_log = -1;     // log2 of the warps that share a slice in the small-level product
                               // (-1: one warp per slice, k_sell)
-  int32_t seg_tile = 0;       // batch: rows per tile of the per-system inner products
+  int32_t seg_tile = 0;       // batch: sizes the tiles of the per-system inner products (tile_rows)
   int64_t sell_entries = 0;
   int64_t *sptr = nullptr;
   int32_t *scol = nullptr;

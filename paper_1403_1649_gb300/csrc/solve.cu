@@ -1915,11 +1915,12 @@ template <class VT>
 inline int default_sell_grid(const Level &L) {
   return grid_for((int64_t)L.nslices, kWarps, sell_min_blocks<VT>() * 152);
 }
-// launches with fused inner products: at most one wave of their kernel, which
-// runs dot_blocks per SM (a second, short wave and its reductions took the
-// 190k-row level of 128^3 from 10 to 17 us)
+// launches with fused inner products: one wave of their kernel, which runs
+// dot_blocks per SM (a second, short wave and its reductions took the 190k-row
+// level of 128^3 from 10 to 17 us), or the autotuner's choice up to it
 template <class VT>
-inline int dot_grid(const Level &L) { return std::min(L.sell_blocks, dot_blocks<VT>() * 152); }
+constexpr int dot_wave() { return dot_blocks<VT>() * 152; }
+inline int dot_grid(const Level &L) { return L.sell_blocks; }
 // launches without inner products have no partial-sum buffer to fill, so the
 // autotuner may give them up to one warp per slice; by default they take the
 // same wave of resident blocks (one warp per slice measured slower on the 128^3
@@ -2001,7 +2002,7 @@ struct Engine {
         check();
         return grid;
       }
-    const int grid = ND ? dot_grid<VT>(L) : plain_grid(L);
+    const int grid = ND ? dot_grid(L) : plain_grid(L);
     if (gate)
       klaunch(k_sell<MV, VT, EPI, 0, true>, grid, kThreads, s, a);
     else
@@ -2340,7 +2341,7 @@ struct Engine {
     klaunch(k_fcg_p<VT>, ng, kSumThreads, s, L0.n, z, h.pdir, L0.slots, (const int *)restart,
             (const double *)L0.partials, zq_blocks, active);
     check();
-    const int nb = std::min(outer_grid(L0), dot_blocks<double>() * 152);
+    const int nb = std::min(outer_grid(L0), dot_wave<double>());
     {  // q = A p (FP64), p^T q, p^T r
       SellArgs<double> a{};
       a.n = L0.n;
@@ -2439,8 +2440,8 @@ void alloc_level_vectors(Hierarchy &h, Level &L, int k) {
     L.d = vec();
     L.w = vec();
   }
-  if (L.sell_blocks <= 0) L.sell_blocks = default_sell_grid<VT>(L);
-  if (L.sell_plain_blocks <= 0) L.sell_plain_blocks = L.sell_blocks;
+  if (L.sell_blocks <= 0) L.sell_blocks = grid_for((int64_t)L.nslices, kWarps, dot_wave<VT>());
+  if (L.sell_plain_blocks <= 0) L.sell_plain_blocks = default_sell_grid<VT>(L);
   L.split_log = split_log_for(L);
   L.slots = h.arena.get<double>(kNumSlots);
   L.flag = h.arena.get<int>(4);
@@ -3042,14 +3043,16 @@ int run_solve_batch_t(Hierarchy &h, const double *b, double *x, double tol, int3
 }
 
 // Row tiles of level L for the per-system inner products, every tile in one system.
-// `tile` rows suit a level that fills the GPU with kSegWave of them; smaller levels
+// `seg_tile` rows suit a level that fills the GPU with kSegWave of them; smaller levels
 // take smaller tiles (two rows a thread at least) so that their FP64 work meets more
 // SMs, larger ones up to four times larger tiles with fewer sums to finish.
 constexpr int32_t kSegWave = 152 * 4;
-void build_tiles(Hierarchy &h, Level &L, int32_t seg_tile, cudaStream_t s) {
-  const int32_t ns = h.nsys;
+int32_t tile_rows(const Level &L, int32_t seg_tile) {
   const int64_t fit = (int64_t)L.n * seg_tile / ((int64_t)kSegWave * 2048);
-  const int32_t tile = (int32_t)std::max<int64_t>(2 * kSegThreads, std::min<int64_t>(4 * (int64_t)seg_tile, (fit + 255) / 256 * 256));
+  return (int32_t)std::max<int64_t>(2 * kSegThreads, std::min<int64_t>(4 * (int64_t)seg_tile, (fit + 255) / 256 * 256));
+}
+void build_tiles(Hierarchy &h, Level &L, int32_t seg_tile, cudaStream_t s) {
+  const int32_t ns = h.nsys, tile = tile_rows(L, seg_tile);
   std::vector<int32_t> trow, tsys, stile(ns + 1, 0);
   for (int32_t q = 0; q < ns; ++q) {
     stile[q] = (int32_t)trow.size();
@@ -3103,8 +3106,8 @@ void prepare_batched(Hierarchy &h, cudaStream_t s) {
 // Autotuner of the launch shapes (setup time).  For every level the SpMV is
 // timed with CUDA events over candidate grid sizes (multiples of the 152 SMs up
 // to one warp per slice) and the smallest grid within 3 % of the fastest is
-// kept, for the launches that fuse inner products among the grids within the
-// partial-sum capacity; for a batch, the row tile of the per-system inner products is chosen
+// kept, for the launches that fuse inner products among the grids within one
+// wave of their kernel; for a batch, the row tile of the per-system inner products is chosen
 // the same way.  The shapes change the grouping of partial sums only.
 template <class MV, class VT>
 void autotune_t(Hierarchy &h, cudaStream_t s) {
@@ -3136,7 +3139,7 @@ void autotune_t(Hierarchy &h, cudaStream_t s) {
       DevBuf<VT> x((size_t)L.n + 1), y((size_t)L.n + 1);
       AMG_CUDA(cudaMemsetAsync(x.p, 0, sizeof(VT) * (L.n + 1), s));
       // the plain product at each grid; launches with fused inner products take
-      // the best grid within the partial-sum capacity.  The split-row kernel of
+      // the best grid within one wave of theirs.  The split-row kernel of
       // the small levels covers its slices in one pass and has no grid to choose.
       const int gfull = full_plain_grid(L);
       std::vector<std::pair<int, float>> t, tr;
@@ -3147,13 +3150,14 @@ void autotune_t(Hierarchy &h, cudaStream_t s) {
         L.sell_plain_blocks = gg;
         const SellArgs<VT> a = eng.sell_args(k, x.p, y.p, nullptr);
         t.push_back({gg, time_it([&] { eng.template sell<E_Y>(a, k); })});
-        if (gg <= kRedBlocks) tr.push_back(t.back());
+        if (gg <= dot_wave<VT>()) tr.push_back(t.back());
       }
       L.sell_plain_blocks = pick(t);
       L.sell_blocks = pick(tr);
       if (h.batched && k < h.L - 1) {
         std::vector<std::pair<int, float>> tt;
         for (int tile : {1024, 2048, 4096, 8192}) {
+          if (!tt.empty() && tile_rows(L, tile) == tile_rows(L, tt.back().first)) continue;  // the same tiles
           build_tiles(h, L, tile, s);
           tt.push_back({tile, time_it([&] {
                           const VT *nil = nullptr;

@@ -137,3 +137,15 @@ def test_second_step_test_with_sums_that_overflow(gpu, orc):
     assert np.isfinite(zo).all() and np.isfinite(z).all()
     s = np.ldexp(1.0, 70)
     assert np.linalg.norm(s * z - s * zo) <= 1e-10 * np.linalg.norm(s * zo)
+
+
+@pytest.mark.parametrize("prec,wave", [(0, 456), (1, 608), (2, 608)])
+def test_reported_blocks_are_those_of_the_launches(gpu, prec, wave):
+    """Levels of 3,082 and 6,329 slices: the launches with inner products run one wave of their
+    kernel (three or four blocks on each of 152 SMs), tuned or not at most that."""
+    A = P.poisson2d(314)
+    n0 = gpu.Hierarchy(A, alpha=0.25, precision=prec).info()[0]
+    assert (n0["n"] + 31) // 32 > 2048 and n0["spmv_blocks"] == min(wave, ((n0["n"] + 31) // 32 + 7) // 8)
+    big = P.poisson2d(450)
+    assert gpu.Hierarchy(big, alpha=0.25, precision=prec).info()[0]["spmv_blocks"] == wave
+    assert gpu.Hierarchy(big, alpha=0.25, precision=prec, autotune=1).info()[0]["spmv_blocks"] <= wave
