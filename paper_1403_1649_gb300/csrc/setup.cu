@@ -984,12 +984,35 @@ struct SellRow {
 };
 
 // The aggregates J != own of the row's neighbours, once each in order of first
-// occurrence: f(J, mask) with the row's entries of J as bits.  Up to K entries with
-// their aggregates in registers.
-template <int K, class Row, class F>
+// occurrence: f(J, mask) with the row's entries of J as bits; before them g(mask) with
+// the entries of the own aggregate.  Up to K entries with their aggregates in registers.
+template <int K, class Row, class G, class F>
 __device__ __forceinline__ void ap_row_regs(const Row &r, int32_t width, int32_t own, const int32_t *__restrict__ agg,
-                                            F &&f) {
+                                            G &&g, F &&f) {
   int32_t J[K];
+#pragma unroll
+  for (int e = 0; e < K; ++e) J[e] = e < width ? agg[r.col(e)] : -1;
+  unsigned seen = 0;
+#pragma unroll
+  for (int e = 0; e < K; ++e) seen |= J[e] == own ? 1u << e : 0u;
+  g(seen);
+#pragma unroll
+  for (int e = 0; e < K; ++e) {
+    if (J[e] >= 0 && !(seen & (1u << e))) {
+      unsigned mask = 0;  // the entries of this aggregate
+#pragma unroll
+      for (int q = e; q < K; ++q) mask |= J[q] == J[e] ? 1u << q : 0u;
+      seen |= mask;
+      f(J[e], mask);
+    }
+  }
+}
+
+// the number of those aggregates
+template <int K, class Row>
+__device__ __forceinline__ int32_t ap_count_regs(const Row &r, int32_t width, int32_t own,
+                                                 const int32_t *__restrict__ agg) {
+  int32_t J[K], cnt = 0;
 #pragma unroll
   for (int e = 0; e < K; ++e) J[e] = e < width ? agg[r.col(e)] : own;
 #pragma unroll
@@ -997,126 +1020,210 @@ __device__ __forceinline__ void ap_row_regs(const Row &r, int32_t width, int32_t
     bool first = J[e] != own;
 #pragma unroll
     for (int q = 0; q < e; ++q) first = first && J[q] != J[e];
-    if (first) {
-      unsigned mask = 0;  // the entries of this aggregate
-#pragma unroll
-      for (int q = e; q < K; ++q) mask |= J[q] == J[e] ? 1u << q : 0u;
-      f(J[e], mask);
-    }
+    cnt += first ? 1 : 0;
   }
+  return cnt;
 }
 
-// Longer rows compare an entry's aggregate with those before it, a thread per row: the
-// square of the width in steps.  Beyond this width (a hub's row: 3,000 entries took the
-// setup 2.2 s) an entry of A stays an entry of A P of its own, which costs the cycle
-// what the row costs in A.
-constexpr int32_t kApMergeWidth = 128;
+// Entries of A P per row without the row's own aggregate: sum_{j in J} a_ij P_j in the
+// vector type, a_ij as the solve-phase matrix holds them (rounded values, compensated
+// diagonal), so that the residual update is that of the same operator; the own entry to
+// `own`.  Two passes, FILL = false: the slices' widths (the longest row's, rounded up to
+// even for the pair layout), FILL = true: the entries.
+//
+// Slices of at most kApNarrow entries a row take a lane per row with the row's
+// aggregates in registers.  Wider ones are shared by the block: its warps stage the
+// slice's aggregates (and values and weights) in shared memory, coalesced, then take a
+// row each, a lane per entry, every lane comparing its aggregate with the row's entries
+// one after the other; the sums keep the entries' order.  By a lane per row those
+// comparisons are a chain of loads, the square of the width long: the two passes took
+// 42 + 61 us on the level of 1,538 rows of 128^3, 7 + 17 us now, and 121 + 249 us on all
+// its levels, 64 + 177 us now.  Beyond kApMergeWidth entries (a hub's row) an
+// entry of A stays an entry of A P of its own, which costs the cycle what the row costs
+// in A: coarse levels of 3D problems have a few slices in a thousand of that width.
+constexpr int32_t kApNarrow = 24, kApMergeWidth = 64;
+constexpr int kApWarps = 8;
+constexpr int kApStride = kSlice + 1;  // a row's entries in shared memory without bank conflicts
 
-// entries of A P per row without the row's own aggregate; slice width = the longest
-// row's, rounded up to even for the pair layout
-template <class MV>
-__global__ void k_ap_width(int32_t n, int32_t nslices, const int64_t *__restrict__ sptr,
-                           const int32_t *__restrict__ scol, const int4 *__restrict__ spair,
-                           const int32_t *__restrict__ agg, bool pairs, int64_t *__restrict__ width32) {
-  pdl_wait_and_trigger();
-  const int lane = threadIdx.x & 31;
-  const int32_t sl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (sl >= nslices) return;
-  const int32_t row = sl * kSlice + lane;
-  const SellRow<MV> r{scol, nullptr, spair, sptr[sl], lane};
-  const int32_t width = (int32_t)((sptr[sl + 1] - r.base) / kSlice);
-  int32_t cnt = 0;
-  if (row < n) {
-    const int32_t own = agg[row];
-    auto count = [&](int32_t, unsigned) { ++cnt; };
-    if (width <= 8) {
-      ap_row_regs<8>(r, width, own, agg, count);
-    } else if (width <= 24) {
-      ap_row_regs<24>(r, width, own, agg, count);
-    } else {
-      const bool merge = width <= kApMergeWidth;
-      for (int32_t e = 0; e < width; ++e) {
-        const int32_t J = agg[r.col(e)];
-        bool first = J != own;
-        for (int32_t q = 0; merge && first && q < e; ++q) first = agg[r.col(q)] != J;
-        cnt += first ? 1 : 0;
-      }
-    }
-  }
-  cnt = __reduce_max_sync(0xffffffffu, cnt);
-  if (pairs) cnt = (cnt + 1) & ~1;
-  if (lane == 0) width32[sl] = (int64_t)cnt * kSlice;
-}
-
-// the entries sum_{j in J} a_ij P_j in the vector type, a_ij as the solve-phase
-// matrix holds them (rounded values, compensated diagonal), so that the residual
-// update is that of the same operator
 template <class MV, class VT>
-__global__ void k_ap_fill(int32_t n, int32_t nslices, const int64_t *__restrict__ sptr,
-                          const int32_t *__restrict__ scol, const MV *__restrict__ sval,
-                          const int4 *__restrict__ spair, const float *__restrict__ sdiag,
-                          const int32_t *__restrict__ agg, const VT *__restrict__ pw,
-                          const int64_t *__restrict__ apptr, int4 *__restrict__ appair, int32_t *__restrict__ apcol,
-                          double *__restrict__ apval, VT *__restrict__ apown) {
+struct ApArgs {
+  int32_t n, nslices;
+  int spb;  // slices per block, at most kApWarps
+  const int64_t *sptr;
+  const int32_t *scol;
+  const MV *sval;
+  const int4 *spair;
+  const float *sdiag;
+  const int32_t *agg;
+  const VT *pw;
+  int64_t *width32;      // FILL = false
+  const int64_t *apptr;  // FILL = true
+  int4 *appair;
+  int32_t *apcol;
+  double *apval;
+  VT *own;
+};
+
+template <class MV, class VT, bool FILL>
+constexpr size_t ap_smem() {
+  return (size_t)kApMergeWidth * kApStride * (sizeof(int32_t) + (FILL ? 2 * sizeof(VT) : 0));
+}
+
+template <class MV, class VT, bool FILL>
+__global__ void __launch_bounds__(kApWarps * 32) k_ap(ApArgs<MV, VT> a) {
   pdl_wait_and_trigger();
-  const int lane = threadIdx.x & 31;
-  const int32_t sl = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (sl >= nslices) return;
-  const int32_t row = sl * kSlice + lane;
-  const SellRow<MV> r{scol, sval, spair, sptr[sl], lane};
-  const int32_t width = (int32_t)((sptr[sl + 1] - r.base) / kSlice);
-  const int64_t base = apptr[sl];
-  const int32_t apw = (int32_t)((apptr[sl + 1] - base) / kSlice);
-  const int32_t own = agg[row < n ? row : n - 1];
-  int32_t cnt = 0;
-  auto put = [&](int32_t c, VT v) {
+  extern __shared__ __align__(16) unsigned char ap_sm[];
+  __shared__ int32_t widest;
+  VT *sV = reinterpret_cast<VT *>(ap_sm), *sP = sV + kApMergeWidth * kApStride;
+  int32_t *sJ = FILL ? reinterpret_cast<int32_t *>(sP + kApMergeWidth * kApStride) : reinterpret_cast<int32_t *>(ap_sm);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int32_t s0 = blockIdx.x * a.spb, s1 = min(s0 + a.spb, a.nslices);
+  auto slice_width = [&](int32_t sl) { return (int32_t)((a.sptr[sl + 1] - a.sptr[sl]) / kSlice); };
+  auto even = [&](int32_t w) { return std::is_same<VT, float>::value ? (w + 1) & ~1 : w; };
+  // entry `at` of row r of slice sl
+  auto put = [&](int32_t sl, int r, int32_t at, int32_t c, VT v) {
+    const int64_t base = a.apptr[sl];
     if constexpr (std::is_same<VT, float>::value) {
-      int2 *w = reinterpret_cast<int2 *>(appair + (base >> 1) + (int64_t)(cnt >> 1) * kSlice + lane) + (cnt & 1);
+      int2 *w = reinterpret_cast<int2 *>(a.appair + (base >> 1) + (int64_t)(at >> 1) * kSlice + r) + (at & 1);
       *w = make_int2(c, __float_as_int(v));
     } else {
-      apcol[base + (int64_t)cnt * kSlice + lane] = c;
-      apval[base + (int64_t)cnt * kSlice + lane] = v;
+      a.apcol[base + (int64_t)at * kSlice + r] = c;
+      a.apval[base + (int64_t)at * kSlice + r] = v;
     }
-    ++cnt;
   };
-  if (row < n) {
-    VT o = VT(0);
-    if (sdiag) o = (VT)sdiag[row] * pw[row];
-    for (int32_t e = 0; e < width; ++e) {
-      const int32_t c = r.col(e);
-      if (agg[c] == own) o += (VT)r.val(e) * pw[c];
-    }
-    apown[row] = o;
-    auto add = [&](int32_t J, unsigned mask) {
-      VT s = VT(0);
-      for (; mask; mask &= mask - 1) {
-        const int32_t e = __ffs(mask) - 1;
-        s += (VT)r.val(e) * pw[r.col(e)];
-      }
-      put(J, s);
-    };
-    if (width <= 8) {
-      ap_row_regs<8>(r, width, own, agg, add);
-    } else if (width <= 24) {
-      ap_row_regs<24>(r, width, own, agg, add);
+  auto ap_width = [&](int32_t sl) { return (int32_t)((a.apptr[sl + 1] - a.apptr[sl]) / kSlice); };
+
+  if (s0 + wid < s1 && slice_width(s0 + wid) <= kApNarrow) {  // a lane per row
+    const int32_t sl = s0 + wid, row = sl * kSlice + lane, width = slice_width(sl);
+    const SellRow<MV> r{a.scol, a.sval, a.spair, a.sptr[sl], lane};
+    const int32_t own = a.agg[row < a.n ? row : a.n - 1];
+    int32_t cnt = 0;
+    if constexpr (!FILL) {
+      if (row < a.n)
+        cnt = width <= 8 ? ap_count_regs<8>(r, width, own, a.agg) : ap_count_regs<kApNarrow>(r, width, own, a.agg);
+      cnt = __reduce_max_sync(0xffffffffu, cnt);
+      if (lane == 0) a.width32[sl] = (int64_t)even(cnt) * kSlice;
     } else {
-      const bool merge = width <= kApMergeWidth;
-      for (int32_t e = 0; e < width; ++e) {
-        const int32_t J = agg[r.col(e)];
-        bool first = J != own;
-        for (int32_t q = 0; merge && first && q < e; ++q) first = agg[r.col(q)] != J;
-        if (!first) continue;
-        VT s = VT(0);
-        const int32_t end = merge ? width : e + 1;
-        for (int32_t q = e; q < end; ++q) {
-          const int32_t c = r.col(q);
-          if (agg[c] == J) s += (VT)r.val(q) * pw[c];
+      if (row < a.n) {
+        const VT dp = a.sdiag ? (VT)a.sdiag[row] * a.pw[row] : VT(0);
+        auto narrow = [&](auto size, auto &&sum) {
+          constexpr int K = decltype(size)::value;
+          ap_row_regs<K>(r, width, own, a.agg, [&](unsigned mask) { a.own[row] = sum(dp, mask); },
+                         [&](int32_t J, unsigned mask) { put(sl, lane, cnt++, J, sum(VT(0), mask)); });
+        };
+        if (width <= 8) {  // values and weights in registers too: all loads go out at once
+          VT v[8], p[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) {
+            v[e] = e < width ? (VT)r.val(e) : VT(0);
+            p[e] = e < width ? a.pw[r.col(e)] : VT(0);
+          }
+          narrow(std::integral_constant<int, 8>{}, [&](VT s, unsigned mask) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+              if (mask & (1u << e)) s += v[e] * p[e];
+            return s;
+          });
+        } else {
+          narrow(std::integral_constant<int, kApNarrow>{}, [&](VT s, unsigned mask) {
+            for (; mask; mask &= mask - 1) {
+              const int32_t e = __ffs(mask) - 1;
+              s += (VT)r.val(e) * a.pw[r.col(e)];
+            }
+            return s;
+          });
         }
-        put(J, s);
       }
+      for (const int32_t apw = ap_width(sl); cnt < apw; ++cnt) put(sl, lane, cnt, own, VT(0));
     }
   }
-  while (cnt < apw) put(own, VT(0));
+  const unsigned below = (1u << lane) - 1u;
+  for (int32_t sl = s0; sl < s1; ++sl) {  // the wide slices: the same in every thread
+    const int32_t width = slice_width(sl);
+    if (width <= kApNarrow) continue;
+    const bool merge = width <= kApMergeWidth;
+    __syncthreads();  // the previous slice's entries have been read
+    if (!FILL && threadIdx.x == 0) widest = 0;
+    if (merge) {
+      const SellRow<MV> r{a.scol, a.sval, a.spair, a.sptr[sl], lane};
+      for (int32_t e = wid; e < width; e += kApWarps) {
+        const int32_t c = r.col(e);
+        sJ[e * kApStride + lane] = a.agg[c];
+        if constexpr (FILL) {
+          sV[e * kApStride + lane] = (VT)r.val(e);
+          sP[e * kApStride + lane] = a.pw[c];
+        }
+      }
+    }
+    __syncthreads();
+    for (int j = wid; j < kSlice; j += kApWarps) {  // a warp per row
+      const int32_t row = sl * kSlice + j;
+      const int32_t own = a.agg[row < a.n ? row : a.n - 1];
+      int32_t cnt = 0;
+      VT o = VT(0);
+      if constexpr (FILL)
+        if (row < a.n && a.sdiag) o = (VT)a.sdiag[row] * a.pw[row];
+      if (row < a.n && merge) {
+        constexpr int kPer = kApMergeWidth / 32;  // entries of a lane
+        int32_t J[kPer];
+        bool first[kPer];  // the first entry of its aggregate carries the aggregate's sum
+        VT s[kPer];
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+          const int32_t e = 32 * u + lane;
+          J[u] = e < width ? sJ[e * kApStride + j] : own;
+          first[u] = J[u] != own;
+          s[u] = VT(0);
+        }
+        for (int32_t q = 0; q < width; ++q) {
+          const int32_t Jq = sJ[q * kApStride + j];
+          VT v = VT(0), p = VT(0);
+          if constexpr (FILL) {
+            v = sV[q * kApStride + j];
+            p = sP[q * kApStride + j];
+            if (Jq == own) o += v * p;
+          }
+#pragma unroll
+          for (int u = 0; u < kPer; ++u)
+            if (Jq == J[u]) {
+              if (q < 32 * u + lane) first[u] = false;
+              else if constexpr (FILL) s[u] += v * p;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+          const unsigned b = __ballot_sync(0xffffffffu, first[u]);
+          if constexpr (FILL)
+            if (first[u]) put(sl, j, cnt + __popc(b & below), J[u], s[u]);
+          cnt += __popc(b);
+        }
+      } else if (row < a.n) {
+        const SellRow<MV> r{a.scol, a.sval, a.spair, a.sptr[sl], j};
+        for (int32_t e0 = 0; e0 < width; e0 += 32) {
+          const bool in = e0 + lane < width;
+          const int32_t c = in ? r.col(e0 + lane) : row, J = a.agg[c];
+          const unsigned b = __ballot_sync(0xffffffffu, in && J != own);
+          if constexpr (FILL) {
+            const VT v = in ? (VT)r.val(e0 + lane) : VT(0), p = a.pw[c];
+            if (in && J != own) put(sl, j, cnt + __popc(b & below), J, v * p);
+            for (unsigned m = __ballot_sync(0xffffffffu, in && J == own); m; m &= m - 1)
+              o += __shfl_sync(0xffffffffu, v, __ffs(m) - 1) * __shfl_sync(0xffffffffu, p, __ffs(m) - 1);
+          }
+          cnt += __popc(b);
+        }
+      }
+      if constexpr (FILL) {
+        if (row < a.n && lane == 0) a.own[row] = o;
+        for (int32_t at = cnt + lane, apw = ap_width(sl); at < apw; at += 32) put(sl, j, at, own, VT(0));
+      } else if (lane == 0) {
+        atomicMax(&widest, cnt);
+      }
+    }
+    if constexpr (!FILL) {
+      __syncthreads();
+      if (threadIdx.x == 0) a.width32[sl] = (int64_t)even(widest) * kSlice;
+    }
+  }
 }
 
 // ============================================================== Arnoldi omega
@@ -2249,14 +2356,37 @@ void build_solve_matrix(Hierarchy &h, Level &L, cudaStream_t s, bool fresh) {
 
 // A P of level q (not the coarsest).  widths: slice widths and their scan, the
 // entry count on its way to the pinned word of the level (read at the caller's
-// next synchronisation); fill: the entries
+// next synchronisation); fill: the entries.  A level of at most kApSpread slices
+// gives each a block, so that its wide slices do not queue behind one another
+constexpr int32_t kApSpread = 4096;
+template <class MV, class VT, bool FILL>
+void ap_launch(const Level &L, int64_t *width32, cudaStream_t s) {
+  ApArgs<MV, VT> a{};
+  a.n = L.n;
+  a.nslices = L.nslices;
+  a.spb = L.nslices <= kApSpread ? 1 : kApWarps;
+  a.sptr = L.sptr;
+  a.scol = L.scol;
+  a.sval = (const MV *)L.sval;
+  a.spair = L.spair;
+  a.sdiag = L.sdiag;
+  a.agg = L.agg;
+  a.pw = (const VT *)L.pw;
+  a.width32 = width32;
+  a.apptr = L.ap_ptr;
+  a.appair = L.ap_pair;
+  a.apcol = L.ap_col;
+  a.apval = L.ap_val;
+  a.own = (VT *)L.ap_own;
+  AMG_COUNT(), klaunch_sm(k_ap<MV, VT, FILL>, (unsigned)((L.nslices + a.spb - 1) / a.spb), kApWarps * 32,
+                          ap_smem<MV, VT, FILL>(), s, a);
+  AMG_LAUNCH_CHECK();
+}
 template <class MV, class VT>
 void ap_widths_t(Hierarchy &h, int q, cudaStream_t s) {
   Level &L = h.lev[q];
   DevBuf<int64_t> w32(L.nslices + 1);
-  AMG_COUNT(), klaunch_sm(k_ap_width<MV>, blocks_for((int64_t)L.nslices * 32), 256, 0, s, L.n, L.nslices, L.sptr, L.scol,
-                          L.spair, L.agg, std::is_same<VT, float>::value, w32.p);
-  AMG_LAUNCH_CHECK();
+  ap_launch<MV, VT, false>(L, w32.p, s);
   L.ap_ptr = h.arena.get<int64_t>(L.nslices + 1);
   exclusive_scan<int64_t, int64_t>(w32.p, L.ap_ptr, L.nslices, s);
   AMG_CUDA(cudaMemcpyAsync(reinterpret_cast<int64_t *>(h.host_pinned + kPinnedSellEntries) + q, L.ap_ptr + L.nslices,
@@ -2275,10 +2405,7 @@ void ap_fill_t(Hierarchy &h, int q, cudaStream_t s, bool fresh) {
       L.ap_val = h.arena.get<double>(L.ap_entries);
     }
   }
-  AMG_COUNT(), klaunch_sm(k_ap_fill<MV, VT>, blocks_for((int64_t)L.nslices * 32), 256, 0, s, L.n, L.nslices, L.sptr,
-                          L.scol, (const MV *)L.sval, L.spair, L.sdiag, L.agg, (const VT *)L.pw, L.ap_ptr, L.ap_pair,
-                          L.ap_col, L.ap_val, (VT *)L.ap_own);
-  AMG_LAUNCH_CHECK();
+  ap_launch<MV, VT, true>(L, nullptr, s);
 }
 void ap_widths(Hierarchy &h, int q, cudaStream_t s) {
   if (h.p.precision == AMG_PREC_F64) ap_widths_t<double, double>(h, q, s);

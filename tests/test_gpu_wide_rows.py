@@ -44,9 +44,9 @@ def hub_grid(m, degree, seed):
 
 
 @pytest.mark.parametrize("prec", [0, 1, 2])
-@pytest.mark.parametrize("degree", [20, 60, 123, 124, 125, 700])
+@pytest.mark.parametrize("degree", [19, 20, 21, 40, 59, 60, 61, 124, 700])
 def test_cycle_with_a_hub(env, prec, degree):
-    """Rows of 25 to 705 entries: the hierarchy's arrays are consistent (the values of A P
+    """Rows of 24 to 705 entries: the hierarchy's arrays are consistent (the values of A P
     among them), and in FP64 the cycle is the oracle's."""
     amg, oracle = env
     A = hub_grid(48, degree, degree)
