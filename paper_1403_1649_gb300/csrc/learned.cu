@@ -148,6 +148,12 @@ struct MlpShared {
   float w1[NH * FS], w2[NH * HS], w3[NO * NH], b1[NH], b2[NH], b3[4];
   float feat[kTile * FS], dout[kTile * 4];
   float h1[kTile * HS], h2[kTile * HS], dz2[kTile * HS];
+  // columns with a nonzero entry, as each warp saw its part of the tile: bit k of
+  // feat[w] for feature k, bit v % 32 of dz2[w] for unit v (w % 2 = v / 32), bit u / 4 of
+  // dz1[w][u % 4] for unit u
+  struct {
+    unsigned feat[kMlpThreads / 32], dz2[kMlpThreads / 32], dz1[kMlpThreads / 32][4];
+  } nz;
 };
 
 __device__ __forceinline__ void mlp_load_weights(MlpShared &m, const float *__restrict__ w) {
@@ -195,10 +201,15 @@ __device__ __forceinline__ void mlp_layer(const float *x, const float *w, const 
 
 // the tile's features (zero beyond the last row) and hidden activations
 __device__ __forceinline__ void mlp_hidden(MlpShared &m, int32_t n, int32_t base, const float *__restrict__ feat) {
-  for (int q = threadIdx.x; q < kTile * NF; q += kMlpThreads) {
+  bool nz = false;
+  for (int q = threadIdx.x; q < kTile * NF; q += kMlpThreads) {  // a thread stays in its column
     const int32_t r = base + q / NF;
-    m.feat[(q / NF) * FS + q % NF] = r < n ? feat[(size_t)r * NF + q % NF] : 0.0f;
+    const float f = r < n ? feat[(size_t)r * NF + q % NF] : 0.0f;
+    nz |= f != 0.0f;
+    m.feat[(q / NF) * FS + q % NF] = f;
   }
+  const unsigned b = __ballot_sync(0xffffffffu, nz);
+  if (threadIdx.x % 32 == 0) m.nz.feat[threadIdx.x / 32] = (b | b >> 16) & 0xffffu;
   __syncthreads();
   mlp_layer<NF, FS>(m.feat, m.w1, m.b1, m.h1);
   __syncthreads();
@@ -240,7 +251,7 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_coef(int32_t n, const float
 // pair to its end) and no product's error is subnormal: what a tile's 64 products can
 // lose there is at most 64 x 2^-150, below 2^-48 of a sum of at least 2^-96.  A sum
 // that is not finite or smaller than that, a parameter's own, is taken again in FP64
-// (wide_sum); a zero column, the usual case, stops there at its first pass.
+// (wide_sum), except for the usual case of a zero sum with a column of zeros.
 struct Pair {
   float hi = 0.0f, lo = 0.0f;
   __device__ __forceinline__ void add_err(float p, float e) {
@@ -254,18 +265,36 @@ struct Pair {
     add_err(p, __fmaf_rn(a, b, -p));
   }
   __device__ __forceinline__ void add(float a) { add_err(a, 0.0f); }
-  __device__ __forceinline__ bool sound() const { return fabsf(hi) >= 0x1p-96f && isfinite(hi) && isfinite(lo); }
+  __device__ __forceinline__ bool zero() const { return hi == 0.0f && lo == 0.0f; }
+  __device__ __forceinline__ bool finite() const { return isfinite(hi) && isfinite(lo); }  // enough for add
+  __device__ __forceinline__ bool sound() const { return fabsf(hi) >= 0x1p-96f && finite(); }
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
 // sum over the tile's rows of x y (y null: of x) in FP64; row strides sx, sy
-__device__ __noinline__ double wide_sum(const float *x, int sx, const float *y, int sy) {
-  bool any = false;
-  for (int r = 0; r < kTile; ++r) any |= x[r * sx] != 0.0f && (!y || y[r * sy] != 0.0f);
+__device__ __forceinline__ double wide_sum(const float *x, int sx, const float *y, int sy) {
   double s = 0.0;
-  if (any)
-    for (int r = 0; r < kTile; ++r) s = fma((double)x[r * sx], y ? (double)y[r * sy] : 1.0, s);
+#pragma unroll 1
+  for (int r = 0; r < kTile; ++r) s = fma((double)x[r * sx], y ? (double)y[r * sy] : 1.0, s);
   return s;
+}
+__device__ __forceinline__ bool nz_feat(const MlpShared &m, int k) {
+  unsigned b = 0;
+#pragma unroll
+  for (int w = 0; w < kMlpThreads / 32; ++w) b |= m.nz.feat[w];
+  return b >> k & 1u;
+}
+__device__ __forceinline__ bool nz_dz2(const MlpShared &m, int v) {
+  unsigned b = 0;
+#pragma unroll
+  for (int w = 0; w < kMlpThreads / 32; w += 2) b |= m.nz.dz2[w + v / 32];
+  return b >> (v % 32) & 1u;
+}
+__device__ __forceinline__ bool nz_dz1(const MlpShared &m, int u) {
+  unsigned b = 0;
+#pragma unroll
+  for (int w = 0; w < kMlpThreads / 32; ++w) b |= m.nz.dz1[w][u % 4];
+  return b >> (u / 4) & 1u;
 }
 
 // the tile's weight gradients, added to the thread's sums: W2 (4 x 4 a thread), W1
@@ -273,6 +302,7 @@ __device__ __noinline__ double wide_sum(const float *x, int sx, const float *y, 
 constexpr int kMisc = 2 * NH + NO * NH + NO;  // 323
 __device__ __forceinline__ void mlp_w2_sums(const MlpShared &m, double (&g2)[16]) {
   const int v0 = 4 * (threadIdx.x / 16), u0 = 4 * (threadIdx.x % 16);
+  unsigned again = 0;  // sums to be taken in FP64
   Pair a[16];
   for (int r = 0; r < kTile; ++r) {
     const float4 d = *reinterpret_cast<const float4 *>(m.dz2 + r * HS + v0);
@@ -284,12 +314,23 @@ __device__ __forceinline__ void mlp_w2_sums(const MlpShared &m, double (&g2)[16]
       for (int j = 0; j < 4; ++j) a[4 * i + j].mac(dv[i], hv[j]);
   }
 #pragma unroll
-  for (int q = 0; q < 16; ++q)
-    g2[q] += a[q].sound() ? a[q].value() : wide_sum(m.dz2 + v0 + q / 4, HS, m.h1 + u0 + q % 4, HS);
+  for (int q = 0; q < 16; ++q) {
+    if (a[q].sound()) g2[q] += a[q].value();
+    else if (!a[q].zero() || nz_dz2(m, v0 + q / 4)) again |= 1u << q;
+  }
+#pragma unroll 1
+  for (; again; again &= again - 1) {
+    const int k = __ffs(again) - 1;
+    const double t = wide_sum(m.dz2 + v0 + k / 4, HS, m.h1 + u0 + k % 4, HS);
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      if (q == k) g2[q] += t;
+  }
 }
 // dz1 is in m.h2's place by then; W3 and b3 come from m.h2 before (pass 0)
 __device__ __forceinline__ void mlp_w1_sums(const MlpShared &m, double (&g1)[4]) {
   const int u = threadIdx.x / 4, k0 = 4 * (threadIdx.x % 4);
+  unsigned again = 0;
   Pair a[4];
   for (int r = 0; r < kTile; ++r) {
     const float d = m.h2[r * HS + u];
@@ -300,7 +341,18 @@ __device__ __forceinline__ void mlp_w1_sums(const MlpShared &m, double (&g1)[4])
     a[3].mac(d, f.w);
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q) g1[q] += a[q].sound() ? a[q].value() : wide_sum(m.h2 + u, HS, m.feat + k0 + q, FS);
+  for (int q = 0; q < 4; ++q) {
+    if (a[q].sound()) g1[q] += a[q].value();
+    else if (!a[q].zero() || (nz_feat(m, k0 + q) && nz_dz1(m, u))) again |= 1u << q;
+  }
+#pragma unroll 1
+  for (; again; again &= again - 1) {
+    const int k = __ffs(again) - 1;
+    const double t = wide_sum(m.h2 + u, HS, m.feat + k0 + k, FS);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (q == k) g1[q] += t;
+  }
 }
 __device__ __forceinline__ void mlp_misc_sums(const MlpShared &m, int pass, double (&g)[2]) {
 #pragma unroll
@@ -316,7 +368,7 @@ __device__ __forceinline__ void mlp_misc_sums(const MlpShared &m, int pass, doub
       if (y) a.mac(x[r * sx], y[r * HS]);
       else a.add(x[r * sx]);
     }
-    g[q] += a.sound() ? a.value() : wide_sum(x, sx, y, HS);
+    g[q] += (y ? a.sound() : a.finite()) ? a.value() : wide_sum(x, sx, y, HS);
   }
 }
 __device__ __forceinline__ int misc_param(int o) {
@@ -326,7 +378,7 @@ __device__ __forceinline__ int misc_param(int o) {
 // partial[block][parameter] = sum over the block's tiles of d<dout, MLP_w(feat)>/dw:
 // dz2 = (W3^T dout) (1 - h2^2), dz1 = (W2^T dz2) (1 - h1^2), and the sums over rows
 // of dz1 x feat, dz2 x h1, dout x h2 and of dz1, dz2, dout
-__global__ void __launch_bounds__(kMlpThreads) k_mlp_grad(int32_t n, const float *__restrict__ wg,
+__global__ void __launch_bounds__(kMlpThreads, 2) k_mlp_grad(int32_t n, const float *__restrict__ wg,
                                                           const float *__restrict__ feat,
                                                           const float *__restrict__ dout,
                                                           double *__restrict__ partial) {
@@ -340,12 +392,18 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_grad(int32_t n, const float
       m.dout[threadIdx.x] = q < NO && base + r < n ? dout[(size_t)(base + r) * NO + q] : 0.0f;
     }
     mlp_hidden(m, n, base, feat);
-    for (int q = threadIdx.x; q < kTile * NH; q += kMlpThreads) {
+    const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
+    bool nz = false;
+    for (int q = threadIdx.x; q < kTile * NH; q += kMlpThreads) {  // a thread stays in its column
       const int r = q / NH, v = q % NH;
       const float h2 = m.h2[r * HS + v];
       const float dh = m.w3[v] * m.dout[4 * r] + m.w3[NH + v] * m.dout[4 * r + 1] + m.w3[2 * NH + v] * m.dout[4 * r + 2];
-      m.dz2[r * HS + v] = dh * (1.0f - h2 * h2);
+      const float d = dh * (1.0f - h2 * h2);
+      nz |= d != 0.0f;
+      m.dz2[r * HS + v] = d;
     }
+    const unsigned b2 = __ballot_sync(0xffffffffu, nz);
+    if (lane == 0) m.nz.dz2[wid] = b2;
     __syncthreads();
     float dz1[4][4];
     const int u0 = 4 * (threadIdx.x % 16), r0 = 4 * (threadIdx.x / 16);
@@ -372,6 +430,12 @@ __global__ void __launch_bounds__(kMlpThreads) k_mlp_grad(int32_t n, const float
         const float h1 = m.h1[(r0 + i) * HS + u0 + j];
         dz1[i][j] *= 1.0f - h1 * h1;
       }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const unsigned b1 = __ballot_sync(0xffffffffu, dz1[0][j] != 0.0f || dz1[1][j] != 0.0f || dz1[2][j] != 0.0f ||
+                                                         dz1[3][j] != 0.0f);
+      if (lane == 0) m.nz.dz1[wid][j] = (b1 | b1 >> 16) & 0xffffu;
+    }
     mlp_w2_sums(m, g2);
     mlp_misc_sums(m, 0, gm);
     __syncthreads();
