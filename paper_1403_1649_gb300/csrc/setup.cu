@@ -1033,17 +1033,19 @@ __device__ __forceinline__ int32_t ap_count_regs(const Row &r, int32_t width, in
 //
 // Slices of at most kApNarrow entries a row take a lane per row with the row's
 // aggregates in registers.  Wider ones are shared by the block: its warps stage the
-// slice's aggregates (and values and weights) in shared memory, coalesced, then take a
-// row each, a lane per entry, every lane comparing its aggregate with the row's entries
+// aggregates (and values and weights) of half a slice in shared memory, coalesced, then
+// take a row each, a lane per entry, every lane comparing its aggregate with the row's entries
 // one after the other; the sums keep the entries' order.  By a lane per row those
 // comparisons are a chain of loads, the square of the width long: the two passes took
-// 42 + 61 us on the level of 1,538 rows of 128^3, 7 + 17 us now, and 121 + 249 us on all
-// its levels, 64 + 177 us now.  Beyond kApMergeWidth entries (a hub's row) an
-// entry of A stays an entry of A P of its own, which costs the cycle what the row costs
-// in A: coarse levels of 3D problems have a few slices in a thousand of that width.
-constexpr int32_t kApNarrow = 24, kApMergeWidth = 64;
+// 42 + 61 us on the level of 1,538 rows of 128^3, 8 + 17 us now, and 120 + 249 us on all
+// its levels, 67 + 176 us now.  Beyond kApMergeWidth entries, the widest rows of the
+// coarse levels of the jump-coefficient problems, an entry of A (a hub's row) stays an
+// entry of A P of its own, which costs the cycle what the row costs in A (merging up to
+// 64 only: 97^3 BF16 step 3 % longer).
+constexpr int32_t kApNarrow = 24, kApMergeWidth = 128;
 constexpr int kApWarps = 8;
-constexpr int kApStride = kSlice + 1;  // a row's entries in shared memory without bank conflicts
+constexpr int kApRows = kSlice / 2;     // rows staged at a time
+constexpr int kApStride = kApRows + 1;  // a row's entries in shared memory without bank conflicts
 
 template <class MV, class VT>
 struct ApArgs {
@@ -1142,81 +1144,93 @@ __global__ void __launch_bounds__(kApWarps * 32) k_ap(ApArgs<MV, VT> a) {
     const int32_t width = slice_width(sl);
     if (width <= kApNarrow) continue;
     const bool merge = width <= kApMergeWidth;
-    __syncthreads();  // the previous slice's entries have been read
     if (!FILL && threadIdx.x == 0) widest = 0;
-    if (merge) {
-      const SellRow<MV> r{a.scol, a.sval, a.spair, a.sptr[sl], lane};
-      for (int32_t e = wid; e < width; e += kApWarps) {
-        const int32_t c = r.col(e);
-        sJ[e * kApStride + lane] = a.agg[c];
-        if constexpr (FILL) {
-          sV[e * kApStride + lane] = (VT)r.val(e);
-          sP[e * kApStride + lane] = a.pw[c];
+    for (int j0 = 0; j0 < kSlice; j0 += kApRows) {
+      __syncthreads();  // the previous rows' entries have been read
+      if (merge) {
+        const int i = lane % kApRows;
+        const SellRow<MV> r{a.scol, a.sval, a.spair, a.sptr[sl], j0 + i};
+        for (int32_t e = 2 * wid + lane / kApRows; e < width; e += 2 * kApWarps) {
+          const int32_t c = r.col(e);
+          sJ[e * kApStride + i] = a.agg[c];
+          if constexpr (FILL) {
+            sV[e * kApStride + i] = (VT)r.val(e);
+            sP[e * kApStride + i] = a.pw[c];
+          }
         }
       }
-    }
-    __syncthreads();
-    for (int j = wid; j < kSlice; j += kApWarps) {  // a warp per row
-      const int32_t row = sl * kSlice + j;
-      const int32_t own = a.agg[row < a.n ? row : a.n - 1];
-      int32_t cnt = 0;
-      VT o = VT(0);
-      if constexpr (FILL)
-        if (row < a.n && a.sdiag) o = (VT)a.sdiag[row] * a.pw[row];
-      if (row < a.n && merge) {
-        constexpr int kPer = kApMergeWidth / 32;  // entries of a lane
-        int32_t J[kPer];
-        bool first[kPer];  // the first entry of its aggregate carries the aggregate's sum
-        VT s[kPer];
+      __syncthreads();
+      for (int i = wid; i < kApRows; i += kApWarps) {  // a warp per row
+        const int j = j0 + i;
+        const int32_t row = sl * kSlice + j;
+        const int32_t own = a.agg[row < a.n ? row : a.n - 1];
+        int32_t cnt = 0;
+        VT o = VT(0);
+        if constexpr (FILL)
+          if (row < a.n && a.sdiag) o = (VT)a.sdiag[row] * a.pw[row];
+        auto merged = [&](auto size) {  // rows of at most 32 kPer entries
+          constexpr int kPer = decltype(size)::value;
+          int32_t J[kPer];
+          bool first[kPer];  // the first entry of its aggregate carries the aggregate's sum
+          VT s[kPer];
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-          const int32_t e = 32 * u + lane;
-          J[u] = e < width ? sJ[e * kApStride + j] : own;
-          first[u] = J[u] != own;
-          s[u] = VT(0);
-        }
-        for (int32_t q = 0; q < width; ++q) {
-          const int32_t Jq = sJ[q * kApStride + j];
-          VT v = VT(0), p = VT(0);
-          if constexpr (FILL) {
-            v = sV[q * kApStride + j];
-            p = sP[q * kApStride + j];
-            if (Jq == own) o += v * p;
+          for (int u = 0; u < kPer; ++u) {
+            const int32_t e = 32 * u + lane;
+            J[u] = e < width ? sJ[e * kApStride + i] : own;
+            first[u] = J[u] != own;
+            s[u] = VT(0);
           }
-#pragma unroll
-          for (int u = 0; u < kPer; ++u)
-            if (Jq == J[u]) {
-              if (q < 32 * u + lane) first[u] = false;
-              else if constexpr (FILL) s[u] += v * p;
+          for (int32_t q = 0; q < width; ++q) {
+            const int32_t Jq = sJ[q * kApStride + i];
+            VT v = VT(0), p = VT(0);
+            if constexpr (FILL) {
+              v = sV[q * kApStride + i];
+              p = sP[q * kApStride + i];
+              if (Jq == own) o += v * p;
             }
-        }
 #pragma unroll
-        for (int u = 0; u < kPer; ++u) {
-          const unsigned b = __ballot_sync(0xffffffffu, first[u]);
-          if constexpr (FILL)
-            if (first[u]) put(sl, j, cnt + __popc(b & below), J[u], s[u]);
-          cnt += __popc(b);
-        }
-      } else if (row < a.n) {
-        const SellRow<MV> r{a.scol, a.sval, a.spair, a.sptr[sl], j};
-        for (int32_t e0 = 0; e0 < width; e0 += 32) {
-          const bool in = e0 + lane < width;
-          const int32_t c = in ? r.col(e0 + lane) : row, J = a.agg[c];
-          const unsigned b = __ballot_sync(0xffffffffu, in && J != own);
-          if constexpr (FILL) {
-            const VT v = in ? (VT)r.val(e0 + lane) : VT(0), p = a.pw[c];
-            if (in && J != own) put(sl, j, cnt + __popc(b & below), J, v * p);
-            for (unsigned m = __ballot_sync(0xffffffffu, in && J == own); m; m &= m - 1)
-              o += __shfl_sync(0xffffffffu, v, __ffs(m) - 1) * __shfl_sync(0xffffffffu, p, __ffs(m) - 1);
+            for (int u = 0; u < kPer; ++u)
+              if (Jq == J[u]) {
+                if (q < 32 * u + lane) first[u] = false;
+                else if constexpr (FILL) s[u] += v * p;
+              }
           }
-          cnt += __popc(b);
+#pragma unroll
+          for (int u = 0; u < kPer; ++u) {
+            const unsigned b = __ballot_sync(0xffffffffu, first[u]);
+            if constexpr (FILL)
+              if (first[u]) put(sl, j, cnt + __popc(b & below), J[u], s[u]);
+            cnt += __popc(b);
+          }
+        };
+        if (row >= a.n) {  // padding only
+        } else if (width <= 32) {
+          merged(std::integral_constant<int, 1>{});
+        } else if (width <= 64) {
+          merged(std::integral_constant<int, 2>{});
+        } else if (merge) {
+          merged(std::integral_constant<int, kApMergeWidth / 32>{});
+        } else {
+          const SellRow<MV> r{a.scol, a.sval, a.spair, a.sptr[sl], j};
+          for (int32_t e0 = 0; e0 < width; e0 += 32) {
+            const bool in = e0 + lane < width;
+            const int32_t c = in ? r.col(e0 + lane) : row, J = a.agg[c];
+            const unsigned b = __ballot_sync(0xffffffffu, in && J != own);
+            if constexpr (FILL) {
+              const VT v = in ? (VT)r.val(e0 + lane) : VT(0), p = a.pw[c];
+              if (in && J != own) put(sl, j, cnt + __popc(b & below), J, v * p);
+              for (unsigned m = __ballot_sync(0xffffffffu, in && J == own); m; m &= m - 1)
+                o += __shfl_sync(0xffffffffu, v, __ffs(m) - 1) * __shfl_sync(0xffffffffu, p, __ffs(m) - 1);
+            }
+            cnt += __popc(b);
+          }
         }
-      }
-      if constexpr (FILL) {
-        if (row < a.n && lane == 0) a.own[row] = o;
-        for (int32_t at = cnt + lane, apw = ap_width(sl); at < apw; at += 32) put(sl, j, at, own, VT(0));
-      } else if (lane == 0) {
-        atomicMax(&widest, cnt);
+        if constexpr (FILL) {
+          if (row < a.n && lane == 0) a.own[row] = o;
+          for (int32_t at = cnt + lane, apw = ap_width(sl); at < apw; at += 32) put(sl, j, at, own, VT(0));
+        } else if (lane == 0) {
+          atomicMax(&widest, cnt);
+        }
       }
     }
     if constexpr (!FILL) {
