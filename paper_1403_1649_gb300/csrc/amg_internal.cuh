@@ -336,10 +336,11 @@ constexpr int kTailMaxRows = 4096;
 
 // ---------------------------------------------------------------- launches
 // Solve kernels are launched with programmatic dependent launch: each kernel
-// may be scheduled while its predecessor in the stream still runs, waits in
+// may be scheduled while its predecessor in the stream still runs and waits in
 // griddepcontrol.wait until the predecessor has completed and its writes are
-// visible, and at once lets its own successor launch.  This hides the launch
-// latency of the many short kernels of a multigrid cycle.
+// visible.  The kernels of the cycle let their successor launch before that wait
+// (pdl_trigger, pdl_wait), the others after it (pdl_wait_and_trigger).  This
+// hides the launch latency of the many short kernels of a multigrid cycle.
 bool &pdl_enabled();  // thread-local, set from the hierarchy's parameters
 
 template <typename... KArgs, typename... Args>

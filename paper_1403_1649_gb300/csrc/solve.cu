@@ -80,7 +80,7 @@ template <class MV> constexpr bool kHalfPairs = std::is_same<MV, __nv_bfloat16>:
 // fence, atomic, partials and scalars, which added ~3.5 us to each of 12 kernels of an
 // iteration (1.5-2 us now, in the kernel that reads them: 128^3 step 16.9 -> 16.5 ms,
 // FEM 1024^2 solve 28.3 -> 26.1, learned 501^2 8.0 -> 7.0, 700^2 re-setup + solve 35.4 ->
-// 32.3, 64^2 step 3.25 -> 3.07).  What the host or a predicate of later launches needs (the end of an
+// 32.3).  What the host or a predicate of later launches needs (the end of an
 // outer iteration) is still formed by the last block (grid_totals).
 // GB300 issues an FP64 warp instruction every 16 cycles an SM, so the reductions
 // count them: the block's values go through shared memory and one warp per product
@@ -111,7 +111,7 @@ constexpr int kSumWarps = kSumThreads / 32;
 inline int sum_grid(int64_t n) { return grid_for(n, kSumThreads, 304); }
 
 // tot[k] = sum of the nb partials of product k, the same bits in every block; valid in
-// warp 0 (all lanes).  Every thread of the block calls it.  An FP64 addition takes ~60
+// thread 0 (up to lane 7 of warp 0, all lanes for few partials).  Every thread of the block calls it.  An FP64 addition takes ~60
 // cycles to its result: up to 128 partials warp 0 sums alone (four loads a lane, all
 // products side by side), more are shared among the block's warps.
 template <int ND>
@@ -731,8 +731,12 @@ struct PostArgs {
   const int *pred;
 };
 
+// Resident blocks per SM, and the grid's wave: the row's operands, its first step's
+// entries and their gathers all in flight at 80 (FP32) and 128 registers.  One block
+// more an SM holds fewer (a solve of FEM 1024^2 in FP32 20.3 -> 20.7 ms, 90^3 in FP64
+// 5.69 -> 6.30), 6 and 4 blocks 22.2 and 6.74 ms.
 template <class VT>
-constexpr int post_blocks() { return sizeof(VT) == 4 ? 3 : 2; }  // resident blocks per SM
+constexpr int post_blocks() { return sizeof(VT) == 4 ? 3 : 2; }
 
 template <class VT, int ND, bool GATE>
 __global__ void __launch_bounds__(kThreads, post_blocks<VT>()) k_post(PostArgs<VT> a) {
@@ -798,6 +802,10 @@ __global__ void __launch_bounds__(kThreads, post_blocks<VT>()) k_post(PostArgs<V
       xi = a.x[rr];
       if constexpr (ND == 1) qi = a.q64[rr];
     };
+    // widths 4 and 6, the neighbouring aggregates of a row of 5- and 7-point and P1
+    // meshes (FP32: rounded up to even), take one step without predicates; all widths
+    // by the predicated step: FEM 1024^2 20.27 -> 20.37 ms, 90^3 FP64 5.69 -> 5.73,
+    // 97^3 BF16 58.7 -> 59.0, 700^2 19.56 -> 19.59
     using S4 = std::integral_constant<int, 4>;
     using S6 = std::integral_constant<int, 6>;
     using SU = std::integral_constant<int, U>;
